@@ -106,12 +106,14 @@ void release(vie_handle* h) {
         cudaFree(h->green64);
         cudaFree(h->green32);
         cudaFree(h->green32t);
-        cudaFree(h->green64t);
+        cudaFree(h->green_d);
+        cudaFree(h->green_e);
         cudaFree(h->greenbf);
         cudaFree(h->colmap);
         cudaFree(h->colkx32);
         cudaFree(h->tw64);
         cudaFree(h->tw32);
+        cudaFree(h->twfx);
         cudaFree(h->toeplitz);
     }
     cudaFree(h->tucker);
@@ -227,8 +229,8 @@ int vie_setup_green_external(const vie_grid* grid, double freq_hz, const double*
 
 size_t handle_green_bytes(const vie_handle* h) {
     const size_t ov = (size_t)h->O[0] * h->O[1] * h->O[2];
-    return 60 * ov * (2 * sizeof(double2) + 2 * sizeof(float2) + sizeof(uint2)) + 60 * h->nv * sizeof(double2) +
-           2048 * (sizeof(double2) + sizeof(float2)) + 2 * (size_t)h->L[0];
+    return 60 * ov * (sizeof(double2) + 2 * sizeof(float2) + sizeof(uint2)) + green_digit_bytes(h, 60) +
+           60 * h->nv * sizeof(double2) + 2048 * (sizeof(double2) + sizeof(float2) + sizeof(int4)) + 2 * (size_t)h->L[0];
 }
 
 int handle_create(const vie_grid* grid, double freq_hz, const double* eps_real, const double* sigma,
@@ -322,13 +324,15 @@ int handle_create(const vie_grid* grid, double freq_hz, const double* eps_real, 
         h->green64 = share->green64;
         h->green32 = share->green32;
         h->green32t = share->green32t;
-        h->green64t = share->green64t;
+        h->green_d = share->green_d;
+        h->green_e = share->green_e;
         h->greenbf = share->greenbf;
         h->colmap = share->colmap;
         h->colkx32 = share->colkx32;
         h->colpos32 = share->colpos32;
         h->tw64 = share->tw64;
         h->tw32 = share->tw32;
+        h->twfx = share->twfx;
         h->toeplitz = share->toeplitz;
         *out = h;
         return VIE_OK;

@@ -117,15 +117,20 @@ struct vie_handle {
     float2* green32;
     // FP32 copy in the layout of the z pass of the FP32 three-kernel path: [Oy][Ox][Oz][60]
     float2* green32t;
-    // FP64 copy in the same layout, for the FP64 fused z pass
-    double2* green64t;
+    // the FP64 values' digits for the FP64 fused z pass (zpass_f64.cu): per octant point and tensor seven
+    // 9-bit digits as fp16 (re, im) pairs, [Oy][Ox][Oz][60][2], and the exponent of each column [Oy][Ox]
+    // (PWL handles with an FFT length along z of 8..512, else null)
+    uint4* green_d;
+    int* green_e;
     // the 30 K tensors' transformed circulants, octant storage [30][Oz][Oy][Ox], scaled by
     // 1/(Lx Ly Lz), FP64 and FP32 (kmatvec.cu, built on the first K product)
     double2* kgreen64;
     float2* kgreen32;
-    // copies [Oy][Ox][Oz][30] for the fused z passes with the K block (zpass_f32.cu, zpass_f64.cu)
+    // copy [Oy][Ox][Oz][30] for the FP32 fused z pass with the K block (zpass_f32.cu)
     float2* kgreen32t;
-    double2* kgreen64t;
+    // and their digits for the FP64 one, as green_d
+    uint4* kgreen_d;
+    int* kgreen_e;
     // bf16 split of green32t in the same layout, for the BF16x3 z pass: per tensor (hi, lo),
     // each a bf16 (re, im) pair with hi = bf16(v), lo = bf16(v - hi)
     uint2* greenbf;
@@ -140,6 +145,7 @@ struct vie_handle {
     // twiddle tables exp(-2 pi i m / L) for L = 2^k, k = 1..11, concatenated at offset L
     double2* tw64;
     float2* tw32;
+    int4* twfx;  // the same as fixed-point factors (fixed.cuh): (hi, lo) of the cosine, then of the sine
     // scratch
     Workspace fft_ws;    // matvec spectrum buffers
     Workspace stage_ws;  // host-buffer staging
@@ -275,6 +281,8 @@ void stats_capture_release(std::vector<CapRec>& list);
 // ---------------------------------------------------------------------------
 int green_setup(vie_handle* h);                 // green.cu
 int green_setup_external(vie_handle* h, const double2* ext);  // green.cu, ext on the device
+// bytes of the digit tables of ng tensors (zero where the FP64 fused z pass does not apply)
+size_t green_digit_bytes(const vie_handle* h, int ng);  // matvec.cu
 int green_split_bf16(vie_handle* h);            // zpass_bf16.cu: greenbf from green32t
 int twiddle_setup(vie_handle* h);               // matvec.cu
 int matvec_device(vie_handle* h, int nrhs, const void* x, void* y, int precision, int op, cudaStream_t s);

@@ -16,6 +16,7 @@
 
 #include "common.cuh"
 #include "kblock.h"
+#include "zpass_f64.cuh"
 
 int green_k_toeplitz(vie_handle* h, double2* out, cudaStream_t s);  // green.cu
 
@@ -75,7 +76,12 @@ __global__ void k_octant_kernel(const double2* __restrict__ C, int Lx, int Ly, i
     g32[dst] = make_float2((float)v.x, (float)v.y);
     const long long dt = (((long long)ky * Ox + kx) * Oz + kz) * 30 + t0 + tl;
     g32t[dt] = make_float2((float)v.x, (float)v.y);
-    g64t[dt] = v;
+    if (g64t) g64t[dt] = v;
+}
+
+// device bytes of a handle's K spectra
+size_t k_bytes(const vie_handle* h) {
+    return (sizeof(double2) + 2 * sizeof(float2)) * 30 * (size_t)h->O[0] * h->O[1] * h->O[2] + green_digit_bytes(h, 30);
 }
 
 unsigned blocks(long long n) { return (unsigned)((n + 255) / 256); }
@@ -91,6 +97,9 @@ int k_octants(vie_handle* h, cudaStream_t s) {
     const long long ovol = (long long)h->O[0] * h->O[1] * h->O[2];
     const int chunk = (int)std::max<long long>(1, std::min<long long>(30, (4LL << 30) / (vol * (long long)sizeof(double2))));
     double2 *P = nullptr, *C = nullptr, *g64 = nullptr, *g64t = nullptr;
+    uint4* gd = nullptr;
+    int* ge = nullptr;
+    const bool digits = green_digit_bytes(h, 30) > 0;
     float2 *g32 = nullptr, *g32t = nullptr;
     auto fail = [&](int code, const char* msg) {
         cudaGetLastError();
@@ -100,6 +109,8 @@ int k_octants(vie_handle* h, cudaStream_t s) {
         cudaFree(g32);
         cudaFree(g32t);
         cudaFree(g64t);
+        cudaFree(gd);
+        cudaFree(ge);
         set_error(msg);
         return code;
     };
@@ -108,7 +119,9 @@ int k_octants(vie_handle* h, cudaStream_t s) {
         cudaMalloc(&g64, sizeof(double2) * 30 * ovol) != cudaSuccess ||
         cudaMalloc(&g32, sizeof(float2) * 30 * ovol) != cudaSuccess ||
         cudaMalloc(&g32t, sizeof(float2) * 30 * ovol) != cudaSuccess ||
-        cudaMalloc(&g64t, sizeof(double2) * 30 * ovol) != cudaSuccess)
+        (digits && (cudaMalloc(&g64t, sizeof(double2) * 30 * ovol) != cudaSuccess ||
+                    cudaMalloc(&gd, 2 * sizeof(uint4) * 30 * ovol) != cudaSuccess ||
+                    cudaMalloc(&ge, sizeof(int) * h->O[0] * h->O[1]) != cudaSuccess)))
         return fail(VIE_ENOMEM, "K spectrum allocation failed");
     int rc = green_k_toeplitz(h, P, s);
     for (int t0 = 0; rc == VIE_OK && t0 < 30; t0 += chunk) {
@@ -123,6 +136,7 @@ int k_octants(vie_handle* h, cudaStream_t s) {
                                                                       g32, g32t, g64t));
         if (cudaGetLastError() != cudaSuccess) return fail(VIE_EDEVICE, "K octant launch failed");
     }
+    if (rc == VIE_OK && digits) rc = green_digits(h, g64t, 30, gd, ge, s);
     if (rc == VIE_OK && cudaStreamSynchronize(s) != cudaSuccess) return fail(VIE_EDEVICE, "K spectrum sync failed");
     if (rc < 0) {
         cudaFree(P);
@@ -131,15 +145,19 @@ int k_octants(vie_handle* h, cudaStream_t s) {
         cudaFree(g32);
         cudaFree(g32t);
         cudaFree(g64t);
+        cudaFree(gd);
+        cudaFree(ge);
         return rc;
     }
     cudaFree(P);
     cudaFree(C);
+    cudaFree(g64t);
     h->kgreen64 = g64;
     h->kgreen32 = g32;
     h->kgreen32t = g32t;
-    h->kgreen64t = g64t;
-    h->bytes_held += 2 * (sizeof(double2) + sizeof(float2)) * 30 * (size_t)ovol;  // until kmatvec_release
+    h->kgreen_d = gd;
+    h->kgreen_e = ge;
+    h->bytes_held += k_bytes(h);  // until kmatvec_release
     return VIE_OK;
 }
 
@@ -154,10 +172,12 @@ void kmatvec_release(vie_handle* h) {
     cudaFree(h->kgreen64);
     cudaFree(h->kgreen32);
     cudaFree(h->kgreen32t);
-    cudaFree(h->kgreen64t);
+    cudaFree(h->kgreen_d);
+    cudaFree(h->kgreen_e);
     h->kgreen64 = nullptr;
     h->kgreen32 = nullptr;
     h->kgreen32t = nullptr;
-    h->kgreen64t = nullptr;
-    h->bytes_held -= 2 * (sizeof(double2) + sizeof(float2)) * 30 * (size_t)h->O[0] * h->O[1] * h->O[2];
+    h->kgreen_d = nullptr;
+    h->kgreen_e = nullptr;
+    h->bytes_held -= k_bytes(h);
 }

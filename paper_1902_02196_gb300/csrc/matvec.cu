@@ -13,6 +13,7 @@
 //            (op A: G x - chi (N - G) x;  op PA: x/eps - tau G^-1 (N - G) x)  W1 -> y
 // The 1/(Lx Ly Lz) normalisation is folded into the stored Green tensor.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <mutex>
 #include <vector>
@@ -21,7 +22,9 @@
 #include "block.cuh"
 #include "fft.cuh"
 #include "fft2.cuh"
+#include "fixed.cuh"
 #include "line2.cuh"
+#include "xy_f64.cuh"
 #include "zpass_f32.cuh"
 #include "zpass_f64.cuh"
 
@@ -187,25 +190,26 @@ __global__ void __launch_bounds__(ZCfg<T, L, NC>::NT) zpass_kernel(ZArgs z, cons
 // ---------------------------------------------------------------------------
 constexpr int kXYThreads = 256;
 
-template <int L, typename C>
+template <int L>
 struct XYCfg {
+    using C = float2;
     static constexpr int H = L / 2;   // rows that are non-zero before / needed after the y transform
     static constexpr int RS = L + 1;  // odd row stride of the x-transform buffer
-    static constexpr int CW0 = sizeof(C) == 8 ? 32 : 16;
-    static constexpr int CW = L < CW0 ? L : CW0;  // stored columns per y-transform chunk
+    static constexpr int CW = L < 32 ? L : 32;  // stored columns per y-transform chunk
     static constexpr int EPV = 16 / (int)sizeof(C);  // elements per 16-byte vector
-    static constexpr int MINB = sizeof(C) == 8 ? 2 : 1;  // CTAs per SM
+    static constexpr int MINB = 2;  // CTAs per SM
     static constexpr size_t smem = sizeof(C) * (size_t)(L * CW + H * RS + L) + sizeof(int4) * H + L;
 };
 
 // Forward: plane (r, alpha, z) of x -> W2 plane [Ly][Lx] (transposed ky, stored kx).  x is
 // [R][12][Nz][Ny][Nx], or [R][12][ns] on a support (rows != NULL; zeros outside it).
-template <int L, typename C>
-__global__ void __launch_bounds__(kXYThreads, XYCfg<L, C>::MINB)
-    xy_fwd_kernel(const C* __restrict__ x, C* __restrict__ w, int nx, int ny, int nz, const int4* __restrict__ rows,
-                  long long ns, const unsigned char* __restrict__ cpos, const C* __restrict__ twg,
+template <int L>
+__global__ void __launch_bounds__(kXYThreads, XYCfg<L>::MINB)
+    xy_fwd_kernel(const float2* __restrict__ x, float2* __restrict__ w, int nx, int ny, int nz, const int4* __restrict__ rows,
+                  long long ns, const unsigned char* __restrict__ cpos, const float2* __restrict__ twg,
                   const int* __restrict__ rmap, MatvecEpi dc) {
-    using Cfg = XYCfg<L, C>;
+    using Cfg = XYCfg<L>;
+    using C = float2;
     constexpr int A = fft2::Split<L>::A, B = fft2::Split<L>::B, NT = kXYThreads, RS = Cfg::RS, CW = Cfg::CW;
     constexpr int EPV = Cfg::EPV;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -286,14 +290,14 @@ __global__ void __launch_bounds__(kXYThreads, XYCfg<L, C>::MINB)
     }
 }
 
-// Inverse: W2 plane -> y plane [Ny][Nx] with the material / Gram / preconditioner epilogue;
-// CONV: also the plane's (N - G) x at every voxel to epi.conv (full grid).
-template <int L, typename C, bool CONV>
-__global__ void __launch_bounds__(kXYThreads, XYCfg<L, C>::MINB)
-    xy_inv_kernel(const C* __restrict__ w, C* __restrict__ y, MatvecEpi epi, const unsigned char* __restrict__ cpos,
-                  const C* __restrict__ twg) {
-    using Cfg = XYCfg<L, C>;
-    using R = decltype(C{}.x);
+// Inverse: W2 plane -> y plane [Ny][Nx] with the material / Gram / preconditioner epilogue.
+template <int L>
+__global__ void __launch_bounds__(kXYThreads, XYCfg<L>::MINB)
+    xy_inv_kernel(const float2* __restrict__ w, float2* __restrict__ y, MatvecEpi epi,
+                  const unsigned char* __restrict__ cpos, const float2* __restrict__ twg) {
+    using Cfg = XYCfg<L>;
+    using C = float2;
+    using R = float;
     constexpr int A = fft2::Split<L>::A, B = fft2::Split<L>::B, NT = kXYThreads, RS = Cfg::RS, CW = Cfg::CW;
     constexpr int EPV = Cfg::EPV;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -394,13 +398,11 @@ __global__ void __launch_bounds__(kXYThreads, XYCfg<L, C>::MINB)
         const double2 d = epi.shift[po / rplanes];
         sh = mk((R)d.x, (R)d.y);
     }
-    C* conv = CONV ? reinterpret_cast<C*>(epi.conv) : nullptr;
 #pragma unroll 4
     for (int idx = tid; idx < ny * nx; idx += NT) {
         const int yy = idx / nx, xx = idx % nx;
         long long o = base + idx;
         C v = xr[yy * RS + xx];
-        if (CONV) conv[base + idx] = v;  // every voxel of the plane, full-grid layout
         if (epi.rows) {
             const int4 q = rw[yy];
             if (xx < q.x || xx >= q.y) continue;
@@ -518,19 +520,38 @@ static int launch_z(const char* name, const vie_handle* h, int L, const ZArgs& z
 static bool xy_ok(const vie_handle* h) { return h->colmap != nullptr; }
 static bool zfused_ok(const vie_handle* h) { return h->L[2] >= 8 && h->L[2] <= 512 && h->L[0] >= 4; }
 
-// in_elems: complex values of the matvec input (and output) vector
-template <int L, typename C>
-static int launch_xy_L(bool fwd, const vie_handle* h, const void* in, void* out, long long planes, int nx, int ny,
-                       const MatvecEpi& e, const Support& sp, double in_elems, cudaStream_t s) {
-    constexpr size_t smem = XYCfg<L, C>::smem;
-    constexpr bool f32 = sizeof(C) == 8;
+size_t green_digit_bytes(const vie_handle* h, int ng) {
+    if (h->nc != 12 || !zfused_ok(h)) return 0;
+    return 2 * sizeof(uint4) * ng * (size_t)h->O[0] * h->O[1] * h->O[2] + sizeof(int) * (size_t)h->O[0] * h->O[1];
+}
+
+// FP32 kernels (the FP64 ones are in xy_f64.cu)
+template <int L>
+static int launch_xy_L(bool fwd, const char* name, double bytes, const vie_handle* h, const float2* in, float2* out,
+                       unsigned planes, int nx, int ny, const MatvecEpi& e, const Support& sp, cudaStream_t s) {
+    constexpr size_t smem = XYCfg<L>::smem;
+    const unsigned char* cpos = h->colmap + L;
+    const float2* tw = h->tw32 + L;
     // set on every call: the attribute is per device and launches may come from several threads
-    VIE_CUDA(cudaFuncSetAttribute(xy_fwd_kernel<L, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    VIE_CUDA(cudaFuncSetAttribute(xy_inv_kernel<L, C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if constexpr (sizeof(C) == 16)
-        VIE_CUDA(cudaFuncSetAttribute(xy_inv_kernel<L, C, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
-    if (e.conv && sizeof(C) != 16) {
+    if (fwd) {
+        VIE_CUDA(cudaFuncSetAttribute(xy_fwd_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        VIE_KLAUNCH_B(name, s, bytes,
+                      xy_fwd_kernel<L><<<planes, kXYThreads, smem, s>>>(in, out, nx, ny, h->nz, sp.rows, sp.ns, cpos, tw,
+                                                                       e.rmap, e));
+    } else {
+        VIE_CUDA(cudaFuncSetAttribute(xy_inv_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        VIE_KLAUNCH_B(name, s, bytes, xy_inv_kernel<L><<<planes, kXYThreads, smem, s>>>(in, out, e, cpos, tw));
+    }
+    VIE_CHECK_LAUNCH();
+    return VIE_OK;
+}
+
+// in_elems: complex values of the matvec input (and output) vector
+template <typename C>
+static int launch_xy(bool fwd, const vie_handle* h, const void* in, void* out, long long planes, int nx, int ny,
+                     const MatvecEpi& e, const Support& sp, double in_elems, cudaStream_t s) {
+    constexpr bool f32 = sizeof(C) == 8;
+    if (e.conv && f32) {
         set_error("internal: the convolution side output is FP64 only");
         return VIE_EINVAL;
     }
@@ -538,67 +559,39 @@ static int launch_xy_L(bool fwd, const vie_handle* h, const void* in, void* out,
         set_error("xy transform grid too large");
         return VIE_EINVAL;
     }
-    const unsigned char* cpos = h->colmap + L;
-    const C* tw = reinterpret_cast<const C*>(f32 ? (const void*)(h->tw32 + L) : (const void*)(h->tw64 + L));
-    const double c = sizeof(C), plane_full = (double)L * L;
+    const double c = sizeof(C), spectrum = (double)planes * h->L[0] * h->L[1];
     // with a device count of right-hand sides (e.nact) the kernel adds its bytes on the device:
     // the part proportional to the planes transformed, per right-hand side of the grid, plus a fixed part
     const double rg = (double)planes / ((double)h->nc * h->nz);  // right-hand sides of the launch grid
+    const char* name = fwd ? (f32 ? "fft_xy_f32" : "fft_xy_f64") : (f32 ? "ifft_xy_epilogue_f32" : "ifft_xy_epilogue_f64");
+    const double fixed = fwd ? 0.0 : c * (double)h->nv * (e.op == VIE_OP_PA ? 2 : e.op == VIE_OP_A ? 1 : 0);
+    const double per = fwd ? c * (in_elems + spectrum)
+                           : c * (spectrum + in_elems * (e.op == VIE_OP_NSCAT ? 1 : 2) +
+                                  (e.conv ? (double)planes * nx * ny : 0.0));
     MatvecEpi ee = e;
-    if (fwd) {
-        const char* name = f32 ? "fft_xy_f32" : "fft_xy_f64";
-        double bytes = c * (in_elems + planes * plane_full);
-        if (e.nact) {
-            ee.bctr = dev_bytes_ptr(name);
-            ee.bfix = 0.0;
-            ee.bper = bytes / rg;
-            bytes = kDevCounted;
-        }
-        VIE_KLAUNCH_B(name, s, bytes,
-                      xy_fwd_kernel<L, C><<<(unsigned)planes, kXYThreads, smem, s>>>(
-                          (const C*)in, (C*)out, nx, ny, h->nz, sp.rows, sp.ns, cpos, tw, e.rmap, ee));
+    double bytes = fixed + per;
+    if (e.nact) {
+        ee.bctr = dev_bytes_ptr(name);
+        ee.bfix = fixed;
+        ee.bper = per / rg;
+        bytes = kDevCounted;
+    }
+    if constexpr (!f32) {
+        return xy_f64(fwd, name, bytes, h, (const C*)in, (C*)out, (unsigned)planes, nx, ny, ee, sp, s);
     } else {
-        const double fixed = c * (double)h->nv * (e.op == VIE_OP_PA ? 2 : e.op == VIE_OP_A ? 1 : 0);
-        const double per = c * (planes * plane_full + in_elems * (e.op == VIE_OP_NSCAT ? 1 : 2) +
-                                (e.conv ? (double)planes * nx * ny : 0.0));
-        double bytes = fixed + per;
-        const bool conv64 = sizeof(C) == 16 && e.conv;
-        const char* name = f32 ? "ifft_xy_epilogue_f32" : "ifft_xy_epilogue_f64";
-        if (e.nact) {
-            ee.bctr = dev_bytes_ptr(name);
-            ee.bfix = fixed;
-            ee.bper = per / rg;
-            bytes = kDevCounted;
+        const C* i = (const C*)in;
+        C* o = (C*)out;
+        const unsigned np = (unsigned)planes;
+        switch (h->L[0]) {
+            case 8: return launch_xy_L<8>(fwd, name, bytes, h, i, o, np, nx, ny, ee, sp, s);
+            case 16: return launch_xy_L<16>(fwd, name, bytes, h, i, o, np, nx, ny, ee, sp, s);
+            case 32: return launch_xy_L<32>(fwd, name, bytes, h, i, o, np, nx, ny, ee, sp, s);
+            case 64: return launch_xy_L<64>(fwd, name, bytes, h, i, o, np, nx, ny, ee, sp, s);
+            case 128: return launch_xy_L<128>(fwd, name, bytes, h, i, o, np, nx, ny, ee, sp, s);
         }
-        if constexpr (sizeof(C) == 16) {
-            if (conv64) {
-                VIE_KLAUNCH_B(name, s, bytes,
-                              xy_inv_kernel<L, C, true><<<(unsigned)planes, kXYThreads, smem, s>>>(
-                                  (const C*)in, (C*)out, ee, cpos, tw));
-                VIE_CHECK_LAUNCH();
-                return VIE_OK;
-            }
-        }
-        VIE_KLAUNCH_B(name, s, bytes,
-                      xy_inv_kernel<L, C, false><<<(unsigned)planes, kXYThreads, smem, s>>>((const C*)in, (C*)out, ee,
-                                                                                           cpos, tw));
+        set_error("xy transform: unsupported length");
+        return VIE_EINVAL;
     }
-    VIE_CHECK_LAUNCH();
-    return VIE_OK;
-}
-
-template <typename C>
-static int launch_xy(bool fwd, const vie_handle* h, const void* in, void* out, long long planes, int nx, int ny,
-                     const MatvecEpi& e, const Support& sp, double in_elems, cudaStream_t s) {
-    switch (h->L[0]) {
-        case 8: return launch_xy_L<8, C>(fwd, h, in, out, planes, nx, ny, e, sp, in_elems, s);
-        case 16: return launch_xy_L<16, C>(fwd, h, in, out, planes, nx, ny, e, sp, in_elems, s);
-        case 32: return launch_xy_L<32, C>(fwd, h, in, out, planes, nx, ny, e, sp, in_elems, s);
-        case 64: return launch_xy_L<64, C>(fwd, h, in, out, planes, nx, ny, e, sp, in_elems, s);
-        case 128: return launch_xy_L<128, C>(fwd, h, in, out, planes, nx, ny, e, sp, in_elems, s);
-    }
-    set_error("xy transform: unsupported length");
-    return VIE_EINVAL;
 }
 
 // Spectrum scratch of one matvec: W2 [R*12][Nz][Ly][Lx] on the fused xy path, W1
@@ -676,10 +669,11 @@ static int matvec_impl(vie_handle* h, int R, const void* x, void* y, int op, cud
                 z.mx = flip_mask(0), z.my = flip_mask(1), z.mz = flip_mask(2);
                 return zpass_f32_fused_k(h, z, s);
             }
-            if (sizeof(T) == 8 && zfused_ok(h) && h->kgreen64t) {
+            if (sizeof(T) == 8 && zfused_ok(h) && h->kgreen_d) {
                 ZDArgs z{};
                 z.w = reinterpret_cast<double2*>(W2);
-                z.green_t = h->kgreen64t;
+                z.green_d = h->kgreen_d;
+                z.gexp = h->kgreen_e;
                 z.colkx = h->colkx32;
                 z.R = Rs, z.nz = nz, z.Lx = Lx, z.Ly = Ly;
                 z.Ox = h->O[0], z.Oy = h->O[1], z.Oz = h->O[2];
@@ -736,7 +730,8 @@ static int matvec_impl(vie_handle* h, int R, const void* x, void* y, int op, cud
         if (sizeof(T) == 8 && zfused_ok(h)) {
             ZDArgs z{};
             z.w = reinterpret_cast<double2*>(W2);
-            z.green_t = h->green64t;
+            z.green_d = h->green_d;
+            z.gexp = h->green_e;
             z.colkx = h->colkx32;
             z.R = Rs, z.nz = nz, z.Lx = Lx, z.Ly = Ly;
             z.Ox = h->O[0], z.Oy = h->O[1], z.Oz = h->O[2];
@@ -1035,21 +1030,36 @@ static bool build_colmap(int L, std::vector<unsigned char>& map) {
     return true;
 }
 
+// 2^62 cos(2 pi m / L), rounded, with exact symmetry between the octants
+static long long cos_fx(int m, int L) {
+    const long double turn = 2.0L * 3.141592653589793238462643383279502884L;
+    m %= L;
+    if (2 * m > L) m = L - m;
+    if (4 * m > L) return -cos_fx(L / 2 - m, L);
+    return 8 * m <= L ? llroundl(cosl(turn * m / L) * 0x1p62L) : llroundl(sinl(turn * (L / 4.0L - m) / L) * 0x1p62L);
+}
+
 int twiddle_setup(vie_handle* h) {
     // tables for L = 2^k, k = 1..10, stored at offset L (total 2048 entries)
     const int total = 2048;
     std::vector<double2> t64(total);
     std::vector<float2> t32(total);
+    std::vector<int4> tfx(total);
     for (int L = 2; L <= 1024; L *= 2)
         for (int m = 0; m < L; ++m) {
             double ang = -2.0 * VIE_PI * (double)m / (double)L;
             double c = std::cos(ang), sn = std::sin(ang);
             t64[L + m] = make_double2(c, sn);
             t32[L + m] = make_float2((float)c, (float)sn);
+            const long long qc = cos_fx(m, L), qs = L % 4 ? 0 : cos_fx(m + L / 4, L);  // -sin a = cos(a + pi/2)
+            auto lo = [](long long q) { return std::max(fx_lo(q), -INT_MAX); };  // its negative is a word, too
+            tfx[L + m] = make_int4(fx_hi(qc), lo(qc), fx_hi(qs), lo(qs));
         }
     VIE_CUDA(cudaMalloc(&h->tw64, total * sizeof(double2)));
     VIE_CUDA(cudaMalloc(&h->tw32, total * sizeof(float2)));
-    h->bytes_held += total * (sizeof(double2) + sizeof(float2));
+    VIE_CUDA(cudaMalloc(&h->twfx, total * sizeof(int4)));
+    h->bytes_held += total * (sizeof(double2) + sizeof(float2) + sizeof(int4));
+    VIE_CUDA(cudaMemcpy(h->twfx, tfx.data(), total * sizeof(int4), cudaMemcpyHostToDevice));
     VIE_CUDA(cudaMemcpy(h->tw64, t64.data(), total * sizeof(double2), cudaMemcpyHostToDevice));
     VIE_CUDA(cudaMemcpy(h->tw32, t32.data(), total * sizeof(float2), cudaMemcpyHostToDevice));
     h->colmap = nullptr;

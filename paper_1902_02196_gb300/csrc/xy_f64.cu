@@ -1,0 +1,456 @@
+// FP64 xy transforms of the matvec (Section IV-A) on square circulants of 8..128: per plane, zero-pad
+// and transform along x and y; and back, with the crop and the voxel-wise terms.  The counterparts of
+// xy_fwd_kernel and xy_inv_kernel (matvec.cu), with the same spectrum layout, on scaled 64-bit integers
+// (fixed.cuh): sm_103a's two FP64 operations per clock and SM made these transforms take 11 to 13 ms each way
+// for 16 right-hand sides on a 64^3 grid.
+//
+// Precision.  A plane's scale is taken from its largest element.  Before each of the four passes the
+// values are brought to the bits which that pass's worst case leaves room for (fx_room): 56 to 58 of
+// them, so that a rounding is 2^-56 of the plane's largest value or less, where FP64 rounds every
+// operation to 2^-53 of its own result.
+//
+// Measured, 16 right-hand sides on 64^3 voxels (12288 planes, 128 x 128 spectra): forward 3.1 ms and inverse
+// 4.6 ms, the FP64 kernels 11.2 and 13.1 ms.
+//
+// A CTA owns one plane.  The x spectra of its rows stay in shared memory; the y transforms run on
+// chunks of CW stored columns, whose spectra go to or come from global memory in registers, 512
+// contiguous bytes to a warp.
+#include "block.cuh"
+#include "fft2.cuh"
+#include "fixed.cuh"
+#include "xy_f64.cuh"
+
+namespace {
+
+template <int L>
+struct XYCfg64 {
+    static constexpr int H = L / 2;                // rows that are non-zero before / needed after the y transform
+    static constexpr int RS = L + 1;               // odd row stride
+    static constexpr int CW = L < 32 ? L : 32;     // stored columns per y-transform chunk
+    static constexpr int NCH = L / CW;
+    static constexpr int NT = L >= 128 ? 512 : (L >= 32 ? 256 : 64);
+    static constexpr int MINB = L >= 128 ? 1 : (L >= 64 ? 2 : 4);
+    static constexpr size_t smem = sizeof(fx2) * (size_t)(L * CW + H * RS + L) + sizeof(int4) * H + 2 * L + 128;
+};
+
+// after a pass whose inputs had room for it, |v| <= 2^60.5: bits that the next pass, of n points, has
+// to drop if any value needs it (0 or log2 n + 1); the decision is the CTA's, and a barrier
+template <int N>
+__device__ __forceinline__ int rescale(unsigned key) {
+    return __syncthreads_or(fx_bits(key) > fx_room(N)) ? fx_log2(N) + 1 : 0;
+}
+__device__ __forceinline__ fx2 down(fx2 v, int k) {  // v 2^-k to nearest, k uniform
+    if (k) {
+        const long long h = 1LL << (k - 1);
+        v.x = (v.x + h) >> k;
+        v.y = (v.y + h) >> k;
+    }
+    return v;
+}
+
+// largest key of the CTA into *dst (zeroed before): followed by a barrier of the caller
+__device__ __forceinline__ void collect_max(unsigned key, unsigned* dst) {
+    key = __reduce_max_sync(0xffffffffu, key);
+    if ((threadIdx.x & 31) == 0) atomicMax(dst, key);
+}
+__device__ __forceinline__ void collect_or(unsigned key, unsigned* dst) {
+    key = __reduce_or_sync(0xffffffffu, key);
+    if ((threadIdx.x & 31) == 0) atomicOr(dst, key);
+}
+
+// Forward: plane (r, alpha, z) of x -> W2 plane [Ly][Lx] (transposed ky, stored kx).  x is
+// [R][nc][Nz][Ny][Nx], or [R][nc][ns] on a support (rows != NULL; zeros outside it).
+template <int L>
+__global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
+    xy64_fwd_kernel(const double2* __restrict__ x, double2* __restrict__ w, int nx, int ny, int nz,
+                    const int4* __restrict__ rows, long long ns, const unsigned char* __restrict__ cpos,
+                    const int4* __restrict__ twg, const int* __restrict__ rmap, MatvecEpi dc) {
+    using Cfg = XYCfg64<L>;
+    constexpr int A = fft2::Split<L>::A, B = fft2::Split<L>::B, NT = Cfg::NT, RS = Cfg::RS, CW = Cfg::CW, H = Cfg::H;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    fx2* ck = reinterpret_cast<fx2*>(smem_raw);  // [L][CW] chunk of stored columns
+    fx2* xr = ck + L * CW;                       // [H][RS] rows: the input, then its x spectra
+    int4* tw = reinterpret_cast<int4*>(xr + H * RS);
+    int4* rw = tw + L;  // [H] support rows of this plane
+    unsigned char* pos = reinterpret_cast<unsigned char*>(rw + H);
+    unsigned* keys = reinterpret_cast<unsigned*>(pos + 2 * L);  // of the input, of the x spectra
+    const int tid = threadIdx.x;
+    const long long p = blockIdx.x;  // spectrum plane; the input plane is pin (rmap: active right-hand sides)
+    const long long rplanes = (long long)dc.nc * nz;  // planes per right-hand side
+    if (dc.nact) {  // planes of right-hand sides beyond the device count are skipped
+        const int cnt = *dc.nact;
+        dev_bytes_add(dc.bctr, dc.bfix + dc.bper * cnt, cnt > 0);
+        if (p / rplanes >= cnt) return;
+    }
+    for (int m = tid; m < L; m += NT) {
+        tw[m] = twg[m];
+        pos[m] = cpos[m];
+    }
+    if (tid < 2) keys[tid] = 0;
+    const long long pin = rmap ? (long long)rmap[p / rplanes] * rplanes + p % rplanes : p;
+    const double2* src = x + pin * (long long)ny * nx;
+    if (rows) {
+        const int z = (int)(p % nz);
+        for (int yy = tid; yy < ny; yy += NT) rw[yy] = rows[(long long)z * ny + yy];
+        src = x + (pin / nz) * ns;
+    }
+    __syncthreads();
+    {
+        unsigned key = 0;
+        for (int i0 = tid; i0 < ny * nx; i0 += 4 * NT) {  // four loads in flight
+            double2 v[4];
+            int dst[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int idx = i0 + q * NT, yy = idx / nx, xx = idx - yy * nx;
+                v[q] = make_double2(0.0, 0.0);
+                dst[q] = idx < ny * nx ? yy * RS + xx : -1;
+                if (idx < ny * nx) {
+                    if (rows) {
+                        const int4 s = rw[yy];
+                        if (xx >= s.x && xx < s.y) v[q] = src[s.z + (xx - s.x)];
+                    } else {
+                        v[q] = src[idx];
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (dst[q] >= 0) {
+                    *reinterpret_cast<double2*>(xr + dst[q]) = v[q];
+                    key = max(key, fx_key(v[q]));
+                }
+        }
+        collect_max(key, keys);
+    }
+    __syncthreads();
+    const bool bad = keys[0] >= 0x7ff00000u;  // an Inf or NaN reaches the whole spectrum
+    const FxScale sc(keys[0], fx_room(A / 2));
+    int ex = sc.ex;
+    // x transform
+    unsigned key = 0;
+    for (int t = tid; t < H * B; t += NT) {
+        const int n = t % H, b = t / H;
+        if (n >= ny) continue;
+        fx2* ln = xr + n * RS;
+        fx2 v[A];
+#pragma unroll
+        for (int a = 0; a < A / 2; ++a) {
+            const int l = b + B * a;
+            v[a] = l < nx ? sc(*reinterpret_cast<const double2*>(ln + l)) : fx2{0, 0};
+        }
+        fft2::dft_half_in<A>(v, -1);
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) {
+            if (k1 && b) v[k1] = cmul(v[k1], tw[b * k1]);
+            ln[b + B * k1] = v[k1];
+            key |= fx_key(v[k1]);
+        }
+    }
+    int k = rescale<B>(key);
+    ex += k;
+    key = 0;
+    for (int t = tid; t < H * A; t += NT) {
+        const int n = t % H, k1 = t / H;
+        if (n >= ny) continue;
+        fx2* ln = xr + n * RS + B * k1;
+        fx2 v[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) v[b] = down(ln[b], k);
+        fft2::DFT<B, fx2>::run(v, -1);
+#pragma unroll
+        for (int k2 = 0; k2 < B; ++k2) {
+            ln[k2] = v[k2];
+            key |= fx_key(v[k2]);
+        }
+    }
+    collect_or(key, keys + 1);
+    __syncthreads();
+    const int ks = max(fx_bits(keys[1]) - fx_room(A / 2), 0);  // to the room of the y transform
+    ex += ks;
+    double2* dst = w + p * (long long)L * L;
+#pragma unroll 1
+    for (int c0 = 0; c0 < L; c0 += CW) {
+        // y transform, pass 1: stored column c0 + c from the x spectra.  An A-point DFT of A/2 values
+        // is two A/2-point ones, of the even and (twisted) of the odd frequencies: a task each
+        key = 0;
+        for (int t = tid; t < 2 * CW * B; t += NT) {
+            const int c = t % CW, b = (t / CW) % B, odd = t / (CW * B);
+            const fx2* col = xr + pos[c0 + c];
+            fx2 v[A / 2];
+#pragma unroll
+            for (int a = 0; a < A / 2; ++a) {  // ny <= L/2: the upper half is zero
+                const int yy = b + B * a;
+                v[a] = yy < ny ? down(col[yy * RS], ks) : fx2{0, 0};
+            }
+            if (odd) {
+#pragma unroll
+                for (int a = 0; a < A / 2; ++a) v[a] = fft2::twist<A>(v[a], a, -1);
+            }
+            fft2::DFT<A / 2, fx2>::run(v, -1);
+#pragma unroll
+            for (int q = 0; q < A / 2; ++q) {
+                const int k1 = 2 * q + odd;
+                if (b && k1) v[q] = cmul(v[q], tw[b * k1]);
+                ck[(b + B * k1) * CW + c] = v[q];
+                key |= fx_key(v[q]);
+            }
+        }
+        k = rescale<B>(key);
+        for (int t = tid; t < CW * A; t += NT) {
+            const int c = t % CW, k1 = t / CW;
+            const fx2* ln = ck + B * k1 * CW + c;
+            fx2 v[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b) v[b] = down(ln[b * CW], k);
+            fft2::DFT<B, fx2>::run(v, -1);
+#pragma unroll
+            for (int k2 = 0; k2 < B; ++k2) {
+                double2 o = fx_double(v[k2], ex + k);
+                if (bad) o.x = o.y = __longlong_as_double(0x7ff8000000000000ll);
+                dst[(long long)(B * k1 + k2) * L + c0 + c] = o;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Inverse: W2 plane -> y plane [Ny][Nx] with the material / Gram / preconditioner epilogue;
+// CONV: also the plane's (N - G) x at every voxel to epi.conv (full grid).
+template <int L, bool CONV>
+__global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
+    xy64_inv_kernel(const double2* __restrict__ w, double2* __restrict__ y, MatvecEpi epi,
+                    const unsigned char* __restrict__ cpos, const int4* __restrict__ twg) {
+    using Cfg = XYCfg64<L>;
+    constexpr int A = fft2::Split<L>::A, B = fft2::Split<L>::B, NT = Cfg::NT, RS = Cfg::RS, CW = Cfg::CW, H = Cfg::H;
+    constexpr int NCH = Cfg::NCH;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    fx2* ck = reinterpret_cast<fx2*>(smem_raw);
+    fx2* xr = ck + L * CW;
+    int4* tw = reinterpret_cast<int4*>(xr + H * RS);
+    int4* rw = tw + L;
+    unsigned char* pos = reinterpret_cast<unsigned char*>(rw + H);
+    unsigned char* chunk_of = pos + L;  // chunk of an x-transform position
+    // per chunk: the key of its spectrum, the key of its y-transformed rows, their exponent
+    unsigned* kin = reinterpret_cast<unsigned*>(pos + 2 * L);
+    unsigned* kout = kin + NCH;
+    int* cex = reinterpret_cast<int*>(kout + NCH);
+    const int tid = threadIdx.x;
+    const int nx = epi.nx, ny = epi.ny, nz = epi.nz;
+    const long long p = blockIdx.x;  // spectrum plane (r * nc + alpha) * nz + z; output plane po
+    const int nc = epi.nc;
+    const long long rplanes = (long long)nc * nz;  // planes per right-hand side
+    if (epi.nact) {
+        const int cnt = *epi.nact;
+        dev_bytes_add(epi.bctr, epi.bfix + epi.bper * cnt, cnt > 0);
+        if (p / rplanes >= cnt) return;
+    }
+    for (int m = tid; m < L; m += NT) {
+        tw[m] = twg[m];
+        pos[m] = cpos[m];
+        chunk_of[cpos[m]] = (unsigned char)(m / CW);
+    }
+    if (tid < 2 * NCH) kin[tid] = 0;
+    const long long po = epi.rmap ? (long long)epi.rmap[p / rplanes] * rplanes + p % rplanes : p;
+    if (epi.rows)
+        for (int yy = tid; yy < ny; yy += NT) rw[yy] = epi.rows[(p % nz) * ny + yy];
+    __syncthreads();
+    const double2* src = w + p * (long long)L * L;
+    bool bad = false;
+#pragma unroll 1
+    for (int h = 0; h < NCH; ++h) {
+        // inverse y transform, pass 1.  One task per thread (CW A <= NT), so its inputs wait in registers
+        // for the chunk's scale
+        static_assert(CW * A <= NT || L < 32, "one pass-1 task per thread");
+        constexpr int NTASK = (CW * A + NT - 1) / NT;
+        double2 d[NTASK][B];
+        unsigned key = 0;
+#pragma unroll
+        for (int q = 0; q < NTASK; ++q) {
+            const int t = tid + q * NT, c = t % CW, k1 = t / CW;
+#pragma unroll
+            for (int k2 = 0; k2 < B; ++k2) {
+                d[q][k2] = t < CW * A ? src[(long long)(B * k1 + k2) * L + h * CW + c] : make_double2(0.0, 0.0);
+                key = max(key, fx_key(d[q][k2]));
+            }
+        }
+        collect_max(key, kin + h);
+        __syncthreads();
+        bad = bad || kin[h] >= 0x7ff00000u;
+        const FxScale sc(kin[h], fx_room(B));
+        key = 0;
+#pragma unroll
+        for (int q = 0; q < NTASK; ++q) {
+            const int t = tid + q * NT, c = t % CW, k1 = t / CW;
+            if (t >= CW * A) continue;
+            fx2 v[B];
+#pragma unroll
+            for (int k2 = 0; k2 < B; ++k2) v[k2] = sc(d[q][k2]);
+            fft2::DFT<B, fx2>::run(v, +1);
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                if (b && k1) v[b] = cmul(v[b], fx_conj(tw[b * k1]));
+                ck[(b + B * k1) * CW + c] = v[b];
+                key |= fx_key(v[b]);
+            }
+        }
+        const int k = rescale<A>(key);
+        // pass 2: rows y < Ny scattered to the x-transform buffer at the column's x position
+        key = 0;
+        for (int t = tid; t < CW * B; t += NT) {
+            const int c = t % CW, b = t / CW;
+            fx2 v[A];
+#pragma unroll
+            for (int k1 = 0; k1 < A; ++k1) v[k1] = down(ck[(b + B * k1) * CW + c], k);
+            fft2::dft_half_out<A>(v, +1);
+            fx2* col = xr + pos[h * CW + c];
+#pragma unroll
+            for (int a = 0; a < A / 2; ++a) {  // ny <= L/2
+                const int yy = b + B * a;
+                if (yy < ny) {
+                    col[yy * RS] = v[a];
+                    key |= fx_key(v[a]);
+                }
+            }
+        }
+        collect_or(key, kout + h);
+        if (tid == 0) cex[h] = sc.ex + k;
+        __syncthreads();
+    }
+    const long long base = po * (long long)ny * nx;
+    const long long cbase = (po / nz) * epi.ns;  // component block on the support
+    const double2* xin = reinterpret_cast<const double2*>(epi.x);
+    // the epilogue's x values of this plane arrive in the free chunk buffer during the x transform
+    const bool pre = epi.op != VIE_OP_NSCAT && L * CW >= ny * nx;
+    if (pre) {
+        for (int idx = tid; idx < ny * nx; idx += NT) {
+            const int yy = idx / nx, xx = idx % nx;
+            long long o = base + idx;
+            bool in = true;
+            if (epi.rows) {
+                const int4 q = rw[yy];
+                in = xx >= q.x && xx < q.y;
+                o = in ? cbase + q.z + (xx - q.x) : cbase;
+            }
+            cp_async_elem(reinterpret_cast<double2*>(ck) + idx, xin + o, in);
+        }
+        cp_async_commit();
+    }
+    // inverse x transform: the chunks' columns on the scale of the largest
+    int E = -100000;
+#pragma unroll
+    for (int h = 0; h < NCH; ++h) E = max(E, fx_bits(kout[h]) + cex[h]);
+    int ex = E - fx_room(B);
+    unsigned key = 0;
+    for (int t = tid; t < H * A; t += NT) {
+        const int n = t % H, k1 = t / H;
+        if (n >= ny) continue;
+        fx2* ln = xr + n * RS + B * k1;
+        fx2 v[B];
+#pragma unroll
+        for (int k2 = 0; k2 < B; ++k2) {
+            const int s = max(cex[chunk_of[B * k1 + k2]] - ex, -63);  // <= 25: the key counts 32 bits at least
+            const fx2 u = ln[k2];
+            v[k2] = s >= 0 ? fx2{u.x << s, u.y << s} : fx2{u.x >> -s, u.y >> -s};
+        }
+        fft2::DFT<B, fx2>::run(v, +1);
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            if (b && k1) v[b] = cmul(v[b], fx_conj(tw[b * k1]));
+            ln[b] = v[b];
+            key |= fx_key(v[b]);
+        }
+    }
+    const int k = rescale<A>(key);
+    ex += k;
+    for (int t = tid; t < H * B; t += NT) {
+        const int n = t % H, b = t / H;
+        if (n >= ny) continue;
+        fx2* ln = xr + n * RS;
+        fx2 v[A];
+#pragma unroll
+        for (int k1 = 0; k1 < A; ++k1) v[k1] = down(ln[b + B * k1], k);
+        fft2::dft_half_out<A>(v, +1);
+#pragma unroll
+        for (int a = 0; a < A / 2; ++a) {
+            const int l = b + B * a;
+            if (l < nx) ln[l] = v[a];
+        }
+    }
+    if (pre) cp_async_wait<0>();
+    __syncthreads();
+    const int alpha = (int)((p / nz) % nc);
+    const long long zoff = (p % nz) * (long long)ny * nx;
+    const double gl = comp_is_constant(alpha, nc) ? epi.g1 : epi.g234;
+    const double ig = 1.0 / gl;
+    const double2* c1 = reinterpret_cast<const double2*>(epi.c1);
+    const double2* c2 = reinterpret_cast<const double2*>(epi.c2);
+    const double2 sh = epi.shift ? epi.shift[po / rplanes] : make_double2(0.0, 0.0);  // op PA
+    double2* conv = CONV ? reinterpret_cast<double2*>(epi.conv) : nullptr;
+#pragma unroll 4
+    for (int idx = tid; idx < ny * nx; idx += NT) {
+        const int yy = idx / nx, xx = idx % nx;
+        long long o = base + idx;
+        bool in = true;
+        if (epi.rows) {
+            const int4 q = rw[yy];
+            in = xx >= q.x && xx < q.y;
+            o = cbase + q.z + (xx - q.x);
+        }
+        if (!CONV && !in) continue;
+        double2 v = fx_double(xr[yy * RS + xx], ex);
+        if (bad) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+        if (CONV) conv[base + idx] = v;  // every voxel of the plane, full-grid layout
+        if (!in) continue;
+        if (epi.op == VIE_OP_A) {
+            const double2 xv = pre ? reinterpret_cast<const double2*>(ck)[idx] : xin[o];
+            v = csub(mk(gl * xv.x, gl * xv.y), cmul(c2[zoff + idx], v));
+        } else if (epi.op == VIE_OP_PA) {
+            const double2 xv = pre ? reinterpret_cast<const double2*>(ck)[idx] : xin[o];
+            const double2 t = cmul(c2[zoff + idx], v);
+            v = csub(cmul(csub(c1[zoff + idx], sh), xv), mk(ig * t.x, ig * t.y));
+        }
+        y[o] = v;
+    }
+}
+
+template <int L>
+int launch_L(bool fwd, const char* name, double bytes, const vie_handle* h, const double2* in, double2* out,
+             unsigned planes, int nx, int ny, const MatvecEpi& e, const Support& sp, cudaStream_t s) {
+    using Cfg = XYCfg64<L>;
+    // set on every call: the attribute is per device and launches may come from several threads
+    auto attr = [](auto kernel) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem);
+    };
+    const unsigned char* cpos = h->colmap + L;
+    const int4* tw = h->twfx + L;
+    if (fwd) {
+        VIE_CUDA(attr(xy64_fwd_kernel<L>));
+        VIE_KLAUNCH_B(name, s, bytes,
+                      xy64_fwd_kernel<L><<<planes, Cfg::NT, Cfg::smem, s>>>(in, out, nx, ny, h->nz, sp.rows, sp.ns, cpos,
+                                                                           tw, e.rmap, e));
+    } else if (e.conv) {
+        VIE_CUDA(attr(xy64_inv_kernel<L, true>));
+        VIE_KLAUNCH_B(name, s, bytes, (xy64_inv_kernel<L, true><<<planes, Cfg::NT, Cfg::smem, s>>>(in, out, e, cpos, tw)));
+    } else {
+        VIE_CUDA(attr(xy64_inv_kernel<L, false>));
+        VIE_KLAUNCH_B(name, s, bytes, (xy64_inv_kernel<L, false><<<planes, Cfg::NT, Cfg::smem, s>>>(in, out, e, cpos, tw)));
+    }
+    VIE_CHECK_LAUNCH();
+    return VIE_OK;
+}
+
+}  // namespace
+
+int xy_f64(bool fwd, const char* name, double bytes, const vie_handle* h, const double2* in, double2* out,
+           unsigned planes, int nx, int ny, const MatvecEpi& e, const Support& sp, cudaStream_t s) {
+    switch (h->L[0]) {
+        case 8: return launch_L<8>(fwd, name, bytes, h, in, out, planes, nx, ny, e, sp, s);
+        case 16: return launch_L<16>(fwd, name, bytes, h, in, out, planes, nx, ny, e, sp, s);
+        case 32: return launch_L<32>(fwd, name, bytes, h, in, out, planes, nx, ny, e, sp, s);
+        case 64: return launch_L<64>(fwd, name, bytes, h, in, out, planes, nx, ny, e, sp, s);
+        case 128: return launch_L<128>(fwd, name, bytes, h, in, out, planes, nx, ny, e, sp, s);
+    }
+    set_error("xy transform: unsupported length");
+    return VIE_EINVAL;
+}

@@ -1,169 +1,515 @@
-// FP64 z pass of the matvec (Section IV-A) with the 12 x 12 Green block product fused
-// between the forward and inverse z transforms: the FP64 counterpart of zpass_f32.cu, for
-// the refinement residuals, the post-processing and the plain FP64 solver; the N block from
-// its 60 tensors, or (KOP) the K block (Eq. 8, 25) from its 30.
+// FP64 z pass of the matvec (Section IV-A) with the 12 x 12 Green block product fused between the
+// forward and inverse z transforms: the FP64 counterpart of zpass_f32.cu, for the refinement
+// residuals, the post-processing and the plain FP64 solver; the N block from its 60 tensors, or
+// (KOP) the K block (Eq. 8, 25) from its 30.
 //
-// Same tiling, item decoding and transposed z spectrum as the FP32 kernel.  FP64 values
-// take twice the registers, so a thread cannot keep an octant point's 60 Green values
-// resident: each frequency point streams them from the [..][60] layout in four groups of
-// 15 tensors (960 contiguous bytes per point, served by L1/L2 for the four points of an
-// item), and applies each group to the entries it feeds, one column at a time.  The
-// kernel is bound by the FP64 pipe, so one shared-memory buffer per CTA suffices: two
-// CTAs per SM overlap one's loads and stores with the other's arithmetic.
+// sm_103a has two FP64 operations per clock and SM, which this pass would need 290 clocks of per
+// frequency point for the product alone and 110 more for the transforms.  So it runs on
+// scaled integers (fixed.cuh) and on the tensor cores:
+//  - a CTA owns one ky row and one mirror pair of columns and loops over groups of RB right-hand
+//    sides, 24 RB lines in shared memory.  The two lines of a component share one power-of-two
+//    scale, taken from their largest element, and the transforms are those of fft2.cuh on 64-bit
+//    integers;
+//  - the block product is exact up to its last digits: with X the spectrum and B the block in 62
+//    bits below their largest values (the digit tables of green_digits), both are cut into seven
+//    signed 9-bit digits, X = sum_i x_i 2^(9(6-i)), and the products of digits with i + j <= 6 are
+//    summed by fp16 mma.sync into FP32, where every sum is an integer below 2^22 and so exact (the
+//    splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012).  The dropped digits
+//    are 2^-59 of the product, where FP64 rounds its operands and every sum to 2^-53;
+//  - the accumulators start at 1.5 2^23, so that their bit patterns are the integers and no
+//    conversion instruction (16 per clock) is needed.
+//
+// Measured, 16 right-hand sides on 64^3 voxels (Lx = Ly = Lz = 128): 15.3 ms, the FP64 kernel of the same
+// structure 70.8 ms; the K block of 8 right-hand sides 6.5 ms against 29.1 ms.  The bound is instruction
+// issue: 260 warp instructions per frequency point, half of them the product (digits, sums, recombination).
+// 2-norm error against long double sums 0.6 to 1.0 times the FP64 kernel's.
+//
+// Roles in the mma: the 24 x 24 real form of B (rows re, im of the outputs; columns re, im of the
+// inputs) is the 16-row operand, the points that share an octant point, +-kx, +-kz and RB = 2
+// right-hand sides, are its 8 columns.  A lane's share of X is then three whole complex values and
+// no digit is built twice.  Rows 0..15 take one instruction; rows 16..23 fill both halves of
+// another with two successive digits of B, whose products belong to successive weights.
+#include <cuda_fp16.h>
+
 #include "block.cuh"
 #include "fft2.cuh"
+#include "fixed.cuh"
 #include "zpass_f64.cuh"
 
 namespace {
 
+constexpr int kD = 7;  // digits of the spectrum and of the block
+constexpr unsigned kMagicBits = 0x4B400000u;  // 1.5 2^23
+// 256 in each digit: makes them 0..511 in a plain bit field
+constexpr unsigned long long kBias =
+    256ull * ((1ull << 54) + (1ull << 45) + (1ull << 36) + (1ull << 27) + (1ull << 18) + (1ull << 9) + 1);
+constexpr int kBits = 62;   // |X|, |B| < 2^62
+constexpr int kShift = 68;  // Y = X B 2^-68: |Y| < 24 2^(62 + 62 - 68) < 2^61
+
 template <int LZ>
 struct ZDCfg {
-    static constexpr int TB = LZ <= 128 ? 4 : 2;
-    static constexpr int NPAIR = TB / 2;
-    static constexpr int NT0 = NPAIR * LZ / 2;
-    static constexpr int NT = NT0 < 128 ? 128 : NT0;
-    static constexpr int GS = LZ * TB + TB;  // 16-byte elements: quarter-warps of 8 lines stay apart
-    static constexpr int BUF = 12 * GS;
-    static constexpr size_t smem = sizeof(double2) * (size_t)(BUF + LZ);
+    static constexpr int RB = LZ <= 256 ? 2 : 1;  // right-hand sides per group
+    static constexpr int NL = 24 * RB;            // lines: RB x 12 components x 2 columns
+    static constexpr int NT = LZ <= 8 ? 96 : (LZ <= 128 ? 192 : 384);
+    static constexpr int MINB = LZ <= 128 ? 2 : 1;
+    static constexpr int GS = 2 * LZ + 2;  // component stride: four components and two columns on distinct banks
+    static constexpr size_t smem = sizeof(fx2) * (size_t)(RB * 12 * GS + LZ) + 4 * 32 * RB + (size_t)(NT / 32) * 60 * 32;
 };
 
-__device__ __forceinline__ double2 xflip64(double2 v, unsigned m, int a) { return ((m >> a) & 1u) ? cneg(v) : v; }
-
-// entries [start(t), start(t + 1)) of the N table (60 tensors) or of the K table (30)
-template <bool KOP>
-__device__ __forceinline__ int entry_start(int t) {
-    if constexpr (KOP)
-        return kKBlock.start[t];
-    else
-        return kBlock.start[t];
+__device__ __forceinline__ void mma16(float* c, unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
+                                      unsigned b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-template <bool KOP>
-__device__ __forceinline__ BlockEntry entry_at(int i) {
-    if constexpr (KOP)
-        return kKBlock.e[i];
-    else
-        return kBlock.e[i];
+// the first of a sum: starts at 1.5 2^23
+__device__ __forceinline__ void mma16s(float* c, unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
+                                       unsigned b1) {
+    const float m = __uint_as_float(kMagicBits);
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};\n"
+        : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(m));
+}
+__device__ __forceinline__ void mma8(float* c, unsigned a0, unsigned a1, unsigned b0) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};\n"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a0), "r"(a1), "r"(b0));
 }
 
-// y = B x at one column of one z position, the Green values streamed from gp (NG = 60 values of
-// N, or 30 of K); input signs m, output signs mo
-template <bool KOP>
-__device__ __forceinline__ void point_product64(const double2* __restrict__ gp, double2* s, int gs, int off,
-                                                unsigned m, unsigned mo) {
-    constexpr int NGRP = KOP ? 2 : 4;  // groups of 15 tensors
-    double2 xv[12], acc[12];
+// Sums of digit products of weight d: S_d = sum over i + j = d of (digit i of X) (digit j of B),
+// for the lane's rows g, g + 8 (s[0..3]) and g + 16 (s[4], s[5]), columns 2t and 2t + 1.  A sum of 24
+// products is below 2^20.6, so an accumulator takes two of them.  Rows g + 16: the lower half of the
+// instruction's rows has the even digits j, the upper one j + 1, whose products have weight d + 1 and
+// come back in next[2] (carry[2] of the call before).
+template <int D>
+__device__ __forceinline__ void digit_sums(const unsigned (&a)[3][3][kD], const unsigned (&b)[3][kD], int* s,
+                                           const unsigned* carry, unsigned* next) {
+    unsigned t[6] = {0, 0, 0, 0, carry[0], carry[1]};
 #pragma unroll
-    for (int b = 0; b < 12; ++b) xv[b] = xflip64(s[b * gs + off], m, b);
+    for (int j = 0; j <= D; j += 2) {
+        const int i = D - j;
+        float c[4];
+        mma16s(c, a[0][0][j], a[1][0][j], a[0][1][j], a[1][1][j], b[0][i], b[1][i]);
+        if (j + 1 <= D) {
+            mma16(c, a[0][2][j], a[1][2][j], a[0][2][j + 1], a[1][2][j + 1], b[2][i], b[2][i - 1]);
+            mma16(c, a[0][0][j + 1], a[1][0][j + 1], a[0][1][j + 1], a[1][1][j + 1], b[0][i - 1], b[1][i - 1]);
+        } else {
+            mma8(c, a[0][2][j], a[1][2][j], b[2][i]);
+        }
 #pragma unroll
-    for (int a = 0; a < 12; ++a) acc[a] = make_double2(0.0, 0.0);
+        for (int q = 0; q < 4; ++q) t[q] += __float_as_uint(c[q]) - kMagicBits;
+    }
+    next[0] = next[1] = 0;
 #pragma unroll
-    for (int g = 0; g < NGRP; ++g) {
-        double2 u[15];
+    for (int j = 0; j <= D; j += 4) {  // even digits two at a time: j with D - j, j + 2 with D - j - 2
+        const int i = D - j;
+        // digit j + 1 of the upper half (past the last one: none)
+        auto up = [&](int e, int d) { return d < kD ? a[2][e][d] : 0u; };
+        float c[4];
+        mma16s(c, a[2][0][j], up(0, j + 1), a[2][1][j], up(1, j + 1), b[0][i], b[1][i]);
+        if (j + 2 <= D) {
+            mma16(c, a[2][2][j], up(2, j + 1), a[2][2][j + 2], up(2, j + 3), b[2][i], b[2][i - 2]);
+            mma16(c, a[2][0][j + 2], up(0, j + 3), a[2][1][j + 2], up(1, j + 3), b[0][i - 2], b[1][i - 2]);
+        } else {
+            mma8(c, a[2][2][j], up(2, j + 1), b[2][i]);
+        }
 #pragma unroll
-        for (int q = 0; q < 15; ++q) u[q] = __ldg(gp + 15 * g + q);
-#pragma unroll
-        for (int q = 0; q < 15; ++q) {
-            const int t = 15 * g + q;
-#pragma unroll
-            for (int i = entry_start<KOP>(t); i < entry_start<KOP>(t + 1); ++i) {
-                const BlockEntry en = entry_at<KOP>(i);
-                cfma(acc[en.a], en.s > 0 ? u[q] : cneg(u[q]), xv[en.b]);
-            }
+        for (int q = 0; q < 2; ++q) {
+            t[4 + q] += __float_as_uint(c[q]) - kMagicBits;
+            next[q] += __float_as_uint(c[2 + q]) - kMagicBits;
         }
     }
 #pragma unroll
-    for (int a = 0; a < 12; ++a) s[a * gs + off] = xflip64(acc[a], mo, a);
+    for (int q = 0; q < 6; ++q) s[q] = (int)t[q];
 }
 
+// Y = sum_d S_d 2^(9 (12 - d) - kShift) for the lane's six values
+__device__ __forceinline__ void block_digits(const unsigned (&a)[3][3][kD], const unsigned (&b)[3][kD], long long* y) {
+    unsigned h[2] = {0, 0}, g[2];
+    int s[6], low[6];
+    digit_sums<0>(a, b, s, h, g);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) y[q] = (long long)s[q] << 40;
+    digit_sums<1>(a, b, s, g, h);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) y[q] += (long long)s[q] << 31;
+    digit_sums<2>(a, b, s, h, g);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) y[q] = fx_mad(s[q], 1 << 22, y[q]);
+    digit_sums<3>(a, b, s, g, h);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) y[q] = fx_mad(s[q], 1 << 13, y[q]);
+    digit_sums<4>(a, b, s, h, g);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) low[q] = s[q] * 16;
+    digit_sums<5>(a, b, s, g, h);
+    int t5[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) t5[q] = s[q] + 16;
+    digit_sums<6>(a, b, s, h, g);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) y[q] += low[q] + ((t5[q] + ((s[q] + 256) >> 9)) >> 5);
+}
+
+// Digits of one complex value as fp16 pairs (re, im), most significant first: w = v 2^sh + bias,
+// fields 0..511 (the top one to 1023); the fp16 1024 + u is 0x6400 | u.  sg (+-1, +-1) flips the sign.
+__device__ __forceinline__ void split_digits(fx2 v, int sh, __half2 sg, unsigned* d) {
+    const unsigned long long re = (unsigned long long)(sh >= 0 ? v.x << sh : v.x >> -sh) + kBias;
+    const unsigned long long im = (unsigned long long)(sh >= 0 ? v.y << sh : v.y >> -sh) + kBias;
+    const unsigned rl = (unsigned)re, rh = (unsigned)(re >> 32), il = (unsigned)im, ih = (unsigned)(im >> 32);
+    const unsigned lo = 0x1ffu, hi = 0x1ff0000u, mg = 0x64006400u;
+    unsigned u[kD];
+    u[6] = (rl & lo) | mg | ((il << 16) & hi);
+    u[5] = ((rl >> 9) & lo) | mg | ((il << 7) & hi);
+    u[4] = ((rl >> 18) & lo) | mg | ((il >> 2) & hi);
+    u[3] = (__funnelshift_r(rl, rh, 27) & lo) | mg | (__funnelshift_r(il, ih, 11) & hi);
+    u[2] = ((rh >> 4) & lo) | mg | ((ih << 12) & hi);
+    u[1] = ((rh >> 13) & lo) | mg | ((ih << 3) & hi);
+    u[0] = ((rh >> 22) & 0x3ffu) | mg | ((ih >> 6) & 0x3ff0000u);
+    const __half2 off = __hmul2(sg, __float2half2_rn(-1280.f));  // 1024 + 256
+#pragma unroll
+    for (int i = 0; i < kD; ++i) {
+        const __half2 r = __hfma2(*reinterpret_cast<__half2*>(&u[i]), sg, off);
+        d[i] = *reinterpret_cast<const unsigned*>(&r);
+    }
+}
+
+__device__ __forceinline__ int pos_of(int L, int k) { return fft2::tpos(L, k); }
+
 template <int LZ, bool KOP>
-__global__ void __launch_bounds__(ZDCfg<LZ>::NT) zfused64_kernel(ZDArgs z, const double2* __restrict__ twg) {
+__global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
+    zfused64_kernel(ZDArgs z, const int4* __restrict__ twg) {
     using Cfg = ZDCfg<LZ>;
-    constexpr int NG = KOP ? 30 : 60;  // Green values per octant point
-    constexpr int A = fft2::Split<LZ>::A, B = fft2::Split<LZ>::B, NT = Cfg::NT, TB = Cfg::TB;
-    constexpr int NPAIR = Cfg::NPAIR, GS = Cfg::GS;
+    constexpr int NG = KOP ? 30 : 60;  // tensors per octant point
+    constexpr int A = fft2::Split<LZ>::A, B = fft2::Split<LZ>::B, NT = Cfg::NT, RB = Cfg::RB, GS = Cfg::GS, NL = Cfg::NL;
+    // bits of the inputs of the forward transform, and of the two passes of the inverse one
+    constexpr int TF = fx_room(LZ / 2), TI1 = fx_room(B), TI2 = fx_room(A);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    double2* s = reinterpret_cast<double2*>(smem_raw);
-    double2* tw = s + Cfg::BUF;
-    const int tid = threadIdx.x;
+    fx2* s = reinterpret_cast<fx2*>(smem_raw);
+    int4* tw = reinterpret_cast<int4*>(s + RB * 12 * GS);
+    // largest elements (fx_key): [RB][12] of the inputs and of the spectrum of each component, [RB] of the
+    // product and after the inverse's first pass; [RB] the exponent of X, [RB] Inf or NaN among the inputs
+    unsigned* kin = reinterpret_cast<unsigned*>(tw + LZ);
+    unsigned *kspec = kin + 12 * RB, *kout = kspec + 12 * RB, *kmid = kout + RB;
+    int *xexp = reinterpret_cast<int*>(kmid + RB), *bad = xexp + RB;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    // the digits of the warp's next octant point, copied while the current one is multiplied
+    uint4* gbuf = reinterpret_cast<uint4*>(kin + 32 * RB) + wid * (NG * 2);
     const int R = z.nact ? min(*z.nact, z.R) : z.R;
     dev_bytes_add(z.bctr, 16.0 * (2.0 * R * 12 * z.nz * z.Ly * z.Lx + (double)NG * z.Ox * z.Oy * z.Oz), R > 0);
     if (R <= 0) return;
     for (int m = tid; m < LZ; m += NT) tw[m] = twg[m];
-    const int ntile = z.Lx / TB;
-    const int py = blockIdx.x / ntile, ct = blockIdx.x % ntile, sc0 = ct * TB;
+    if (tid < 26 * RB) kin[tid] = 0;
+    __syncthreads();
+    const int ntile = z.Lx / 2;
+    const int py = blockIdx.x / ntile, ct = blockIdx.x % ntile, sc0 = 2 * ct;
     const long long plane = (long long)z.Ly * z.Lx;
     const int ky = py / z.by + z.ay * (py % z.by);
     const int kyo = ky <= z.Ly / 2 ? ky : z.Ly - ky;
     const unsigned fy = ky > z.Ly / 2 ? z.my : 0u;
-    const int nz = z.nz;
-    auto line = [](int n) { return (n / TB) * GS + n % TB; };
-    // K: the block's overall sign flips at points reflected along an odd number of axes
-    const unsigned ko = KOP ? 0xFFFu : 0u;
     const bool ry = ky > z.Ly / 2;
-
-    // block-product item of this thread (as in the FP32 kernel)
-    const int ci = tid % NPAIR, j = tid / NPAIR;
-    const bool single = ct == ntile - 1 && ci == NPAIR - 1;
-    const int kx0 = z.colkx[sc0 + 2 * ci], kx1 = z.colkx[sc0 + 2 * ci + 1];
-    const unsigned fx0 = kx0 > z.Lx / 2 ? z.mx : 0u, fx1 = kx1 > z.Lx / 2 ? z.mx : 0u;
-    constexpr int NREG = (A / 2 - 1) * B;
-    int pa = -1, pb = -1, pc = -1;
-    if (j < NREG) {
-        const int k1 = 1 + j / B, k2 = j % B;
-        pa = k2 + B * k1;
-        pb = (B - 1 - k2) + B * (A - k1);
-    } else if (j < NREG + B / 2) {
-        const int k2 = j - NREG;
-        pa = k2 + B * (A / 2);
-        pb = (B - 1 - k2) + B * (A / 2);
-    } else if (j < LZ / 2) {
-        const int k2 = j - NREG - B / 2;
-        pa = k2;
-        if (k2 == 0)
-            pc = B / 2;
-        else
-            pb = B - k2;
-    }
+    const int nz = z.nz;
+    const unsigned nzq = 0xffffffffu / (unsigned)nz + 1u;  // idx / nz = umulhi(idx, nzq) for idx < 2^14, nz <= 512 (nz > 1)
+    const bool single = ct == ntile - 1;  // columns 0 and Lx/2: own octant columns
+    const int kx0 = z.colkx[sc0], kx1 = z.colkx[sc0 + 1];
     const int kxo0 = kx0 <= z.Lx / 2 ? kx0 : z.Lx - kx0, kxo1 = kx1 <= z.Lx / 2 ? kx1 : z.Lx - kx1;
-    const double2* gcol0 = z.green_t + ((long long)kyo * z.Ox + kxo0) * z.Oz * NG;
-    const double2* gcol1 = z.green_t + ((long long)kyo * z.Ox + kxo1) * z.Oz * NG;
+    const unsigned fx0 = kx0 > z.Lx / 2 ? z.mx : 0u, fx1 = kx1 > z.Lx / 2 ? z.mx : 0u;
+    const int gc0 = kyo * z.Ox + kxo0, gc1 = kyo * z.Ox + kxo1;
+    const int gex0 = z.gexp[gc0], gex1 = z.gexp[gc1];
+
+    // block-product roles of this lane.  Points (mma columns) 0..7: bit 0 the column, bit 1 the sign of
+    // kz, bit 2 the right-hand side; n is the point whose X this lane splits, components t, t + 4, t + 8.
+    const int n = lane >> 2, t = lane & 3;
+    const int ncol = n & 1, nneg = (n >> 1) & 1, nr_ = n >> 2;
+    const int qcol = t & 1;  // of the outputs (points 2t, 2t + 1): the sign of kz; t >> 1 the right-hand side
+    const int ra = (lane >> 2) >> 1, part = (lane >> 2) & 1;  // output rows: components ra, ra + 4, ra + 8, re or im
+    // B: entry (row component 4 p + ra, input 4 q + t): scalar pair (ra, t), vector pair (p, q)
+    const int l0 = min(ra, t), l1 = max(ra, t);
+    const int ll = l0 == 0 ? l1 : (l0 == 1 ? 3 + l1 : (l0 == 2 ? 5 + l1 : 9));  // ll_index
+    const bool swapneg = ra > t && (((ra > 0) + (t > 0)) & 1);  // l > l' with one of them constant: sign -1
+    // re rows take (Br, -Bi), im rows (Bi, Br)
+    const unsigned bsel = part ? 0x1032u : 0x3210u;
+    const unsigned bneg = (part ? 0u : 0x80000000u) ^ (swapneg ? 0x80008000u : 0u);
+
+    // octant points q of this CTA: 0..LZ/2, for each column when the columns are self-mirrored
+    constexpr int NO = LZ / 2 + 1, NW = NT / 32;
+    const int nq = single ? 2 * NO : NO;
+    auto fetch = [&](int q) {
+        const bool col = q >= NO;
+        const uint4* src = z.green_d + ((long long)(col ? gc1 : gc0) * z.Oz + (q - (col ? NO : 0))) * (NG * 2);
+        for (int i = lane; i < NG * 2; i += 32) cp_async16(gbuf + i, src + i);
+        cp_async_commit();
+    };
+    if (wid < nq) fetch(wid);
 
 #pragma unroll 1
-    for (int r = 0; r < R; ++r) {
-        const double2* base = z.w + (long long)r * 12 * nz * plane + (long long)py * z.Lx + sc0;
-        for (int idx = tid; idx < 12 * nz * TB; idx += NT) {
-            const int c = idx % TB, l = (idx / TB) % nz, a = idx / (TB * nz);
-            cp_async16(s + a * GS + l * TB + c, base + ((long long)a * nz + l) * plane + c);
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-        __syncthreads();
-        fft2::forward<LZ, NT>(s, 12 * TB, line, TB, tw, nz);
-        if (pa >= 0) {
-            // points (pa, pb: one octant point; pc: kz = LZ/2), each column with its octant point
+    for (int r0 = 0; r0 < R; r0 += RB) {
+        const int nr = min(RB, R - r0);
+        // load, with the largest element of each component
 #pragma unroll 1
-            for (int q = 0; q < 6; ++q) {
-                const int e = q % 3, col = q / 3;
-                const int pp = e == 0 ? pa : (e == 1 ? pb : pc);
-                if (pp < 0) continue;
-                const int kz = fft2::freq_at(LZ, pp);
-                const int kzo = kz <= LZ / 2 ? kz : LZ - kz;
-                const bool rz = kz > LZ / 2;
-                const unsigned fz = rz ? z.mz : 0u;
-                const double2* gp = ((single && col) ? gcol1 : gcol0) + (long long)kzo * NG;
-                const unsigned mi = fy ^ fz ^ (col ? fx1 : fx0);
-                const bool odd = ry ^ rz ^ (col ? kx1 > z.Lx / 2 : kx0 > z.Lx / 2);
-                point_product64<KOP>(gp, s, GS, pp * TB + 2 * ci + col, mi, odd ? mi ^ ko : mi);
+        for (int rr = 0; rr < nr; ++rr) {
+            const double2* base = z.w + (long long)(r0 + rr) * 12 * nz * plane + (long long)py * z.Lx + sc0;
+#pragma unroll 1
+            for (int i0 = tid - lane; i0 < 24 * nz; i0 += 8 * NT) {  // eight loads in flight
+                double2 v[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int idx = i0 + q * NT + lane;
+                    v[q] = idx < 24 * nz ? base[(long long)(idx >> 1) * plane + (idx & 1)] : make_double2(0.0, 0.0);
+                }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const int idx = i0 + q * NT + lane, e = min(idx >> 1, 12 * nz - 1);
+                    const int a = nz > 1 ? (int)__umulhi((unsigned)e, nzq) : e;
+                    if (idx < 24 * nz) *reinterpret_cast<double2*>(s + (rr * 12 + a) * GS + 2 * (e - a * nz) + (idx & 1)) = v[q];
+                    const unsigned key = fx_key(v[q]);
+                    if (__all_sync(0xffffffffu, a == __shfl_sync(0xffffffffu, a, 0))) {
+                        const unsigned m = __reduce_max_sync(0xffffffffu, key);
+                        if (lane == 0) atomicMax(kin + rr * 12 + a, m);
+                    } else {
+                        atomicMax(kin + rr * 12 + a, key);
+                    }
+                }
             }
         }
         __syncthreads();
-        fft2::inverse<LZ, NT>(s, 12 * TB, line, TB, tw, nz);
-        double2* out = z.w + (long long)r * 12 * nz * plane + (long long)py * z.Lx + sc0;
-        for (int idx = tid; idx < 12 * nz * TB; idx += NT) {
-            const int c = idx % TB, l = (idx / TB) % nz, a = idx / (TB * nz);
-            out[((long long)a * nz + l) * plane + c] = s[a * GS + l * TB + c];
+        // forward z transform; pass 1 (A points, the upper half zero) converts to fixed point
+        for (int w = tid; w < NL * B; w += NT) {
+            const int ln = w % NL, b = w / NL, rr = ln / 24;
+            if (RB > 1 && rr >= nr) continue;
+            const FxScale sc(kin[ln >> 1], TF);
+            fx2* p = s + (ln >> 1) * GS + (ln & 1);
+            fx2 v[A];
+#pragma unroll
+            for (int a = 0; a < A / 2; ++a) {
+                const int l = b + B * a;
+                v[a] = l < nz ? sc(*reinterpret_cast<const double2*>(p + 2 * l)) : fx2{0, 0};
+            }
+            fft2::dft_half_in<A>(v, -1);
+#pragma unroll
+            for (int k1 = 1; k1 < A; ++k1)
+                if (b) v[k1] = cmul(v[k1], tw[b * k1]);
+#pragma unroll
+            for (int k1 = 0; k1 < A; ++k1) p[2 * (b + B * k1)] = v[k1];
         }
         __syncthreads();
+        for (int w = tid; w < NL * A; w += NT) {
+            const int ln = w % NL, k1 = w / NL;
+            if (RB > 1 && ln / 24 >= nr) continue;
+            fx2* p = s + (ln >> 1) * GS + (ln & 1) + 2 * B * k1;
+            fx2 v[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b) v[b] = p[2 * b];
+            fft2::DFT<B, fx2>::run(v, -1);
+            unsigned m = 0;
+#pragma unroll
+            for (int k2 = 0; k2 < B; ++k2) {
+                p[2 * k2] = v[k2];
+                m |= fx_key(v[k2]);
+            }
+            atomicOr(kspec + (ln >> 1), m);
+        }
+        __syncthreads();
+        // block product, a warp per octant point
+        {
+            const int nrx = RB == 1 ? 0 : nr_;
+            const bool nval = RB == 1 ? nr_ == 0 : nr_ < nr;
+            const int rout = t >> 1;
+            const bool oval = RB == 1 ? rout == 0 : rout < nr;
+            // X = spectrum 2^(kBits - E), the linear components' a quarter of that (their rows and
+            // columns of B are raised by 4): E the exponent of the largest
+            int E = 0, sh[3];
+#pragma unroll
+            for (int rr = 0; rr < RB; ++rr) {
+                int e = -100000;
+                bool b = false;
+                if (lane < 12) {
+                    const unsigned k = kin[rr * 12 + lane];
+                    e = fx_bits(kspec[rr * 12 + lane]) + FxScale(k, TF).ex - (lane % 4 ? 2 : 0);
+                    b = k >= 0x7ff00000u;
+                }
+                e = __reduce_max_sync(0xffffffffu, e);
+                b = __any_sync(0xffffffffu, b);
+                if (rr == nrx) E = e;
+                if (tid == 0) xexp[rr] = e, bad[rr] = b;
+            }
+#pragma unroll
+            for (int e = 0; e < 3; ++e)
+                sh[e] = max(kBits - E + FxScale(kin[nrx * 12 + t + 4 * e], TF).ex - (t ? 2 : 0), -63);
+            unsigned key = 0;
+            for (int q = wid; q < nq; q += NW) {
+                const int col = q >= NO, ko = q - (col ? NO : 0);
+                const bool self = ko == 0 || ko == LZ / 2;
+                // digits of B: rows ra + 4 p, inputs t + 4 q
+                unsigned a[3][3][kD];
+                cp_async_wait<0>();
+                __syncwarp();
+#pragma unroll
+                for (int p = 0; p < 3; ++p)
+#pragma unroll
+                    for (int e = 0; e < 3; ++e) {
+                        const bool zero = KOP && p == e;
+                        const int tens = (KOP ? 10 * (3 - p - e) : 10 * pq_index(p, e)) + ll;
+                        const unsigned neg = bneg ^ (KOP && kblock::levi_civita(p, 3 - p - e, e) > 0 ? 0x80008000u : 0u);
+const uint4 g = zero ? make_uint4(0, 0, 0, 0) : gbuf[tens * 2];
+                        const uint4 f = zero ? make_uint4(0, 0, 0, 0) : gbuf[tens * 2 + 1];
+                        const unsigned v[kD] = {g.x, g.y, g.z, g.w, f.x, f.y, f.z};
+#pragma unroll
+                        for (int d = 0; d < kD; ++d) a[p][e][d] = zero ? 0u : __byte_perm(v[d], 0, bsel) ^ neg;
+                    }
+                __syncwarp();
+                fetch(q + NW < nq ? q + NW : wid);  // after the last one, the next group's first
+                // digits of X: components t + 4 e of point n
+                unsigned b[3][kD];
+                {
+                    const bool v = nval && !(nneg && self) && !(single && ncol != col);
+                    const int kz = nneg && ko ? LZ - ko : ko;
+                    const unsigned m = fy ^ (ncol ? fx1 : fx0) ^ (nneg ? z.mz : 0u);
+                    const fx2* p = s + (nrx * 12 + t) * GS + 2 * pos_of(LZ, kz) + ncol;
+#pragma unroll
+                    for (int e = 0; e < 3; ++e) {
+                        const fx2 x = v ? p[4 * e * GS] : fx2{0, 0};
+                        const __half2 sg = __float2half2_rn(((m >> (t + 4 * e)) & 1u) ? -1.f : 1.f);
+                        split_digits(x, sh[e], sg, b[e]);
+                    }
+                }
+                long long y[6];
+                block_digits(a, b, y);
+                __syncwarp();
+                // outputs: components ra + 4 p, re or im, points 2t (column 0) and 2t + 1 (column 1)
+                {
+                    const int kz = qcol && ko ? LZ - ko : ko;
+                    const bool rz = qcol;
+                    if (oval && !(qcol && self)) {
+                        long long* p = reinterpret_cast<long long*>(s + ((RB == 1 ? 0 : rout) * 12 + ra) * GS + 2 * pos_of(LZ, kz)) + part;
+#pragma unroll
+                        for (int c = 0; c < 2; ++c) {
+                            if (single && c != col) continue;
+                            unsigned m = fy ^ (c ? fx1 : fx0) ^ (rz ? z.mz : 0u);
+                            if (KOP && (ry ^ rz ^ ((c ? fx1 : fx0) != 0))) m ^= 0xFFFu;
+#pragma unroll
+                            for (int e = 0; e < 3; ++e) {
+                                long long v = y[2 * e + c];
+                                if ((m >> (ra + 4 * e)) & 1u) v = -v;
+                                key |= fx_key(v);
+                                p[8 * e * GS + 2 * c] = v;
+                            }
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+            // a lane's outputs belong to one right-hand side
+#pragma unroll
+            for (int rr = 0; rr < RB; ++rr) {
+                const unsigned m = __reduce_or_sync(0xffffffffu, RB == 1 || rout == rr ? key : 0u);
+                if (lane == 0) atomicOr(kout + rr, m);
+            }
+        }
+        __syncthreads();
+        // inverse z transform, rescaled before each pass
+        {
+            unsigned key[RB] = {};
+            for (int w = tid; w < NL * A; w += NT) {
+                const int ln = w % NL, k1 = w / NL, rr = ln / 24;
+                if (RB > 1 && rr >= nr) continue;
+                const int k = max(fx_bits(kout[rr]) - TI1, 0);
+                fx2* p = s + (ln >> 1) * GS + (ln & 1) + 2 * B * k1;
+                fx2 v[B];
+#pragma unroll
+                for (int k2 = 0; k2 < B; ++k2) v[k2] = fx_shift(p[2 * k2], k);
+                fft2::DFT<B, fx2>::run(v, +1);
+#pragma unroll
+                for (int b = 1; b < B; ++b)
+                    if (k1) v[b] = cmul(v[b], fx_conj(tw[b * k1]));
+                unsigned m = 0;
+#pragma unroll
+                for (int b = 0; b < B; ++b) {
+                    p[2 * b] = v[b];
+                    m |= fx_key(v[b]);
+                }
+#pragma unroll
+                for (int u = 0; u < RB; ++u) key[u] |= rr == u ? m : 0u;
+            }
+#pragma unroll
+            for (int rr = 0; rr < RB; ++rr) {
+                const unsigned m = __reduce_or_sync(0xffffffffu, key[rr]);
+                if (lane == 0) atomicOr(kmid + rr, m);
+            }
+        }
+        __syncthreads();
+        for (int w = tid; w < NL * B; w += NT) {
+            const int ln = w % NL, b = w / NL, rr = ln / 24;
+            if (RB > 1 && rr >= nr) continue;
+            const fx2* p = s + (ln >> 1) * GS + (ln & 1);
+            const int k = max(fx_bits(kmid[rr]) - TI2, 0);
+            fx2 v[A];
+#pragma unroll
+            for (int k1 = 0; k1 < A; ++k1) v[k1] = fx_shift(p[2 * (b + B * k1)], k);
+            fft2::dft_half_out<A>(v, +1);
+            // exponent of the result: that of X, of Y, of B and of the two shifts
+            const int comp = (ln % 24) >> 1, c = ln & 1;
+            const int ex = xexp[rr] - kBits + kShift - (c ? gex1 : gex0) + max(fx_bits(kout[rr]) - TI1, 0) + k -
+                           (comp % 4 ? 2 : 0);
+            double2* out = z.w + (long long)(r0 + rr) * 12 * nz * plane + (long long)py * z.Lx + sc0 + c;
+#pragma unroll
+            for (int a = 0; a < A / 2; ++a) {
+                const int l = b + B * a;
+                if (l < nz) {
+                    double2 o = fx_double(v[a], ex);
+                    if (bad[rr]) o.x = o.y = __longlong_as_double(0x7ff8000000000000ll);  // it reaches every output
+                    out[((long long)comp * nz + l) * plane] = o;
+                }
+            }
+        }
+        __syncthreads();
+        if (tid < 26 * RB) kin[tid] = 0;
+        __syncthreads();
+    }
+    cp_async_wait<0>();
+}
+
+// Digit tables from the octant values [Oy][Ox][Oz][NG] of one column (ky, kx) per block: the column's
+// exponent (|B 2^gexp| < 2^62 with the linear functions' rows and columns raised by 4, which brings
+// to the size of the constant ones: their Gram entries are 1/12) and seven signed 9-bit digits per value.
+__global__ void __launch_bounds__(128) digits_kernel(const double2* __restrict__ g, int Oz, int NG,
+                                                     uint4* __restrict__ d, int* __restrict__ gexp) {
+    __shared__ unsigned key;
+    const long long n = (long long)Oz * NG, o = blockIdx.x * n;
+    if (threadIdx.x == 0) key = 0;
+    __syncthreads();
+    unsigned m = 0;
+    for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+        const int ll = (int)(i % NG) % 10;  // pairs (1,1), (1,l') and (l,l'): raised by 1, 4 and 16
+        const double f = ll == 0 ? 1.0 : (ll < 4 ? 4.0 : 16.0);
+        const double2 v = g[o + i];
+        m = max(m, fx_key(make_double2(f * v.x, f * v.y)));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(&key, m);
+    __syncthreads();
+    const int sb = key ? kBits + 1022 - (int)(key >> 20) : 0;
+    if (threadIdx.x == 0) gexp[blockIdx.x] = sb;
+    for (long long i = threadIdx.x; i < n; i += blockDim.x) {
+        const int ll = (int)(i % NG) % 10;
+        const int up = sb + (ll == 0 ? 0 : (ll < 4 ? 2 : 4));
+        const double2 v = g[o + i];
+        unsigned long long re = (unsigned long long)__double2ll_rn(scalbn(v.x, up)) + kBias;
+        unsigned long long im = (unsigned long long)__double2ll_rn(scalbn(v.y, up)) + kBias;
+        unsigned u[8] = {};
+#pragma unroll
+        for (int q = kD - 1; q >= 0; --q) {
+            const int mask = q ? 511 : 1023;
+            const __half2 h = __halves2half2(__int2half_rn((int)(re & mask) - 256), __int2half_rn((int)(im & mask) - 256));
+            u[q] = *reinterpret_cast<const unsigned*>(&h);
+            re >>= 9;
+            im >>= 9;
+        }
+        d[2 * (o + i)] = make_uint4(u[0], u[1], u[2], u[3]);
+        d[2 * (o + i) + 1] = make_uint4(u[4], u[5], u[6], 0);
     }
 }
 
@@ -173,10 +519,10 @@ int launch_zd_L(const vie_handle* h, const ZDArgs& z, cudaStream_t s) {
     constexpr double NG = KOP ? 30.0 : 60.0;
     // set on every call: the attribute is per device and launches may come from several threads
     VIE_CUDA(cudaFuncSetAttribute(zfused64_kernel<LZ, KOP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const long long blocks = (long long)z.Ly * (z.Lx / ZDCfg<LZ>::TB);
+    const long long blocks = (long long)z.Ly * (z.Lx / 2);
     const double bytes = z.nact ? kDevCounted : 16.0 * (2.0 * z.R * 12 * z.nz * z.Ly * z.Lx + NG * z.Ox * z.Oy * z.Oz);
     VIE_KLAUNCH_B(KOP ? "zpass_block_k_f64" : "zpass_block_f64", s, bytes,
-                  zfused64_kernel<LZ, KOP><<<(unsigned)blocks, ZDCfg<LZ>::NT, smem, s>>>(z, h->tw64 + LZ));
+                  zfused64_kernel<LZ, KOP><<<(unsigned)blocks, ZDCfg<LZ>::NT, smem, s>>>(z, h->twfx + LZ));
     VIE_CHECK_LAUNCH();
     return VIE_OK;
 }
@@ -197,6 +543,13 @@ int launch_zd(const vie_handle* h, const ZDArgs& z, cudaStream_t s) {
 }
 
 }  // namespace
+
+int green_digits(const vie_handle* h, const double2* g, int ng, uint4* d, int* gexp, cudaStream_t s) {
+    VIE_KLAUNCH("green_digits", s,
+                digits_kernel<<<(unsigned)(h->O[0] * h->O[1]), 128, 0, s>>>(g, h->O[2], ng, d, gexp));
+    VIE_CHECK_LAUNCH();
+    return VIE_OK;
+}
 
 int zpass_f64_fused(const vie_handle* h, const ZDArgs& z, cudaStream_t s) { return launch_zd<false>(h, z, s); }
 

@@ -5,7 +5,8 @@
 
 struct ZDArgs {
     double2* w;                // spectrum [R*12][Nz][Ly][Lx], in place
-    const double2* green_t;    // [Oy][Ox][Oz][60] (N), [Oy][Ox][Oz][30] (K)
+    const uint4* green_d;      // digits of the block's tensors (green_digits): [Oy][Ox][Oz][60 (N) or 30 (K)][2]
+    const int* gexp;           // [Oy][Ox] their exponents
     const int* colkx;          // [Lx] kx of each stored column (mirror pairs)
     int R, nz, Lx, Ly, Ox, Oy, Oz;
     int ay, by;                // row py holds ky = py / by + ay * (py % by)
@@ -14,6 +15,8 @@ struct ZDArgs {
     unsigned long long* bctr;
 };
 
+// Digit tables of the octant values g [Oy][Ox][Oz][ng] (device): d [Oy][Ox][Oz][ng][2], gexp [Oy][Ox].
+int green_digits(const vie_handle* h, const double2* g, int ng, uint4* d, int* gexp, cudaStream_t s);
 // Launches the FP64 z pass (Lz in 8..512, Lx >= 4).
 int zpass_f64_fused(const vie_handle* h, const ZDArgs& z, cudaStream_t s);
 // The same z pass with the K block (VIE_OP_K) on the K octant [Oy][Ox][Oz][30].

@@ -1,0 +1,131 @@
+"""The FP64 matvec's scaled-integer transforms and split block product at every compiled FFT length, on inputs of
+very different sizes, against NumPy's FP64 FFTs with a random Toeplitz table of the right parities.
+
+Tolerance per right-hand side (relative 2-norm): 5e-15.  NumPy's three transforms each way and the 24-term sums
+are good for about 1e-15 at these lengths; the kernels round at 2^-56 of the largest value, with the spectrum
+stored in FP64 twice.
+"""
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+TOL = 5e-15
+
+
+@pytest.fixture(scope="module")
+def vie():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1902_02196_gb300 as v
+
+    v.build()
+    return v
+
+
+def parity(a, i):
+    return (-1 if a // 4 == i else 1) * (-1 if a % 4 == i + 1 else 1)
+
+
+def make(vie, shape, seed):
+    """(handle on random tensors, the 144 circulant spectra by entry and sign) of an nx x ny x nz grid."""
+    nx, ny, nz = shape
+    rng = np.random.default_rng(seed)
+    table = np.zeros((144, 2 * nz - 1, 2 * ny - 1, 2 * nx - 1), dtype=np.complex128)
+    spectra = {}
+    dec = 1.0 / (1 + np.add.outer(np.add.outer(np.arange(nz), np.arange(ny)), np.arange(nx)))  # decays as the entries do
+    for p in range(3):
+        for q in range(p, 3):
+            for l in range(4):
+                for m in range(l, 4):
+                    a, b = 4 * p + l, 4 * q + m
+                    size = 12.0 ** (-0.5 * ((l > 0) + (m > 0)))  # of the Gram entries' square roots
+                    t = size * dec * (rng.standard_normal((nz, ny, nx)) + 1j * rng.standard_normal((nz, ny, nx)))
+                    circ = np.zeros((2 * nz, 2 * ny, 2 * nx), dtype=np.complex128)
+                    for axis, i in ((2, 0), (1, 1), (0, 2)):  # an odd tensor vanishes at offset 0 of its axis
+                        if parity(a, i) * parity(b, i) < 0:
+                            t[(slice(None),) * axis + (0,)] = 0
+                    circ[:nz, :ny, :nx] = t
+                    for axis, i, n in ((2, 0, nx), (1, 1, ny), (0, 2, nz)):
+                        s = parity(a, i) * parity(b, i)
+                        src = np.moveaxis(circ, axis, 0)
+                        for d in range(1, n):
+                            src[2 * n - d] = s * src[d]
+                    table[12 * a + b, nz - 1:, ny - 1:, nx - 1:] = t
+                    if a == b:  # the library keeps N - G
+                        table[12 * a + b, nz - 1, ny - 1, nx - 1] += 1.0 if l == 0 else 1 / 12
+                    hat = np.fft.fftn(circ)
+                    swap = -1.0 if (l > 0) != (m > 0) else 1.0
+                    for u, v in {(p, q), (q, p)}:
+                        spectra[4 * u + l, 4 * v + m] = (hat, 1.0)
+                        if l != m:
+                            spectra[4 * u + m, 4 * v + l] = (hat, swap)
+    eps = np.full((nz, ny, nx), 3.0)
+    h = vie.vie_setup_green_external((nx, ny, nz, 1.0, 1.0, 1.0), 3e6, eps, 0 * eps, table)
+    return h, spectra
+
+
+def reference(spectra, shape, x):
+    nx, ny, nz = shape
+    hat = [np.fft.fftn(x[b], s=(2 * nz, 2 * ny, 2 * nx), axes=(0, 1, 2)) for b in range(12)]
+    out = np.empty_like(x)
+    for a in range(12):
+        acc = sum(spectra[a, b][1] * spectra[a, b][0] * hat[b] for b in range(12))
+        out[a] = np.fft.ifftn(acc)[:nz, :ny, :nx]
+    return out
+
+
+def apply(vie, h, x):
+    xd = torch.from_numpy(x).cuda()
+    yd = torch.empty_like(xd)
+    vie.vie_matvec(h, xd, yd, vie.VIE_FP64, vie.VIE_OP_NSCAT)
+    torch.cuda.synchronize()
+    return yd.cpu().numpy()
+
+
+# FFT lengths (x, y, z): (8, 8, 8), (16, 16, 16), (32, 32, 32), (64, 64, 64), (128, 128, 8), (8, 8, 128), (8, 8, 256),
+# (8, 8, 512), and the line transforms with (8, 16, 64) and (256, 8, 16)
+@pytest.mark.parametrize("shape", [(4, 3, 4), (8, 7, 5), (13, 16, 9), (20, 17, 32), (33, 40, 3), (4, 4, 40), (3, 4, 100),
+                                   (4, 3, 200), (3, 7, 20), (70, 3, 5)])
+def test_sizes_and_scales(vie, shape):
+    nx, ny, nz = shape
+    h, spectra = make(vie, shape, seed=nx + 10 * ny + 100 * nz)
+    rng = np.random.default_rng(5)
+    x = rng.standard_normal((6, 12, nz, ny, nx)) + 1j * rng.standard_normal((6, 12, nz, ny, nx))
+    x[1] *= 1e-295  # close to the smallest normal numbers
+    x[2] = 0
+    x[2, 7, nz // 2, ny - 1, 0] = 3e200 - 1e200j  # one large value
+    x[3] *= 1e-9 ** rng.random((12, 1, 1, 1))  # components of different sizes
+    x[4, :, :, :, 1:] *= 1e-12  # one column above the rest
+    x[5] = x[5].astype(np.complex64)  # short mantissas: low words of the fixed-point values at their ends
+    y = apply(vie, h, x)
+    for r in range(6):
+        s = 10.0 ** -np.round(np.log10(np.max(np.abs(x[r]))))  # the reference at ordinary sizes
+        ref = reference(spectra, shape, x[r] * s)
+        err = np.linalg.norm(y[r] * s - ref) / np.linalg.norm(ref)
+        assert err <= TOL, (r, err)
+    # a right-hand side does not depend on its neighbours, of any size
+    assert np.array_equal(apply(vie, h, x[3:4])[0], y[3])
+    h.close()
+
+
+@pytest.mark.parametrize("shape", [(5, 6, 7), (3, 7, 20)])
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_not_finite(vie, shape, value):
+    """A NaN or an Inf leaves no finite value in its right-hand side, as every output depends on every input, and
+    the others as they are; zero stays zero."""
+    nx, ny, nz = shape
+    h, _ = make(vie, shape, seed=3)
+    rng = np.random.default_rng(6)
+    x = rng.standard_normal((3, 12, nz, ny, nx)) + 1j * rng.standard_normal((3, 12, nz, ny, nx))
+    x[1] = 0
+    clean = apply(vie, h, x)
+    assert np.all(clean[1] == 0)
+    x[0, 4, 1, 2, 1] = value
+    y = apply(vie, h, x)
+    assert not np.any(np.isfinite(y[0]))
+    assert np.array_equal(y[1:], clean[1:])
+    h.close()
