@@ -33,6 +33,15 @@ constexpr BlockTable make_block_table() {
 __device__ constexpr BlockTable kBlock = make_block_table();
 static_assert(make_block_table().start[60] == 144, "every block entry maps to one of the 60 tensors");
 
+// tensors t whose reflection parity under x_i -> -x_i (that of any of their entries) is -1, as a bit mask
+constexpr unsigned long long odd_tensors(int i) {
+    const BlockTable T = make_block_table();
+    unsigned long long m = 0;
+    for (int n = 0; n < 144; ++n)
+        if (parity_of(T.e[n].a, i) * parity_of(T.e[n].b, i) < 0) m |= 1ull << tensor_of(T.e[n].a, T.e[n].b);
+    return m;
+}
+
 // The same 144 entries ordered by input component b, then output a: consecutive
 // multiply-adds go to different accumulators, so each accumulator's chain of dependent
 // FMAs is interleaved with the other rows' (FMA latency hidden within one thread).
@@ -82,6 +91,15 @@ constexpr KBlockTable make_kblock_table() {
 }
 __device__ constexpr KBlockTable kKBlock = make_kblock_table();
 static_assert(make_kblock_table().start[30] == 96, "the K block has 96 non-zero entries from 30 tensors");
+
+// as odd_tensors for the K tensors
+constexpr unsigned long long odd_ktensors(int i) {
+    unsigned long long m = 0;
+    for (int a = 0; a < 12; ++a)
+        for (int b = 0; b < 12; ++b)
+            if (kblock::tensor(a, b) >= 0 && kblock::reflection(a, b, i) < 0) m |= 1ull << kblock::tensor(a, b);
+    return m;
+}
 
 // The 96 non-zero K entries ordered by input component b, then output a (as kBlockB)
 struct KBlockTableB {
