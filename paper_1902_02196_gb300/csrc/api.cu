@@ -107,13 +107,11 @@ void release(vie_handle* h) {
         cudaFree(h->green32);
         cudaFree(h->green32t);
         cudaFree(h->green_d);
-        cudaFree(h->green_e);
         cudaFree(h->greenbf);
         cudaFree(h->colmap);
         cudaFree(h->colkx32);
         cudaFree(h->tw64);
         cudaFree(h->tw32);
-        cudaFree(h->twfx);
         cudaFree(h->toeplitz);
     }
     cudaFree(h->tucker);
@@ -325,7 +323,6 @@ int handle_create(const vie_grid* grid, double freq_hz, const double* eps_real, 
         h->green32 = share->green32;
         h->green32t = share->green32t;
         h->green_d = share->green_d;
-        h->green_e = share->green_e;
         h->greenbf = share->greenbf;
         h->colmap = share->colmap;
         h->colkx32 = share->colkx32;

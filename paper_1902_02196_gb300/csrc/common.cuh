@@ -118,10 +118,9 @@ struct vie_handle {
     // FP32 copy in the layout of the z pass of the FP32 three-kernel path: [Oy][Ox][Oz][60]
     float2* green32t;
     // the FP64 values' digits for the FP64 fused z pass (zpass_f64.cu): per octant point and tensor seven
-    // 9-bit digits as fp16 (re, im) pairs, [Oy][Ox][Oz][60][2], and the exponent of each column [Oy][Ox]
+    // 9-bit digits as fp16 (re, im) pairs, [Oy][Ox][Oz][60][2], then the exponent of each column [Oy][Ox]
     // (PWL handles with an FFT length along z of 8..512, else null)
     uint4* green_d;
-    int* green_e;
     // the 30 K tensors' transformed circulants, octant storage [30][Oz][Oy][Ox], scaled by
     // 1/(Lx Ly Lz), FP64 and FP32 (kmatvec.cu, built on the first K product)
     double2* kgreen64;
@@ -130,7 +129,6 @@ struct vie_handle {
     float2* kgreen32t;
     // and their digits for the FP64 one, as green_d
     uint4* kgreen_d;
-    int* kgreen_e;
     // bf16 split of green32t in the same layout, for the BF16x3 z pass: per tensor (hi, lo),
     // each a bf16 (re, im) pair with hi = bf16(v), lo = bf16(v - hi)
     uint2* greenbf;
@@ -145,7 +143,7 @@ struct vie_handle {
     // twiddle tables exp(-2 pi i m / L) for L = 2^k, k = 1..11, concatenated at offset L
     double2* tw64;
     float2* tw32;
-    int4* twfx;  // the same as fixed-point factors (fixed.cuh): (hi, lo) of the cosine, then of the sine
+    int4* twfx;  // the same as fixed-point factors (fixed.cuh): (hi, lo) of the cosine, then of the sine; behind tw64
     // scratch
     Workspace fft_ws;    // matvec spectrum buffers
     Workspace stage_ws;  // host-buffer staging

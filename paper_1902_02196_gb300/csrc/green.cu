@@ -540,8 +540,7 @@ __global__ void embed_kernel(const double2* __restrict__ T, int nx, int ny, int 
 
 // Octant k_i in [0, L_i/2] of the transformed circulants, scaled, into FP64 and FP32 tables [60][Oz][Oy][Ox].
 __global__ void octant_kernel(const double2* __restrict__ C, int Lx, int Ly, int Lz, int t0, int nt, double scale,
-                              double2* __restrict__ g64, float2* __restrict__ g32, float2* __restrict__ g32t,
-                              double2* __restrict__ g64t) {
+                              double2* __restrict__ g64, float2* __restrict__ g32, float2* __restrict__ g32t) {
     const int Ox = Lx / 2 + 1, Oy = Ly / 2 + 1, Oz = Lz / 2 + 1;
     const long long ovol = (long long)Ox * Oy * Oz;
     long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -557,7 +556,6 @@ __global__ void octant_kernel(const double2* __restrict__ C, int Lx, int Ly, int
     g32[dst] = make_float2((float)v.x, (float)v.y);
     const long long tdst = (((long long)ky * Ox + kx) * Oz + kz) * 60 + t0 + tl;
     g32t[tdst] = make_float2((float)v.x, (float)v.y);
-    if (g64t) g64t[tdst] = v;
 }
 
 // Gauss-Legendre tables of the cell-moment kernels in constant memory (current device)
@@ -633,12 +631,11 @@ int green_setup(vie_handle* h) {
 int green_embed(vie_handle* h, double2* T, bool keep_table) {
     cudaStream_t s = h->stream;
     const long long nd = (long long)h->nx * h->ny * h->nz;
-    double2 *C = nullptr, *g64t = nullptr;  // g64t: the octants as [Oy][Ox][Oz][60], for the digit tables
-    const bool digits = green_digit_bytes(h, 60) > 0;
+    double2* C = nullptr;
+    const size_t digit_bytes = green_digit_bytes(h, 60);
     auto fail = [&](int code) {
         cudaFree(T);
         cudaFree(C);
-        cudaFree(g64t);
         return code;
     };
     int rc = VIE_OK;
@@ -650,13 +647,10 @@ int green_embed(vie_handle* h, double2* T, bool keep_table) {
             cudaMalloc(&h->green32, sizeof(float2) * 60 * ovol) != cudaSuccess ||
             cudaMalloc(&h->green32t, sizeof(float2) * 60 * ovol) != cudaSuccess ||
             cudaMalloc(&h->greenbf, sizeof(uint2) * 60 * ovol) != cudaSuccess ||
-            (digits && (cudaMalloc(&h->green_d, 2 * sizeof(uint4) * 60 * ovol) != cudaSuccess ||
-                        cudaMalloc(&h->green_e, sizeof(int) * h->O[0] * h->O[1]) != cudaSuccess)))
+            (digit_bytes && cudaMalloc(&h->green_d, digit_bytes) != cudaSuccess))
             return fail((set_error("green alloc"), VIE_ENOMEM));
-        h->bytes_held += (sizeof(double2) + 2 * sizeof(float2) + sizeof(uint2)) * 60 * ovol + green_digit_bytes(h, 60);
+        h->bytes_held += (sizeof(double2) + 2 * sizeof(float2) + sizeof(uint2)) * 60 * ovol + digit_bytes;
     }
-    if (digits && cudaMalloc(&g64t, sizeof(double2) * 60 * ovol) != cudaSuccess)
-        return fail((set_error("green digits alloc"), VIE_ENOMEM));
     int chunk = (int)std::max<long long>(1, std::min<long long>(60, (4LL << 30) / (vol * (long long)sizeof(double2))));
     if (cudaMalloc(&C, sizeof(double2) * vol * chunk) != cudaSuccess) return fail((set_error("embed alloc"), VIE_ENOMEM));
     for (int t0 = 0; t0 < 60; t0 += chunk) {
@@ -668,16 +662,14 @@ int green_embed(vie_handle* h, double2* T, bool keep_table) {
         if (rc < 0) return fail(rc);
         long long tho = ovol * nt;
         VIE_KLAUNCH("octant", s, octant_kernel<<<(unsigned)((tho + 255) / 256), 256, 0, s>>>(C, Lx, Ly, Lz, t0, nt, 1.0 / (double)vol,
-                                                                     h->green64, h->green32, h->green32t,
-                                                                     g64t));
+                                                                     h->green64, h->green32, h->green32t));
         if (cudaGetLastError() != cudaSuccess) return fail((set_error("octant launch"), VIE_EDEVICE));
     }
     rc = green_split_bf16(h);
-    if (rc == VIE_OK && digits) rc = green_digits(h, g64t, 60, h->green_d, h->green_e, s);
+    if (rc == VIE_OK && digit_bytes) rc = green_digits(h, h->green64, 60, h->green_d, s);
     if (rc < 0) return fail(rc);
     if (cudaStreamSynchronize(s) != cudaSuccess) return fail((set_error("green setup sync"), VIE_EDEVICE));
     cudaFree(C);
-    cudaFree(g64t);
     if (!keep_table) {
         cudaFree(T);
         return VIE_OK;

@@ -7,8 +7,8 @@
 // The 30 Toeplitz tensors P_t (green.cu, assemble_k_kernel) are embedded into full 2N
 // circulants, the entries at negative offsets taken from the reflection parities of the block
 // table (kblock.h), transformed, and their octant k_i in [0, L_i/2] kept, scaled by
-// 1/(Lx Ly Lz), as [30][Oz][Oy][Ox] in FP64 and FP32, and once more in both as [Oy][Ox][Oz][30]
-// (the 30 values of a point side by side, for the fused z passes).  The other octants follow
+// 1/(Lx Ly Lz), as [30][Oz][Oy][Ox] in FP64 and FP32, and once more as [Oy][Ox][Oz][30] (the 30
+// values of a point side by side, for the fused z passes), in FP32 and as FP64 digits.  The other octants follow
 // in the z pass from the same parities: K(R_i k) = -S_i K(k) S_i.  Built on the first K product
 // of a handle and released with it.
 #include <algorithm>
@@ -59,8 +59,7 @@ __global__ void embed_k_kernel(const double2* __restrict__ P, int nx, int ny, in
 
 // octant k_i in [0, L_i/2] of the transformed circulants of tensors t0 .. t0 + nt - 1, scaled
 __global__ void k_octant_kernel(const double2* __restrict__ C, int Lx, int Ly, int Lz, int t0, int nt, double scale,
-                                double2* __restrict__ g64, float2* __restrict__ g32, float2* __restrict__ g32t,
-                                double2* __restrict__ g64t) {
+                                double2* __restrict__ g64, float2* __restrict__ g32, float2* __restrict__ g32t) {
     const int Ox = Lx / 2 + 1, Oy = Ly / 2 + 1, Oz = Lz / 2 + 1;
     const long long ovol = (long long)Ox * Oy * Oz;
     const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -76,7 +75,6 @@ __global__ void k_octant_kernel(const double2* __restrict__ C, int Lx, int Ly, i
     g32[dst] = make_float2((float)v.x, (float)v.y);
     const long long dt = (((long long)ky * Ox + kx) * Oz + kz) * 30 + t0 + tl;
     g32t[dt] = make_float2((float)v.x, (float)v.y);
-    if (g64t) g64t[dt] = v;
 }
 
 // device bytes of a handle's K spectra
@@ -96,10 +94,9 @@ int k_octants(vie_handle* h, cudaStream_t s) {
     const long long vol = (long long)Lx * Ly * Lz, nd = (long long)h->nv;
     const long long ovol = (long long)h->O[0] * h->O[1] * h->O[2];
     const int chunk = (int)std::max<long long>(1, std::min<long long>(30, (4LL << 30) / (vol * (long long)sizeof(double2))));
-    double2 *P = nullptr, *C = nullptr, *g64 = nullptr, *g64t = nullptr;
+    double2 *P = nullptr, *C = nullptr, *g64 = nullptr;
     uint4* gd = nullptr;
-    int* ge = nullptr;
-    const bool digits = green_digit_bytes(h, 30) > 0;
+    const size_t digit_bytes = green_digit_bytes(h, 30);
     float2 *g32 = nullptr, *g32t = nullptr;
     auto fail = [&](int code, const char* msg) {
         cudaGetLastError();
@@ -108,9 +105,7 @@ int k_octants(vie_handle* h, cudaStream_t s) {
         cudaFree(g64);
         cudaFree(g32);
         cudaFree(g32t);
-        cudaFree(g64t);
         cudaFree(gd);
-        cudaFree(ge);
         set_error(msg);
         return code;
     };
@@ -119,9 +114,7 @@ int k_octants(vie_handle* h, cudaStream_t s) {
         cudaMalloc(&g64, sizeof(double2) * 30 * ovol) != cudaSuccess ||
         cudaMalloc(&g32, sizeof(float2) * 30 * ovol) != cudaSuccess ||
         cudaMalloc(&g32t, sizeof(float2) * 30 * ovol) != cudaSuccess ||
-        (digits && (cudaMalloc(&g64t, sizeof(double2) * 30 * ovol) != cudaSuccess ||
-                    cudaMalloc(&gd, 2 * sizeof(uint4) * 30 * ovol) != cudaSuccess ||
-                    cudaMalloc(&ge, sizeof(int) * h->O[0] * h->O[1]) != cudaSuccess)))
+        (digit_bytes && cudaMalloc(&gd, digit_bytes) != cudaSuccess))
         return fail(VIE_ENOMEM, "K spectrum allocation failed");
     int rc = green_k_toeplitz(h, P, s);
     for (int t0 = 0; rc == VIE_OK && t0 < 30; t0 += chunk) {
@@ -133,10 +126,10 @@ int k_octants(vie_handle* h, cudaStream_t s) {
         if (rc < 0) break;
         VIE_KLAUNCH("k_octant", s,
                     k_octant_kernel<<<blocks(ovol * nt), 256, 0, s>>>(C, Lx, Ly, Lz, t0, nt, 1.0 / (double)vol, g64,
-                                                                      g32, g32t, g64t));
+                                                                      g32, g32t));
         if (cudaGetLastError() != cudaSuccess) return fail(VIE_EDEVICE, "K octant launch failed");
     }
-    if (rc == VIE_OK && digits) rc = green_digits(h, g64t, 30, gd, ge, s);
+    if (rc == VIE_OK && digit_bytes) rc = green_digits(h, g64, 30, gd, s);
     if (rc == VIE_OK && cudaStreamSynchronize(s) != cudaSuccess) return fail(VIE_EDEVICE, "K spectrum sync failed");
     if (rc < 0) {
         cudaFree(P);
@@ -144,19 +137,15 @@ int k_octants(vie_handle* h, cudaStream_t s) {
         cudaFree(g64);
         cudaFree(g32);
         cudaFree(g32t);
-        cudaFree(g64t);
         cudaFree(gd);
-        cudaFree(ge);
         return rc;
     }
     cudaFree(P);
     cudaFree(C);
-    cudaFree(g64t);
     h->kgreen64 = g64;
     h->kgreen32 = g32;
     h->kgreen32t = g32t;
     h->kgreen_d = gd;
-    h->kgreen_e = ge;
     h->bytes_held += k_bytes(h);  // until kmatvec_release
     return VIE_OK;
 }
@@ -173,11 +162,9 @@ void kmatvec_release(vie_handle* h) {
     cudaFree(h->kgreen32);
     cudaFree(h->kgreen32t);
     cudaFree(h->kgreen_d);
-    cudaFree(h->kgreen_e);
     h->kgreen64 = nullptr;
     h->kgreen32 = nullptr;
     h->kgreen32t = nullptr;
     h->kgreen_d = nullptr;
-    h->kgreen_e = nullptr;
     h->bytes_held -= k_bytes(h);
 }

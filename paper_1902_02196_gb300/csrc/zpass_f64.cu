@@ -472,33 +472,49 @@ const uint4 g = zero ? make_uint4(0, 0, 0, 0) : gbuf[tens * 2];
     cp_async_wait<0>();
 }
 
-// Digit tables from the octant values [Oy][Ox][Oz][NG] of one column (ky, kx) per block: the column's
-// exponent (|B 2^gexp| < 2^62 with the linear functions' rows and columns raised by 4, which brings
-// to the size of the constant ones: their Gram entries are 1/12) and seven signed 9-bit digits per value.
-__global__ void __launch_bounds__(128) digits_kernel(const double2* __restrict__ g, int Oz, int NG,
+// Digit tables from the octant spectra g [NG][Oz][Oy][Ox]: per column (ky, kx) the exponent of its
+// values (|B 2^gexp| < 2^62 with the linear functions' rows and columns raised by 4, which brings them to
+// the size of the constant ones: their Gram entries are 1/12) and seven signed 9-bit digits per value.
+// A block takes kDigitCols neighbouring columns, whose values of one (tensor, kz) are 128 contiguous bytes, and reads
+// them twice; the digits of a value are 32 contiguous bytes.
+constexpr int kDigitCols = 8;
+__global__ void __launch_bounds__(256) digits_kernel(const double2* __restrict__ g, int Ox, int Oy, int Oz, int NG,
                                                      uint4* __restrict__ d, int* __restrict__ gexp) {
-    __shared__ unsigned key;
-    const long long n = (long long)Oz * NG, o = blockIdx.x * n;
-    if (threadIdx.x == 0) key = 0;
+    __shared__ unsigned key[kDigitCols];
+    const int c = threadIdx.x % kDigitCols, kx = blockIdx.x * kDigitCols + c, ky = blockIdx.y;
+    if (threadIdx.x < kDigitCols) key[threadIdx.x] = 0;
     __syncthreads();
-    unsigned m = 0;
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) {
-        const int ll = (int)(i % NG) % 10;  // pairs (1,1), (1,l') and (l,l'): raised by 1, 4 and 16
-        const double f = ll == 0 ? 1.0 : (ll < 4 ? 4.0 : 16.0);
-        const double2 v = g[o + i];
-        m = max(m, fx_key(make_double2(f * v.x, f * v.y)));
+    const int n = NG * Oz;
+    auto raise = [&](int t) {  // pairs (1,1), (1,l') and (l,l'): by 2^0, 2^2 and 2^4
+        const int ll = t % 10;
+        return ll == 0 ? 0 : (ll < 4 ? 2 : 4);
+    };
+    if (kx < Ox) {
+        unsigned m = 0;
+        for (int i = threadIdx.x / kDigitCols; i < n; i += 256 / kDigitCols) {
+            const double2 v = g[((long long)i * Oy + ky) * Ox + kx];
+            const unsigned k = fx_key(v);
+            m = max(m, k >= 0x00100000u ? k + (raise(i / Oz) << 20) : 0u);
+        }
+        atomicMax(key + c, m);
     }
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) atomicMax(&key, m);
     __syncthreads();
-    const int sb = key ? kBits + 1022 - (int)(key >> 20) : 0;
-    if (threadIdx.x == 0) gexp[blockIdx.x] = sb;
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) {
-        const int ll = (int)(i % NG) % 10;
-        const int up = sb + (ll == 0 ? 0 : (ll < 4 ? 2 : 4));
-        const double2 v = g[o + i];
-        unsigned long long re = (unsigned long long)__double2ll_rn(scalbn(v.x, up)) + kBias;
-        unsigned long long im = (unsigned long long)__double2ll_rn(scalbn(v.y, up)) + kBias;
+    if (kx >= Ox) return;
+    const int sb = key[c] ? kBits + 1022 - (int)(key[c] >> 20) : 0;
+    const long long col = (long long)ky * Ox + kx;
+    if (threadIdx.x < kDigitCols) gexp[col] = sb;
+    for (int i = threadIdx.x / kDigitCols; i < n; i += 256 / kDigitCols) {
+        const int t = i / Oz, kz = i - t * Oz;
+        const int up = sb + raise(t);
+        double2 v = g[((long long)i * Oy + ky) * Ox + kx];
+        if (up > 1000 || up < -1000) {
+            v = make_double2(scalbn(v.x, up), scalbn(v.y, up));
+        } else {
+            const double f = __hiloint2double((1023 + up) << 20, 0);
+            v = make_double2(f * v.x, f * v.y);
+        }
+        unsigned long long re = (unsigned long long)__double2ll_rn(v.x) + kBias;
+        unsigned long long im = (unsigned long long)__double2ll_rn(v.y) + kBias;
         unsigned u[8] = {};
 #pragma unroll
         for (int q = kD - 1; q >= 0; --q) {
@@ -508,8 +524,9 @@ __global__ void __launch_bounds__(128) digits_kernel(const double2* __restrict__
             re >>= 9;
             im >>= 9;
         }
-        d[2 * (o + i)] = make_uint4(u[0], u[1], u[2], u[3]);
-        d[2 * (o + i) + 1] = make_uint4(u[4], u[5], u[6], 0);
+        uint4* out = d + 2 * ((col * Oz + kz) * NG + t);
+        out[0] = make_uint4(u[0], u[1], u[2], u[3]);
+        out[1] = make_uint4(u[4], u[5], u[6], 0);
     }
 }
 
@@ -544,9 +561,10 @@ int launch_zd(const vie_handle* h, const ZDArgs& z, cudaStream_t s) {
 
 }  // namespace
 
-int green_digits(const vie_handle* h, const double2* g, int ng, uint4* d, int* gexp, cudaStream_t s) {
+int green_digits(const vie_handle* h, const double2* g, int ng, uint4* d, cudaStream_t s) {
+    const dim3 grid((unsigned)((h->O[0] + kDigitCols - 1) / kDigitCols), (unsigned)h->O[1]);
     VIE_KLAUNCH("green_digits", s,
-                digits_kernel<<<(unsigned)(h->O[0] * h->O[1]), 128, 0, s>>>(g, h->O[2], ng, d, gexp));
+                digits_kernel<<<grid, 256, 0, s>>>(g, h->O[0], h->O[1], h->O[2], ng, d, digit_exponents(h, ng, d)));
     VIE_CHECK_LAUNCH();
     return VIE_OK;
 }

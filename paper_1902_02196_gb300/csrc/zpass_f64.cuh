@@ -15,8 +15,12 @@ struct ZDArgs {
     unsigned long long* bctr;
 };
 
-// Digit tables of the octant values g [Oy][Ox][Oz][ng] (device): d [Oy][Ox][Oz][ng][2], gexp [Oy][Ox].
-int green_digits(const vie_handle* h, const double2* g, int ng, uint4* d, int* gexp, cudaStream_t s);
+// Digit tables of the octant spectra g [ng][Oz][Oy][Ox] (device) into d, green_digit_bytes(h, ng) bytes: the
+// digits [Oy][Ox][Oz][ng][2], then the exponents [Oy][Ox].
+int green_digits(const vie_handle* h, const double2* g, int ng, uint4* d, cudaStream_t s);
+inline int* digit_exponents(const vie_handle* h, int ng, uint4* d) {
+    return reinterpret_cast<int*>(d + 2 * (size_t)ng * h->O[0] * h->O[1] * h->O[2]);
+}
 // Launches the FP64 z pass (Lz in 8..512, Lx >= 4).
 int zpass_f64_fused(const vie_handle* h, const ZDArgs& z, cudaStream_t s);
 // The same z pass with the K block (VIE_OP_K) on the K octant [Oy][Ox][Oz][30].
