@@ -27,6 +27,7 @@
 #include "xy_f64.cuh"
 #include "zpass_f32.cuh"
 #include "zpass_f64.cuh"
+#include "zpass_pwc.cuh"
 
 int zpass_bf16_fused(const vie_handle* h, const ZFArgs& z, cudaStream_t s);  // zpass_bf16.cu
 int zpass_bf16_tune(const vie_handle* h, const ZFArgs& z, cudaStream_t s);   // zpass_bf16.cu
@@ -765,10 +766,20 @@ static int matvec_impl(vie_handle* h, int R, const void* x, void* y, int op, cud
             z.ay = ay, z.by = by;
             return launch_z<T, 12, true>(sizeof(T) == 8 ? "zpass_block_k_f64" : "zpass_block_k_f32", h, Lz, z, s);
         }
-        if (nc == 3) {  // PWC: the generic z pass with the 3 x 3 block of the l = 1 tensors
+        if (nc == 3) {  // PWC: the 3 x 3 block of the l = 1 tensors, else in the generic z pass
             if (bf16) {
                 set_error("the BF16x3 matvec is built for the PWL system only");
                 return VIE_EINVAL;
+            }
+            if (zpwc_ok(h)) {
+                ZPArgs z{};
+                z.w = W2;
+                z.green = sizeof(T) == 8 ? (const void*)h->green64 : (const void*)h->green32;
+                z.colkx = h->colkx32;
+                z.R = Rs, z.nz = nz, z.Lx = Lx, z.Ly = Ly;
+                z.Ox = h->O[0], z.Oy = h->O[1], z.Oz = h->O[2];
+                z.ay = ay, z.by = by;
+                return zpass_pwc(h, z, sizeof(T) == 8, s);
             }
             ZArgs z{};
             z.w = W2;

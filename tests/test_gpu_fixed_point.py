@@ -129,3 +129,39 @@ def test_not_finite(vie, shape, value):
     assert not np.any(np.isfinite(y[0]))
     assert np.array_equal(y[1:], clean[1:])
     h.close()
+
+
+# FFT lengths (x, y, z) of the PWC z pass: tiles of 8 columns up to 256 points, of 4 at 512, and Lx = 8 with one tile
+@pytest.mark.parametrize("shape", [(4, 4, 4), (8, 7, 7), (5, 5, 13), (9, 16, 31), (33, 35, 50), (4, 3, 70), (7, 2, 150)])
+def test_pwc_sizes_and_scales(vie, shape):
+    """The 3 x 3 block's z pass against the constant components of the 12 x 12 one on the same grid and materials, on
+    the same inputs (5e-15: both are within about 1e-15 of the exact product), and FP32 against FP64 (2e-6, some
+    tens of FP32 roundings)."""
+    nx, ny, nz = shape
+    rng = np.random.default_rng(11)
+    grid = (nx, ny, nz, 0.004, 0.005, 0.0045)
+    eps = rng.uniform(1, 80, (nz, ny, nx))
+    h12 = vie.vie_setup(grid, 298e6, eps, 0 * eps)
+    h3 = vie.vie_setup(grid, 298e6, eps, 0 * eps, vie.VIE_SETUP_PWC)
+    x3 = rng.standard_normal((4, 3, nz, ny, nx)) + 1j * rng.standard_normal((4, 3, nz, ny, nx))
+    x3[1] *= 1e-280
+    x3[2, :, nz // 2:] *= 1e-10
+    x3[3] = 0
+    x12 = np.zeros((4, 12, nz, ny, nx), dtype=np.complex128)
+    x12[:, [0, 4, 8]] = x3
+    want = apply(vie, h12, x12)[:, [0, 4, 8]]
+    got = apply(vie, h3, x3)
+    assert np.all(got[3] == 0)
+    for r in range(3):
+        s = 10.0 ** -np.round(np.log10(np.max(np.abs(x3[r]))))
+        assert np.linalg.norm((got[r] - want[r]) * s) <= TOL * np.linalg.norm(want[r] * s), r
+    xd = torch.from_numpy(x3[[0, 2]]).to("cuda", torch.complex64)
+    yd = torch.empty_like(xd)
+    vie.vie_matvec(h3, xd, yd, vie.VIE_FP32, vie.VIE_OP_NSCAT)
+    torch.cuda.synchronize()
+    assert np.linalg.norm(yd.cpu().numpy() - want[[0, 2]]) <= 2e-6 * np.linalg.norm(want[[0, 2]])
+    x3[0, 1, 0, 0, 0] = np.nan
+    bad = apply(vie, h3, x3)
+    assert not np.any(np.isfinite(bad[0])) and np.array_equal(bad[1:], got[1:])
+    h12.close()
+    h3.close()
