@@ -209,7 +209,7 @@ struct XYCfg {
     static constexpr int H = L / 2;   // rows that are non-zero before / needed after the y transform
     static constexpr int RS = L + 1;  // odd row stride of the x-transform buffer
     static constexpr int CW = L < 32 ? L : 32;  // stored columns per y-transform chunk
-    static constexpr int MINB = 2;  // CTAs per SM
+    static constexpr int MINB = L >= 128 ? 2 : 3;  // CTAs per SM (three hold the registers at 80; at 84 the 64-point kernels lost one)
     static constexpr size_t smem = sizeof(C) * (size_t)(L * CW + H * RS + L) + sizeof(int4) * H + L;
 };
 
