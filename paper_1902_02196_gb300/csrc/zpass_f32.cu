@@ -1,6 +1,8 @@
 // FP32 z pass of the matvec (Section IV-A) with the 12 x 12 Green block product fused
 // between the forward and inverse z transforms, on the spectrum left by xy_fwd_kernel: the
 // N block from its 60 tensors, or (KOP) the K block (Eq. 8, 25) from its 30.
+#include <algorithm>
+
 #include "block.cuh"
 #include "fft2.cuh"
 #include "autotune.h"
@@ -32,6 +34,9 @@ struct ZFCfg {
     static constexpr int NPAIR = TB / 2;
     static constexpr int NT0 = NPAIR * LZ / 2;
     static constexpr int NT = NT0 < 128 ? 128 : NT0;
+    // threads per item: where a tile has fewer items than the CTA threads, an item's four points go to two or
+    // four of them, each with the Green values in its registers
+    static constexpr int SPLIT = NT0 >= 128 ? 1 : (NT0 == 64 ? 2 : 4);
     static constexpr int GS = LZ * TB + TB;  // component stride: TB float2 of padding keep half-warps apart
     static constexpr int BUF = 12 * GS;
     static constexpr size_t smem = sizeof(float2) * (size_t)(2 * BUF + LZ + 2 * NPAIR * 60);
@@ -157,8 +162,10 @@ __global__ void __launch_bounds__(ZFCfg<LZ, TB_>::NT, ZFCfg<LZ, TB_>::MINB)
     float2* gsec = tw + LZ;  // [NPAIR pairs][2 sets][NG] Green values of the item that holds kz = LZ/2
     const int tid = threadIdx.x;
     const int R = z.nact ? min(*z.nact, z.R) : z.R;
-    dev_bytes_add(z.bctr, 8.0 * (2.0 * R * 12 * z.nz * z.Ly * z.Lx + (double)NG * z.Ox * z.Oy * z.Oz), R > 0);
-    if (R <= 0) return;
+    dev_bytes_add(z.bctr, 8.0 * (2.0 * R * 12 * z.nz * z.Ly * z.Lx + (double)NG * z.Ox * z.Oy * z.Oz),
+                  R > 0 && blockIdx.y == 0);
+    const int r0 = blockIdx.y, rstep = gridDim.y;  // this CTA's right-hand sides
+    if (r0 >= R) return;
     for (int m = tid; m < LZ; m += NT) tw[m] = twg[m];
     const int ntile = z.Lx / TB;
     const int py = blockIdx.x / ntile, ct = blockIdx.x % ntile, sc0 = ct * TB;
@@ -189,7 +196,9 @@ __global__ void __launch_bounds__(ZFCfg<LZ, TB_>::NT, ZFCfg<LZ, TB_>::MINB)
     auto line = [](int n) { return (n / TB) * GS + n % TB; };
 
     // block-product item of this thread: column pair ci, kz item j
-    const int ci = tid % NPAIR, j = tid / NPAIR;
+    constexpr int SPLIT = Cfg::SPLIT;
+    const int ci = tid % NPAIR, j = (tid / NPAIR) % (LZ / 2);
+    const int part = SPLIT > 1 ? tid / Cfg::NT0 : 0;  // which of the item's points (SPLIT = 2: pa or pb; 4: one column of it)
     const bool single = ct == ntile - 1 && ci == NPAIR - 1;  // columns 0 and Lx/2: own octant columns
     const int kx0 = z.colkx[sc0 + 2 * ci], kx1 = z.colkx[sc0 + 2 * ci + 1];
     // kz items, in transposed positions p = k2 + B k1 holding kz = k1 + A k2:
@@ -218,6 +227,7 @@ __global__ void __launch_bounds__(ZFCfg<LZ, TB_>::NT, ZFCfg<LZ, TB_>::MINB)
         else
             pb = B - k2;
     }
+    if (part >= SPLIT || (single && part)) pa = pb = pc = -1;  // the self-mirrored columns' items are not split
     const int kxo0 = kx0 <= z.Lx / 2 ? kx0 : z.Lx - kx0, kxo1 = kx1 <= z.Lx / 2 ? kx1 : z.Lx - kx1;
     const float2* gcol0 = z.green_t + ((long long)kyo * z.Ox + kxo0) * z.Oz * NG;
     const float2* gcol1 = z.green_t + ((long long)kyo * z.Ox + kxo1) * z.Oz * NG;
@@ -228,25 +238,31 @@ __global__ void __launch_bounds__(ZFCfg<LZ, TB_>::NT, ZFCfg<LZ, TB_>::MINB)
     const int kzoa = kza <= LZ / 2 ? kza : LZ - kza;
     float2 u[NG];
     if (pa >= 0 && !single) {
-        if (pc >= 0) {
-            load_green<NG>(u, gcol0 + (long long)(LZ / 2) * NG);
+        if (SPLIT > 1) {  // the mirror's thread holds what the mirror takes
+            load_green<NG>(u, gcol0 + (long long)(pc >= 0 && part >= SPLIT / 2 ? LZ / 2 : kzoa) * NG);
             if (ry) mirror_y<KOP>(u);
+        } else {
+            if (pc >= 0) {
+                load_green<NG>(u, gcol0 + (long long)(LZ / 2) * NG);
+                if (ry) mirror_y<KOP>(u);
 #pragma unroll
-            for (int t = 0; t < NG; ++t) gsec[(2 * ci + 1) * NG + t] = u[t];
+                for (int t = 0; t < NG; ++t) gsec[(2 * ci + 1) * NG + t] = u[t];
+            }
+            load_green<NG>(u, gcol0 + (long long)kzoa * NG);
+            if (ry) mirror_y<KOP>(u);
+            if (pc >= 0)
+#pragma unroll
+                for (int t = 0; t < NG; ++t) gsec[(2 * ci) * NG + t] = u[t];
         }
-        load_green<NG>(u, gcol0 + (long long)kzoa * NG);
-        if (ry) mirror_y<KOP>(u);
-        if (pc >= 0)
-#pragma unroll
-            for (int t = 0; t < NG; ++t) gsec[(2 * ci) * NG + t] = u[t];
     }
 
-    issue(0, sb);
+    issue(r0, sb);
+    int odd = 0;
 #pragma unroll 1
-    for (int r = 0; r < R; ++r) {
-        float2* s = sb + (r & 1) * BUF;
-        if (r + 1 < R) {
-            issue(r + 1, sb + ((r + 1) & 1) * BUF);
+    for (int r = r0; r < R; r += rstep, odd ^= 1) {
+        float2* s = sb + odd * BUF;
+        if (r + rstep < R) {
+            issue(r + rstep, sb + (odd ^ 1) * BUF);
             cp_async_wait<1>();
         } else {
             cp_async_wait<0>();
@@ -257,19 +273,33 @@ __global__ void __launch_bounds__(ZFCfg<LZ, TB_>::NT, ZFCfg<LZ, TB_>::MINB)
             // columns kx and Lx - kx at pa (kz <= LZ/2) and at its mirror pb; the item without one (kz = 0) takes
             // kz = LZ/2 in its place with that point's values: it is its own mirror, where the tensors of odd z
             // parity vanish
-            const int off = pa * TB + 2 * ci;
-            col_point_r<KOP, false, false>(u, s, GS, off);
-            col_point_r<KOP, true, false>(u, s, GS, off + 1);
-            if (pc >= 0) {
+            const int off = pa * TB + 2 * ci, off2 = (pc >= 0 ? pc : pb) * TB + 2 * ci;
+            if constexpr (SPLIT == 4) {
+                if (part == 0) col_point_r<KOP, false, false>(u, s, GS, off);
+                if (part == 1) col_point_r<KOP, true, false>(u, s, GS, off + 1);
+                if (part == 2) col_point_r<KOP, false, true>(u, s, GS, off2);
+                if (part == 3) col_point_r<KOP, true, true>(u, s, GS, off2 + 1);
+            } else if constexpr (SPLIT == 2) {
+                if (part == 0) {
+                    col_point_r<KOP, false, false>(u, s, GS, off);
+                    col_point_r<KOP, true, false>(u, s, GS, off + 1);
+                } else {
+                    col_point_r<KOP, false, true>(u, s, GS, off2);
+                    col_point_r<KOP, true, true>(u, s, GS, off2 + 1);
+                }
+            } else {
+                col_point_r<KOP, false, false>(u, s, GS, off);
+                col_point_r<KOP, true, false>(u, s, GS, off + 1);
+                if (pc >= 0) {
 #pragma unroll
-                for (int t = 0; t < NG; ++t) u[t] = gsec[(2 * ci + 1) * NG + t];
-            }
-            const int off2 = (pc >= 0 ? pc : pb) * TB + 2 * ci;
-            col_point_r<KOP, false, true>(u, s, GS, off2);
-            col_point_r<KOP, true, true>(u, s, GS, off2 + 1);
-            if (pc >= 0) {
+                    for (int t = 0; t < NG; ++t) u[t] = gsec[(2 * ci + 1) * NG + t];
+                }
+                col_point_r<KOP, false, true>(u, s, GS, off2);
+                col_point_r<KOP, true, true>(u, s, GS, off2 + 1);
+                if (pc >= 0) {
 #pragma unroll
-                for (int t = 0; t < NG; ++t) u[t] = gsec[(2 * ci) * NG + t];
+                    for (int t = 0; t < NG; ++t) u[t] = gsec[(2 * ci) * NG + t];
+                }
             }
         } else if (pa >= 0) {
             // the self-mirrored columns 0 and Lx/2, each with its own Green values from global memory, one after
@@ -308,10 +338,15 @@ static int launch_zf_LT(const vie_handle* h, const ZFArgs& z, cudaStream_t s, co
     VIE_CUDA(cudaFuncSetAttribute(zfused_kernel<LZ, TB, KOP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)smem));
     const long long blocks = (long long)z.Ly * (z.Lx / TB);
+    // Small spectra: the right-hand sides are dealt out to several CTAs per tile, until four CTAs wait for every place on
+    // the 152 SMs; a CTA then loads the Green values for fewer of them.  16 right-hand sides on 10^3 voxels
+    // (32^3 points): 142 to 61 us with the items' points split as well; 8 on 32^3 voxels: 211 to 172 us.
+    const long long places = 152LL * Cfg::MINB;
+    const unsigned parts = (unsigned)std::min<long long>(z.R, std::max<long long>(1, (4 * places + blocks - 1) / blocks));
     // with a device count the kernel adds its bytes to z.bctr
     const double bytes = z.nact ? kDevCounted : 8.0 * (2.0 * z.R * 12 * z.nz * z.Ly * z.Lx + NG * z.Ox * z.Oy * z.Oz);
     VIE_KLAUNCH_B(name, s, bytes,
-                  zfused_kernel<LZ, TB, KOP><<<(unsigned)blocks, Cfg::NT, smem, s>>>(z, h->tw32 + LZ));
+                  zfused_kernel<LZ, TB, KOP><<<dim3((unsigned)blocks, parts), Cfg::NT, smem, s>>>(z, h->tw32 + LZ));
     VIE_CHECK_LAUNCH();
     return VIE_OK;
 }
