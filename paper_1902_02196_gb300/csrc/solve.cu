@@ -232,23 +232,6 @@ __global__ void __launch_bounds__(kThreads) finalize2_kernel(const double2* __re
     }
 }
 
-__global__ void __launch_bounds__(kThreads) finalize1_kernel(const double* __restrict__ part, int nblk,
-                                                             double* __restrict__ out, const int* __restrict__ flag) {
-    __shared__ double sh[kWarps];
-    const int r = blockIdx.x;
-    if (flag && !flag[r]) return;
-    double a = 0;
-    for (int b = threadIdx.x; b < nblk; b += kThreads) a += part[(long long)r * nblk + b];
-    a = warp_sum(a);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0;
-        for (int q = 0; q < kWarps; ++q) s += sh[q];
-        out[r] = s;
-    }
-}
-
 __global__ void copy_norm_kernel(const double2* __restrict__ D, int ldd, double* out, int R) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r < R) out[r] = D[(long long)r * ldd].x;
@@ -366,6 +349,7 @@ struct GState {
     int* reflag;     // [R] second Gram-Schmidt pass needed
     int* k;          // [R] Arnoldi steps of the current cycle
     int* nactive;    // [1 + R]: the number of active right-hand sides, then their indices
+    int* arrived;    // [1] blocks of step_end_kernel that have finished (0 between its launches)
     double2* shift;  // [R] shift of the Arnoldi matvec: w = (P^-1 A - shift) u_j
 };
 
@@ -384,117 +368,202 @@ __global__ void cycle_init_kernel(GState s, int R, const double* __restrict__ rn
     s.nrm[r * (s.m + 1)] = 1.0;
 }
 
-// after the first projection pass: H[:, j], coefficients, rescale 1/|w|
-// (one block per right-hand side, a thread per entry i <= j)
-__global__ void coef1_kernel(GState s, int R, int j) {
-    const int r = blockIdx.x;
-    if (r >= R || !s.active[r]) return;
-    const int m = s.m;
-    const double2* D = s.D + (long long)r * (m + 2);
-    const double* n = s.nrm + (long long)r * (m + 1);
-    double2* H = s.H + (long long)r * (m + 1) * m;
-    const double nj = n[j];
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
-        const double2 d = D[i];
-        H[i * m + j] = make_double2(d.x / (n[i] * nj), d.y / (n[i] * nj));
-        s.coef[(long long)r * (m + 1) + i] = make_double2(d.x / (n[i] * n[i]), d.y / (n[i] * n[i]));
-    }
+// block sum of part[0..nblk) in a fixed order; thread 0 has the sum
+__device__ __forceinline__ double sum_partials(const double* __restrict__ part, int nblk, double* sh) {
+    double a = 0;
+    for (int b = threadIdx.x; b < nblk; b += kThreads) a += part[b];
+    a = warp_sum(a);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const double e = D[j + 1].x;
-        const double sc = e > 0.0 ? 1.0 / sqrt(e) : 0.0;
-        s.scale[r] = sc;
-        s.sigma[r] = sc;
-        // the matvec applied P^-1 A - shift: restore the diagonal entry, and shift the next
-        // step by it (the Krylov space and H are those of P^-1 A; the shift only removes
-        // the part of the new vector along u_j before the projections, which keeps the
-        // Gram-Schmidt passes from cancelling most of it)
-        double2 hjj = H[j * m + j];
-        hjj.x += s.shift[r].x;
-        hjj.y += s.shift[r].y;
-        H[j * m + j] = hjj;
-        if (isfinite(hjj.x) && isfinite(hjj.y)) s.shift[r] = hjj;
+    double t = 0;
+    if (threadIdx.x == 0)
+        for (int q = 0; q < kWarps; ++q) t += sh[q];
+    return t;
+}
+
+// The small kernels of an Arnoldi step are each a launch on the critical path, 3 to 4 us on small grids, so
+// what follows from one sum is done by the block that forms it: a step has four of them besides the
+// matvec and the passes over the basis, where it had nine.  8 right-hand sides on 32^3 voxels: 1186 launches and
+// 13 ms less per solve of 215 steps, most of it one thread's rotations (32 us a step, now below 10).
+
+// After a projection pass's inner products, one block per (entry i <= j + 1, right-hand side): the sum over
+// the partials, and what follows from it alone.
+// PASS 1: H[i][j], the coefficient of u_i, and from |w|^2 (i = j + 1) the rescale factor 1/|w|.
+// PASS 2 (right-hand sides with reflag): their corrections.
+template <int PASS>
+__global__ void __launch_bounds__(kThreads) project_kernel(GState s, const double2* __restrict__ partial, int nblk, int j) {
+    __shared__ double2 sh[kWarps];
+    const int i = blockIdx.x, r = blockIdx.y, m = s.m, nv = j + 2;
+    if (PASS == 1 ? !s.active[r] : !s.reflag[r]) return;
+    double2 a = make_double2(0, 0);
+    for (int b = threadIdx.x; b < nblk; b += kThreads) {
+        const double2 v = partial[((long long)r * nblk + b) * nv + i];
+        a.x += v.x, a.y += v.y;
+    }
+    a.x = warp_sum(a.x);
+    a.y = warp_sum(a.y);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    double2 d = make_double2(0, 0);
+    for (int q = 0; q < kWarps; ++q) d.x += sh[q].x, d.y += sh[q].y;
+    if (i == j + 1) {
+        if (PASS == 1) {
+            const double sc = d.x > 0.0 ? 1.0 / sqrt(d.x) : 0.0;
+            s.scale[r] = sc;
+            s.sigma[r] = sc;
+        }
+        return;
+    }
+    const double* n = s.nrm + (long long)r * (m + 1);
+    double2* h = s.H + (long long)r * (m + 1) * m + i * m + j;
+    s.coef[(long long)r * (m + 1) + i] = make_double2(d.x / (n[i] * n[i]), d.y / (n[i] * n[i]));
+    if (PASS == 1) {
+        double2 v = make_double2(d.x / (n[i] * n[j]), d.y / (n[i] * n[j]));
+        if (i == j) {
+            // the matvec applied P^-1 A - shift: restore the diagonal entry, and shift the next
+            // step by it (the Krylov space and H are those of P^-1 A; the shift only removes
+            // the part of the new vector along u_j before the projections, which keeps the
+            // Gram-Schmidt passes from cancelling most of it)
+            v.x += s.shift[r].x;
+            v.y += s.shift[r].y;
+            if (isfinite(v.x) && isfinite(v.y)) s.shift[r] = v;
+        }
+        *h = v;
+    } else {
+        const double f = n[j] * s.sigma[r];
+        h->x += d.x / (n[i] * f);
+        h->y += d.y / (n[i] * f);
     }
 }
 
-// second pass where the rescaled new vector has squared length below 1/2
-__global__ void reorth_kernel(GState s, int R) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    const double f = s.F[r];
-    const int fl = s.active[r] && f > 0.0 && f < 0.5;
+// after the first update: its squared norm, and the second pass where the rescaled new vector has squared
+// length below 1/2.  One block per right-hand side.
+__global__ void __launch_bounds__(kThreads) reorth_kernel(GState s, const double* __restrict__ npart, int nblk) {
+    __shared__ double sh[kWarps];
+    const int r = blockIdx.x;
+    if (!s.active[r]) {
+        if (threadIdx.x == 0) s.reflag[r] = 0;
+        return;
+    }
+    const double f = sum_partials(npart + (long long)r * nblk, nblk, sh);
+    if (threadIdx.x != 0) return;
+    s.F[r] = f;
+    const int fl = f > 0.0 && f < 0.5;
     s.reflag[r] = fl;
     if (fl) s.scale[r] = 1.0 / sqrt(f);
 }
 
-// after the second projection pass: correction of H[:, j], coefficients, cumulative rescale
-// (one block per right-hand side, a thread per entry i <= j)
-__global__ void coef2_kernel(GState s, int R, int j) {
-    const int r = blockIdx.x;
-    if (r >= R || !s.reflag[r]) return;
-    const int m = s.m;
-    const double2* D = s.D + (long long)r * (m + 2);
-    const double* n = s.nrm + (long long)r * (m + 1);
-    double2* H = s.H + (long long)r * (m + 1) * m;
-    const double f = n[j] * s.sigma[r];
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
-        const double2 d = D[i];
-        H[i * m + j].x += d.x / (n[i] * f);
-        H[i * m + j].y += d.y / (n[i] * f);
-        s.coef[(long long)r * (m + 1) + i] = make_double2(d.x / (n[i] * n[i]), d.y / (n[i] * n[i]));
+// End of step j, one block per right-hand side: the second update's squared norm where there was one, the
+// Givens rotations, and (the last block) the list of right-hand sides still active: out[0] their number, then their
+// indices in increasing order.
+__global__ void __launch_bounds__(kThreads) step_end_kernel(GState s, int R, const double* __restrict__ npart, int nblk,
+                                                            int j) {
+    __shared__ double sh[kWarps];
+    __shared__ double2 col[kMaxV], rs[kMaxV], ch[kMaxV];
+    __shared__ double rc[kMaxV];
+    __shared__ int last;
+    const int r = blockIdx.x, m = s.m;
+    if (s.active[r]) {
+        double2* H = s.H + (long long)r * (m + 1) * m;
+        const int re = s.reflag[r];
+        const double f2 = re ? sum_partials(npart + (long long)r * nblk, nblk, sh) : 0.0;
+        // rotation i takes (a_i, b = h_{i+1}) to h_i = c a_i + sn b and a_{i+1} = c b - conj(sn) a_i.  Only the a_i
+        // are a chain: real and imaginary part in a lane each, two multiply-adds a link (an FP64
+        // instruction takes a warp 16 clocks at the least); the rest is done for all i at once.
+        for (int i = threadIdx.x; i <= j; i += kThreads) {
+            col[i] = H[i * m + j];
+            rc[i] = i < j ? s.cs[r * m + i].x : 0.0;
+            rs[i] = i < j ? s.sn[r * m + i] : make_double2(0, 0);
+        }
+        __syncthreads();
+        if (threadIdx.x < 2) {
+            const bool im = threadIdx.x == 1;
+            double a = im ? col[0].y : col[0].x;
+            for (int i = 0; i < j; ++i) {
+                if (im)
+                    ch[i].y = a;
+                else
+                    ch[i].x = a;
+                const double other = __shfl_xor_sync(3u, a, 1);
+                const double2 sn = rs[i], b = col[i + 1];
+                a = fma(im ? sn.y : -sn.y, other, fma(-sn.x, a, rc[i] * (im ? b.y : b.x)));
+            }
+            if (im)
+                ch[j].y = a;
+            else
+                ch[j].x = a;
+        }
+        __syncthreads();
+        double2 hi = make_double2(0, 0);
+        if (threadIdx.x < j) {  // j < kThreads
+            const int i = threadIdx.x;
+            const double2 a = ch[i], b = col[i + 1], sn = rs[i];
+            const double c = rc[i];
+            hi = make_double2(c * a.x + sn.x * b.x - sn.y * b.y, c * a.y + sn.x * b.y + sn.y * b.x);
+        }
+        __syncthreads();
+        if (threadIdx.x < j) col[threadIdx.x] = hi;
+        if (threadIdx.x == 0) {
+            double* n = s.nrm + (long long)r * (m + 1);
+            const double F = re ? f2 : s.F[r], sigma = re ? s.sigma[r] * s.scale[r] : s.sigma[r];
+            if (re) s.F[r] = F, s.sigma[r] = sigma;
+            const double nn = sqrt(fmax(F, 0.0));
+            n[j + 1] = nn;
+            const double hnext = (sigma > 0.0 && n[j] > 0.0) ? nn / (sigma * n[j]) : 0.0;
+            const double2 a = ch[j];
+            const double b = hnext;
+            const double aa = hypot(a.x, a.y);
+            const double den = hypot(aa, b);
+            double c;
+            double2 sn;
+            if (den == 0.0) {
+                c = 1.0;
+                sn = make_double2(0, 0);
+            } else if (aa == 0.0) {
+                c = 0.0;
+                sn = make_double2(1.0, 0);
+            } else {
+                c = aa / den;
+                sn = make_double2(a.x / aa * b / den, a.y / aa * b / den);  // (a/|a|) conj(b)/den, b real
+            }
+            s.cs[r * m + j] = make_double2(c, 0);
+            s.sn[r * m + j] = sn;
+            col[j] = make_double2(c * a.x + sn.x * b, c * a.y + sn.y * b);
+            double2* g = s.g + r * (m + 1);
+            const double2 gj = g[j];
+            const double2 gn = make_double2(-(sn.x * gj.x + sn.y * gj.y), -(sn.x * gj.y - sn.y * gj.x));
+            g[j + 1] = gn;
+            g[j] = make_double2(c * gj.x, c * gj.y);
+            s.k[r] = j + 1;
+            const double res = hypot(gn.x, gn.y);
+            if (res <= s.target[r] || hnext == 0.0 || !isfinite(res)) s.active[r] = 0;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i <= j; i += kThreads) H[i * m + j] = col[i];
     }
-    __syncthreads();  // every thread has read sigma
-    if (threadIdx.x == 0) s.sigma[r] *= s.scale[r];
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(s.arrived, 1) == R - 1;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    int c = 0;
+    for (int base = 0; base < R; base += 32) {
+        const int q = base + (int)threadIdx.x;
+        const bool act = q < R && __ldcg(s.active + q);
+        const unsigned mask = __ballot_sync(0xffffffffu, act);
+        if (act) s.nactive[1 + c + __popc(mask & ((1u << threadIdx.x) - 1u))] = q;
+        c += __popc(mask);
+    }
+    if (threadIdx.x == 0) {
+        s.nactive[0] = c;
+        *s.arrived = 0;
+    }
 }
 
-// Givens step j for every active right-hand side
-__global__ void givens_kernel(GState s, int R, int j) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R || !s.active[r]) return;
-    const int m = s.m;
-    double2* H = s.H + (long long)r * (m + 1) * m;
-    double* n = s.nrm + (long long)r * (m + 1);
-    const double nn = sqrt(fmax(s.F[r], 0.0));
-    n[j + 1] = nn;
-    const double hnext = (s.sigma[r] > 0.0 && n[j] > 0.0) ? nn / (s.sigma[r] * n[j]) : 0.0;
-    for (int i = 0; i < j; ++i) {
-        const double2 a = H[i * m + j], b = H[(i + 1) * m + j];
-        const double c = s.cs[r * m + i].x;
-        const double2 sn = s.sn[r * m + i];
-        const double2 t = make_double2(c * a.x + sn.x * b.x - sn.y * b.y, c * a.y + sn.x * b.y + sn.y * b.x);
-        const double2 bb = make_double2(-(sn.x * a.x + sn.y * a.y) + c * b.x, -(sn.x * a.y - sn.y * a.x) + c * b.y);
-        H[i * m + j] = t;
-        H[(i + 1) * m + j] = bb;
-    }
-    const double2 a = H[j * m + j];
-    const double b = hnext;
-    const double aa = hypot(a.x, a.y);
-    const double den = hypot(aa, b);
-    double c;
-    double2 sn;
-    if (den == 0.0) {
-        c = 1.0;
-        sn = make_double2(0, 0);
-    } else if (aa == 0.0) {
-        c = 0.0;
-        sn = make_double2(1.0, 0);
-    } else {
-        c = aa / den;
-        sn = make_double2(a.x / aa * b / den, a.y / aa * b / den);  // (a/|a|) conj(b)/den, b real
-    }
-    s.cs[r * m + j] = make_double2(c, 0);
-    s.sn[r * m + j] = sn;
-    H[j * m + j] = make_double2(c * a.x + sn.x * b, c * a.y + sn.y * b);
-    double2* g = s.g + r * (m + 1);
-    const double2 gj = g[j];
-    g[j + 1] = make_double2(-(sn.x * gj.x + sn.y * gj.y), -(sn.x * gj.y - sn.y * gj.x));
-    g[j] = make_double2(c * gj.x, c * gj.y);
-    s.k[r] = j + 1;
-    const double res = hypot(g[j + 1].x, g[j + 1].y);
-    if (res <= s.target[r] || hnext == 0.0 || !isfinite(res)) s.active[r] = 0;
-}
-
-// out[0] = number of active right-hand sides, out[1..] = their indices in increasing order
+// out[0] = number of active right-hand sides, out[1..] = their indices in increasing order (start of a cycle)
 __global__ void count_active_kernel(const int* __restrict__ active, int R, int* out) {
     int c = 0;
     for (int r = 0; r < R; ++r)
@@ -502,30 +571,34 @@ __global__ void count_active_kernel(const int* __restrict__ active, int R, int* 
     out[0] = c;
 }
 
-// back substitution H(0:k,0:k) y = g(0:k), then the update coefficients y_i / n_i
-__global__ void trisolve_kernel(GState s, int R) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
+// back substitution H(0:k,0:k) y = g(0:k), then the update coefficients y_i / n_i: one block per right-hand side, thread
+// q keeps the remainder of row q and takes column i's part off it once y_i is known
+__global__ void __launch_bounds__(128) trisolve_kernel(GState s) {
+    __shared__ double2 yi;
+    const int r = blockIdx.x, q = threadIdx.x;
     const int m = s.m, k = s.k[r];
     const double2* H = s.H + (long long)r * (m + 1) * m;
-    const double2* g = s.g + r * (m + 1);
-    const double* n = s.nrm + (long long)r * (m + 1);
-    double2* y = s.y + r * m;
+    double2 acc = q < k ? s.g[r * (m + 1) + q] : make_double2(0, 0);
+    double2 h = q < k ? H[q * m + k - 1] : make_double2(0, 0);
     for (int i = k - 1; i >= 0; --i) {
-        double2 acc = g[i];
-        for (int q = i + 1; q < k; ++q) {
-            const double2 hq = H[i * m + q], yv = y[q];
+        const double2 hq = h;
+        if (q < i) h = H[q * m + i - 1];
+        if (q == i) {
+            const double dd = hq.x * hq.x + hq.y * hq.y;
+            yi = dd > 0 ? make_double2((acc.x * hq.x + acc.y * hq.y) / dd, (acc.y * hq.x - acc.x * hq.y) / dd)
+                        : make_double2(0, 0);
+        }
+        __syncthreads();
+        const double2 yv = yi;
+        if (q < i) {
             acc.x -= hq.x * yv.x - hq.y * yv.y;
             acc.y -= hq.x * yv.y + hq.y * yv.x;
         }
-        const double2 d = H[i * m + i];
-        const double dd = d.x * d.x + d.y * d.y;
-        y[i] = dd > 0 ? make_double2((acc.x * d.x + acc.y * d.y) / dd, (acc.y * d.x - acc.x * d.y) / dd)
-                      : make_double2(0, 0);
-    }
-    for (int i = 0; i < k; ++i) {
-        const double ni = n[i];
-        y[i] = make_double2(y[i].x / ni, y[i].y / ni);
+        if (q == i) {
+            const double ni = s.nrm[(long long)r * (m + 1) + i];
+            s.y[r * m + i] = make_double2(yv.x / ni, yv.y / ni);
+        }
+        __syncthreads();
     }
 }
 
@@ -685,14 +758,16 @@ struct Solver {
     double* npart;     // [R][nblk]
     GState gs;
 
-    template <typename VC>
-    int dots(const VC* U, long long ustride, const VC* w, int nvec, const int* flag) {
+    // inner products of w with nvec basis vectors and what follows from them (project_kernel), for the
+    // active right-hand sides (PASS 1) or those that need a second pass (2)
+    template <int PASS, typename VC>
+    int dots(const VC* U, long long ustride, const VC* w, int nvec) {
         const dim3 g1(nblk, R);
         VIE_KLAUNCH("gs_dots", st,
-                    gs_dots_kernel<VC><<<g1, kThreads, 0, st>>>(U, ustride, w, n, nvec, partial, nblk, flag));
+                    gs_dots_kernel<VC><<<g1, kThreads, 0, st>>>(U, ustride, w, n, nvec, partial, nblk,
+                                                               PASS == 1 ? gs.active : gs.reflag));
         const dim3 g2(nvec + 1, R);
-        VIE_KLAUNCH("gs_finalize", st,
-                    finalize2_kernel<<<g2, kThreads, 0, st>>>(partial, nblk, nvec + 1, gs.D, m + 2, flag));
+        VIE_KLAUNCH("arnoldi_project", st, project_kernel<PASS><<<g2, kThreads, 0, st>>>(gs, partial, nblk, nvec - 1));
         VIE_CHECK_LAUNCH();
         return VIE_OK;
     }
@@ -702,7 +777,6 @@ struct Solver {
         VIE_KLAUNCH("gs_update", st,
                     gs_update_kernel<VC><<<g1, kThreads, 0, st>>>(U, ustride, w, n, nvec, gs.coef, m + 1, gs.scale,
                                                                  npart, nblk, flag));
-        VIE_KLAUNCH("gs_norm", st, finalize1_kernel<<<R, kThreads, 0, st>>>(npart, nblk, gs.F, flag));
         VIE_CHECK_LAUNCH();
         return VIE_OK;
     }
@@ -726,24 +800,22 @@ struct Solver {
 
 // Arnoldi steps [j0, j1) of a GMRES(m) cycle from the residual r64 (squared norms rn2), enqueued
 // on the stream with no host read inside: every step works on the device's list of active
-// right-hand sides (count_active before each step), so a step after every right-hand side has
-// stopped finds an empty list and its kernels return at once.  The first chunk starts the cycle;
-// every chunk ends by counting the right-hand sides still active.
+// right-hand sides (which every step's last kernel renews), so a step after every right-hand side has
+// stopped finds an empty list and its kernels return at once.  The first chunk starts the cycle.
 template <typename VC>
 int enqueue_steps(Solver& S, VC* U, const double2* r64, const double* rn2, int precision, int j0, int j1) {
     vie_handle* h = S.h;
     const int R = S.R;
     const long long n = S.n, ustride = (long long)R * n;
     cudaStream_t st = S.st;
-    const unsigned gr = (unsigned)((R + 127) / 128);
     if (j0 == 0) {
         VIE_KLAUNCH("cycle_init", st, cycle_init_kernel<<<(R + 127) / 128, 128, 0, st>>>(S.gs, R, rn2));
         const dim3 ge((unsigned)((n + 255) / 256), R);
         VIE_KLAUNCH("basis_init", st, scale_from64_kernel<VC><<<ge, 256, 0, st>>>(r64, U, n, S.gs.scale));
+        VIE_KLAUNCH("count_active", st, count_active_kernel<<<1, 1, 0, st>>>(S.gs.active, R, S.gs.nactive));
         VIE_CHECK_LAUNCH();
     }
     for (int j = j0; j < j1; ++j) {
-        VIE_KLAUNCH("count_active", st, count_active_kernel<<<1, 1, 0, st>>>(S.gs.active, R, S.gs.nactive));
         VC* uj = U + j * ustride;
         VC* w = U + (j + 1) * ustride;
         // only the active right-hand sides (the others' w is never read)
@@ -753,18 +825,14 @@ int enqueue_steps(Solver& S, VC* U, const double2* r64, const double* rn2, int p
         else
             VIE_TRY(matvec_support(h, R, uj, w, precision, VIE_OP_PA, S.sp, S.mv_tmp, st, S.gs.shift, nullptr,
                                    S.gs.nactive + 1, S.gs.nactive));
-        VIE_TRY(S.dots<VC>(U, ustride, w, j + 1, S.gs.active));
-        VIE_KLAUNCH("arnoldi_coef", st, coef1_kernel<<<R, 128, 0, st>>>(S.gs, R, j));
+        VIE_TRY((S.dots<1, VC>(U, ustride, w, j + 1)));
         VIE_TRY(S.update<VC>(U, ustride, w, j + 1, S.gs.active));
-        VIE_KLAUNCH("arnoldi_reorth", st, reorth_kernel<<<gr, 128, 0, st>>>(S.gs, R));
-        VIE_TRY(S.dots<VC>(U, ustride, w, j + 1, S.gs.reflag));
-        VIE_KLAUNCH("arnoldi_coef", st, coef2_kernel<<<R, 128, 0, st>>>(S.gs, R, j));
+        VIE_KLAUNCH("arnoldi_reorth", st, reorth_kernel<<<R, kThreads, 0, st>>>(S.gs, S.npart, S.nblk));
+        VIE_TRY((S.dots<2, VC>(U, ustride, w, j + 1)));
         VIE_TRY(S.update<VC>(U, ustride, w, j + 1, S.gs.reflag));
-        VIE_KLAUNCH("givens", st, givens_kernel<<<gr, 128, 0, st>>>(S.gs, R, j));
+        VIE_KLAUNCH("arnoldi_step_end", st, step_end_kernel<<<R, kThreads, 0, st>>>(S.gs, R, S.npart, S.nblk, j));
         VIE_CHECK_LAUNCH();
     }
-    VIE_KLAUNCH("count_active", st, count_active_kernel<<<1, 1, 0, st>>>(S.gs.active, R, S.gs.nactive));
-    VIE_CHECK_LAUNCH();
     return VIE_OK;
 }
 
@@ -774,8 +842,7 @@ int enqueue_finish(Solver& S, VC* U, double2* x64) {
     const int R = S.R, m = S.m;
     const long long n = S.n, ustride = (long long)R * n;
     cudaStream_t st = S.st;
-    const unsigned gr = (unsigned)((R + 127) / 128);
-    VIE_KLAUNCH("trisolve", st, trisolve_kernel<<<gr, 128, 0, st>>>(S.gs, R));
+    VIE_KLAUNCH("trisolve", st, trisolve_kernel<<<R, 128, 0, st>>>(S.gs));
     const dim3 gx((unsigned)((n + kThreads * Prec<VC>::K - 1) / (kThreads * Prec<VC>::K)), R);
     VIE_KLAUNCH("solution_update", st,
                 xupdate_kernel<VC><<<gx, kThreads, 0, st>>>(U, ustride, x64, n, S.gs.y, m, S.gs.k, 0));
@@ -949,7 +1016,7 @@ int solve_device(vie_handle* h, int R, const double2* b, double2* x, double tol,
     const size_t oAct = take(sizeof(int) * R);
     const size_t oRe = take(sizeof(int) * R);
     const size_t oK = take(sizeof(int) * R);
-    const size_t oNact = take(sizeof(int) * (R + 1));
+    const size_t oNact = take(sizeof(int) * (R + 2));
     const size_t oBn = take(sizeof(double) * R);
     const size_t oRn = take(sizeof(double) * R);
     const size_t oDone = take(sizeof(int) * R);
@@ -1010,6 +1077,8 @@ int solve_device(vie_handle* h, int R, const double2* b, double2* x, double tol,
     S.gs.reflag = reinterpret_cast<int*>(base + oRe);
     S.gs.k = reinterpret_cast<int*>(base + oK);
     S.gs.nactive = reinterpret_cast<int*>(base + oNact);
+    S.gs.arrived = S.gs.nactive + R + 1;
+    VIE_CUDA(cudaMemsetAsync(S.gs.arrived, 0, sizeof(int), st));
     S.gs.shift = reinterpret_cast<double2*>(base + oShift);
     VIE_CUDA(cudaMemsetAsync(S.gs.shift, 0, sizeof(double2) * R, st));  // the first step is unshifted
     double2* r64 = reinterpret_cast<double2*>(base + oR);
