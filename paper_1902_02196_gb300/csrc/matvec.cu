@@ -217,9 +217,9 @@ struct XYCfg {
 // [R][12][Nz][Ny][Nx], or [R][12][ns] on a support (rows != NULL; zeros outside it).
 template <int L>
 __global__ void __launch_bounds__(kXYThreads, XYCfg<L>::MINB)
-    xy_fwd_kernel(const float2* __restrict__ x, float2* __restrict__ w, int nx, int ny, int nz, const int4* __restrict__ rows,
+    xy_fwd_kernel(const float2* x, float2* w, int nx, int ny, int nz, const int4* __restrict__ rows,
                   long long ns, const unsigned char* __restrict__ cpos, const float2* __restrict__ twg,
-                  const int* __restrict__ rmap, MatvecEpi dc) {
+                  const int* rmap, MatvecEpi dc) {
     using Cfg = XYCfg<L>;
     using C = float2;
     constexpr int A = fft2::Split<L>::A, B = fft2::Split<L>::B, NT = kXYThreads, RS = Cfg::RS, CW = Cfg::CW;
@@ -233,14 +233,16 @@ __global__ void __launch_bounds__(kXYThreads, XYCfg<L>::MINB)
     const long long p = blockIdx.x;  // spectrum plane; the input plane is pin (rmap: active right-hand sides)
     const long long rplanes = (long long)dc.nc * nz;  // planes per right-hand side
     const SmallDiv dnx(nx), dny(ny);
+    grid_release();
+    for (int m = tid; m < L; m += NT) {
+        tw[m] = twg[m];
+        pos[m] = cpos[m];
+    }
+    grid_wait();
     if (dc.nact) {  // planes of right-hand sides beyond the device count are skipped
         const int cnt = *dc.nact;
         dev_bytes_add(dc.bctr, dc.bfix + dc.bper * cnt, cnt > 0);
         if (p / rplanes >= cnt) return;
-    }
-    for (int m = tid; m < L; m += NT) {
-        tw[m] = twg[m];
-        pos[m] = cpos[m];
     }
     const long long pin = rmap ? (long long)rmap[p / rplanes] * rplanes + p % rplanes : p;
     if (rows) {
@@ -330,7 +332,7 @@ __global__ void __launch_bounds__(kXYThreads, XYCfg<L>::MINB)
 // Inverse: W2 plane -> y plane [Ny][Nx] with the material / Gram / preconditioner epilogue.
 template <int L>
 __global__ void __launch_bounds__(kXYThreads, XYCfg<L>::MINB)
-    xy_inv_kernel(const float2* __restrict__ w, float2* __restrict__ y, MatvecEpi epi,
+    xy_inv_kernel(const float2* w, float2* y, MatvecEpi epi,
                   const unsigned char* __restrict__ cpos, const float2* __restrict__ twg) {
     using Cfg = XYCfg<L>;
     using C = float2;
@@ -348,14 +350,16 @@ __global__ void __launch_bounds__(kXYThreads, XYCfg<L>::MINB)
     const int nc = epi.nc;
     const long long rplanes = (long long)nc * nz;  // planes per right-hand side
     const SmallDiv dnx(nx), dny(ny);
+    grid_release();
+    for (int m = tid; m < L; m += NT) {
+        tw[m] = twg[m];
+        pos[m] = cpos[m];
+    }
+    grid_wait();
     if (epi.nact) {
         const int cnt = *epi.nact;
         dev_bytes_add(epi.bctr, epi.bfix + epi.bper * cnt, cnt > 0);
         if (p / rplanes >= cnt) return;
-    }
-    for (int m = tid; m < L; m += NT) {
-        tw[m] = twg[m];
-        pos[m] = cpos[m];
     }
     const long long po = epi.rmap ? (long long)epi.rmap[p / rplanes] * rplanes + p % rplanes : p;
     if (epi.rows)
@@ -609,12 +613,11 @@ static int launch_xy_L(bool fwd, const char* name, double bytes, const vie_handl
     // set on every call: the attribute is per device and launches may come from several threads
     if (fwd) {
         VIE_CUDA(cudaFuncSetAttribute(xy_fwd_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        VIE_KLAUNCH_B(name, s, bytes,
-                      xy_fwd_kernel<L><<<planes, kXYThreads, smem, s>>>(in, out, nx, ny, h->nz, sp.rows, sp.ns, cpos, tw,
-                                                                       e.rmap, e));
+        VIE_LAUNCH(name, s, bytes, (xy_fwd_kernel<L>), planes, kXYThreads, smem, in, out, nx, ny, h->nz, sp.rows, sp.ns,
+                   cpos, tw, e.rmap, e);
     } else {
         VIE_CUDA(cudaFuncSetAttribute(xy_inv_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        VIE_KLAUNCH_B(name, s, bytes, xy_inv_kernel<L><<<planes, kXYThreads, smem, s>>>(in, out, e, cpos, tw));
+        VIE_LAUNCH(name, s, bytes, (xy_inv_kernel<L>), planes, kXYThreads, smem, in, out, e, cpos, tw);
     }
     VIE_CHECK_LAUNCH();
     return VIE_OK;

@@ -73,7 +73,7 @@ __device__ __forceinline__ bool al16(const void* p) { return (reinterpret_cast<u
 // K consecutive complex values starting at element e0 of p (zero past n); 16-byte loads
 // when the chunk is complete and aligned.
 template <typename C, int K>
-__device__ __forceinline__ void load_chunk(const C* __restrict__ p, long long e0, long long n, C* v) {
+__device__ __forceinline__ void load_chunk(const C* p, long long e0, long long n, C* v) {
     if (e0 + K <= n && (sizeof(C) != 8 || al16(p + e0))) {
         if constexpr (sizeof(C) == 8) {
             const float4* q = reinterpret_cast<const float4*>(p + e0);
@@ -112,14 +112,16 @@ __device__ __forceinline__ void store_chunk(C* __restrict__ p, long long e0, lon
 
 // partial[r][blk][i] = sum over the block's elements of conj(U_i) w (i < nvec) and, at i = nvec, |w|^2
 template <typename VC>
-__global__ void __launch_bounds__(kThreads) gs_dots_kernel(const VC* __restrict__ U, long long ustride,
-                                                           const VC* __restrict__ w, long long n, int nvec,
-                                                           double2* __restrict__ partial, int nblk,
-                                                           const int* __restrict__ flag) {
+__global__ void __launch_bounds__(kThreads) gs_dots_kernel(const VC* U, long long ustride,
+                                                           const VC* w, long long n, int nvec,
+                                                           double2* partial, int nblk,
+                                                           const int* flag) {
     using R = typename Prec<VC>::R;
     constexpr int K = Prec<VC>::K;
     __shared__ double2 sh[kWarps][kMaxV + 1];
     const int r = blockIdx.y, blk = blockIdx.x;
+    grid_release();
+    grid_wait();
     if (flag && !flag[r]) return;
     if (blk == 0 && threadIdx.x == 0) atomicAdd(&g_gs_bytes[0], (unsigned long long)(n * sizeof(VC) * (nvec + 1)));
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -159,16 +161,18 @@ __global__ void __launch_bounds__(kThreads) gs_dots_kernel(const VC* __restrict_
 
 // w <- scale * (w - sum_i coef_i U_i), in place; npart[r][blk] = |new w|^2 over the block
 template <typename VC>
-__global__ void __launch_bounds__(kThreads) gs_update_kernel(const VC* __restrict__ U, long long ustride, VC* w,
-                                                             long long n, int nvec, const double2* __restrict__ coef,
-                                                             int ldc, const double* __restrict__ scale,
-                                                             double* __restrict__ npart, int nblk,
-                                                             const int* __restrict__ flag) {
+__global__ void __launch_bounds__(kThreads) gs_update_kernel(const VC* U, long long ustride, VC* w,
+                                                             long long n, int nvec, const double2* coef,
+                                                             int ldc, const double* scale,
+                                                             double* npart, int nblk,
+                                                             const int* flag) {
     using R = typename Prec<VC>::R;
     constexpr int K = Prec<VC>::K;
     __shared__ VC c[kMaxV];
     __shared__ double shn[kWarps];
     const int r = blockIdx.y, blk = blockIdx.x;
+    grid_release();
+    grid_wait();
     if (flag && !flag[r]) return;
     if (blk == 0 && threadIdx.x == 0) atomicAdd(&g_gs_bytes[1], (unsigned long long)(n * sizeof(VC) * (nvec + 2)));
     for (int i = threadIdx.x; i < nvec; i += kThreads) c[i] = from_d<VC>(coef[(long long)r * ldc + i]);
@@ -369,7 +373,7 @@ __global__ void cycle_init_kernel(GState s, int R, const double* __restrict__ rn
 }
 
 // block sum of part[0..nblk) in a fixed order; thread 0 has the sum
-__device__ __forceinline__ double sum_partials(const double* __restrict__ part, int nblk, double* sh) {
+__device__ __forceinline__ double sum_partials(const double* part, int nblk, double* sh) {
     double a = 0;
     for (int b = threadIdx.x; b < nblk; b += kThreads) a += part[b];
     a = warp_sum(a);
@@ -391,9 +395,11 @@ __device__ __forceinline__ double sum_partials(const double* __restrict__ part, 
 // PASS 1: H[i][j], the coefficient of u_i, and from |w|^2 (i = j + 1) the rescale factor 1/|w|.
 // PASS 2 (right-hand sides with reflag): their corrections.
 template <int PASS>
-__global__ void __launch_bounds__(kThreads) project_kernel(GState s, const double2* __restrict__ partial, int nblk, int j) {
+__global__ void __launch_bounds__(kThreads) project_kernel(GState s, const double2* partial, int nblk, int j) {
     __shared__ double2 sh[kWarps];
     const int i = blockIdx.x, r = blockIdx.y, m = s.m, nv = j + 2;
+    grid_release();
+    grid_wait();
     if (PASS == 1 ? !s.active[r] : !s.reflag[r]) return;
     double2 a = make_double2(0, 0);
     for (int b = threadIdx.x; b < nblk; b += kThreads) {
@@ -439,9 +445,11 @@ __global__ void __launch_bounds__(kThreads) project_kernel(GState s, const doubl
 
 // after the first update: its squared norm, and the second pass where the rescaled new vector has squared
 // length below 1/2.  One block per right-hand side.
-__global__ void __launch_bounds__(kThreads) reorth_kernel(GState s, const double* __restrict__ npart, int nblk) {
+__global__ void __launch_bounds__(kThreads) reorth_kernel(GState s, const double* npart, int nblk) {
     __shared__ double sh[kWarps];
     const int r = blockIdx.x;
+    grid_release();
+    grid_wait();
     if (!s.active[r]) {
         if (threadIdx.x == 0) s.reflag[r] = 0;
         return;
@@ -457,13 +465,15 @@ __global__ void __launch_bounds__(kThreads) reorth_kernel(GState s, const double
 // End of step j, one block per right-hand side: the second update's squared norm where there was one, the
 // Givens rotations, and (the last block) the list of right-hand sides still active: out[0] their number, then their
 // indices in increasing order.
-__global__ void __launch_bounds__(kThreads) step_end_kernel(GState s, int R, const double* __restrict__ npart, int nblk,
+__global__ void __launch_bounds__(kThreads) step_end_kernel(GState s, int R, const double* npart, int nblk,
                                                             int j) {
     __shared__ double sh[kWarps];
     __shared__ double2 col[kMaxV], rs[kMaxV], ch[kMaxV];
     __shared__ double rc[kMaxV];
     __shared__ int last;
     const int r = blockIdx.x, m = s.m;
+    grid_release();
+    grid_wait();
     if (s.active[r]) {
         double2* H = s.H + (long long)r * (m + 1) * m;
         const int re = s.reflag[r];
@@ -763,20 +773,18 @@ struct Solver {
     template <int PASS, typename VC>
     int dots(const VC* U, long long ustride, const VC* w, int nvec) {
         const dim3 g1(nblk, R);
-        VIE_KLAUNCH("gs_dots", st,
-                    gs_dots_kernel<VC><<<g1, kThreads, 0, st>>>(U, ustride, w, n, nvec, partial, nblk,
-                                                               PASS == 1 ? gs.active : gs.reflag));
+        VIE_LAUNCH("gs_dots", st, 0.0, (gs_dots_kernel<VC>), g1, kThreads, 0, U, ustride, w, n, nvec, partial, nblk,
+                   PASS == 1 ? gs.active : gs.reflag);
         const dim3 g2(nvec + 1, R);
-        VIE_KLAUNCH("arnoldi_project", st, project_kernel<PASS><<<g2, kThreads, 0, st>>>(gs, partial, nblk, nvec - 1));
+        VIE_LAUNCH("arnoldi_project", st, 0.0, (project_kernel<PASS>), g2, kThreads, 0, gs, partial, nblk, nvec - 1);
         VIE_CHECK_LAUNCH();
         return VIE_OK;
     }
     template <typename VC>
     int update(const VC* U, long long ustride, VC* w, int nvec, const int* flag) {
         const dim3 g1(nblk, R);
-        VIE_KLAUNCH("gs_update", st,
-                    gs_update_kernel<VC><<<g1, kThreads, 0, st>>>(U, ustride, w, n, nvec, gs.coef, m + 1, gs.scale,
-                                                                 npart, nblk, flag));
+        VIE_LAUNCH("gs_update", st, 0.0, (gs_update_kernel<VC>), g1, kThreads, 0, U, ustride, w, n, nvec, gs.coef, m + 1,
+                   gs.scale, npart, nblk, flag);
         VIE_CHECK_LAUNCH();
         return VIE_OK;
     }
@@ -827,10 +835,10 @@ int enqueue_steps(Solver& S, VC* U, const double2* r64, const double* rn2, int p
                                    S.gs.nactive + 1, S.gs.nactive));
         VIE_TRY((S.dots<1, VC>(U, ustride, w, j + 1)));
         VIE_TRY(S.update<VC>(U, ustride, w, j + 1, S.gs.active));
-        VIE_KLAUNCH("arnoldi_reorth", st, reorth_kernel<<<R, kThreads, 0, st>>>(S.gs, S.npart, S.nblk));
+        VIE_LAUNCH("arnoldi_reorth", st, 0.0, (reorth_kernel), R, kThreads, 0, S.gs, S.npart, S.nblk);
         VIE_TRY((S.dots<2, VC>(U, ustride, w, j + 1)));
         VIE_TRY(S.update<VC>(U, ustride, w, j + 1, S.gs.reflag));
-        VIE_KLAUNCH("arnoldi_step_end", st, step_end_kernel<<<R, kThreads, 0, st>>>(S.gs, R, S.npart, S.nblk, j));
+        VIE_LAUNCH("arnoldi_step_end", st, 0.0, (step_end_kernel), R, kThreads, 0, S.gs, R, S.npart, S.nblk, j);
         VIE_CHECK_LAUNCH();
     }
     return VIE_OK;

@@ -62,9 +62,9 @@ __device__ __forceinline__ void collect_or(unsigned key, unsigned* dst) {
 // [R][nc][Nz][Ny][Nx], or [R][nc][ns] on a support (rows != NULL; zeros outside it).
 template <int L>
 __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
-    xy64_fwd_kernel(const double2* __restrict__ x, double2* __restrict__ w, int nx, int ny, int nz,
+    xy64_fwd_kernel(const double2* x, double2* w, int nx, int ny, int nz,
                     const int4* __restrict__ rows, long long ns, const unsigned char* __restrict__ cpos,
-                    const int4* __restrict__ twg, const int* __restrict__ rmap, MatvecEpi dc) {
+                    const int4* __restrict__ twg, const int* rmap, MatvecEpi dc) {
     using Cfg = XYCfg64<L>;
     constexpr int A = fft2::Split<L>::A, B = fft2::Split<L>::B, NT = Cfg::NT, RS = Cfg::RS, CW = Cfg::CW, H = Cfg::H;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -77,6 +77,8 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
     const int tid = threadIdx.x;
     const long long p = blockIdx.x;  // spectrum plane; the input plane is pin (rmap: active right-hand sides)
     const long long rplanes = (long long)dc.nc * nz;  // planes per right-hand side
+    grid_release();
+    grid_wait();
     if (dc.nact) {  // planes of right-hand sides beyond the device count are skipped
         const int cnt = *dc.nact;
         dev_bytes_add(dc.bctr, dc.bfix + dc.bper * cnt, cnt > 0);
@@ -219,7 +221,7 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
 // CONV: also the plane's (N - G) x at every voxel to epi.conv (full grid).
 template <int L, bool CONV>
 __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
-    xy64_inv_kernel(const double2* __restrict__ w, double2* __restrict__ y, MatvecEpi epi,
+    xy64_inv_kernel(const double2* w, double2* y, MatvecEpi epi,
                     const unsigned char* __restrict__ cpos, const int4* __restrict__ twg) {
     using Cfg = XYCfg64<L>;
     constexpr int A = fft2::Split<L>::A, B = fft2::Split<L>::B, NT = Cfg::NT, RS = Cfg::RS, CW = Cfg::CW, H = Cfg::H;
@@ -240,6 +242,8 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
     const long long p = blockIdx.x;  // spectrum plane (r * nc + alpha) * nz + z; output plane po
     const int nc = epi.nc;
     const long long rplanes = (long long)nc * nz;  // planes per right-hand side
+    grid_release();
+    grid_wait();
     if (epi.nact) {
         const int cnt = *epi.nact;
         dev_bytes_add(epi.bctr, epi.bfix + epi.bper * cnt, cnt > 0);
@@ -426,15 +430,14 @@ int launch_L(bool fwd, const char* name, double bytes, const vie_handle* h, cons
     const int4* tw = h->twfx + L;
     if (fwd) {
         VIE_CUDA(attr(xy64_fwd_kernel<L>));
-        VIE_KLAUNCH_B(name, s, bytes,
-                      xy64_fwd_kernel<L><<<planes, Cfg::NT, Cfg::smem, s>>>(in, out, nx, ny, h->nz, sp.rows, sp.ns, cpos,
-                                                                           tw, e.rmap, e));
+        VIE_LAUNCH(name, s, bytes, (xy64_fwd_kernel<L>), planes, Cfg::NT, Cfg::smem, in, out, nx, ny, h->nz, sp.rows,
+                   sp.ns, cpos, tw, e.rmap, e);
     } else if (e.conv) {
         VIE_CUDA(attr(xy64_inv_kernel<L, true>));
-        VIE_KLAUNCH_B(name, s, bytes, (xy64_inv_kernel<L, true><<<planes, Cfg::NT, Cfg::smem, s>>>(in, out, e, cpos, tw)));
+        VIE_LAUNCH(name, s, bytes, (xy64_inv_kernel<L, true>), planes, Cfg::NT, Cfg::smem, in, out, e, cpos, tw);
     } else {
         VIE_CUDA(attr(xy64_inv_kernel<L, false>));
-        VIE_KLAUNCH_B(name, s, bytes, (xy64_inv_kernel<L, false><<<planes, Cfg::NT, Cfg::smem, s>>>(in, out, e, cpos, tw)));
+        VIE_LAUNCH(name, s, bytes, (xy64_inv_kernel<L, false>), planes, Cfg::NT, Cfg::smem, in, out, e, cpos, tw);
     }
     VIE_CHECK_LAUNCH();
     return VIE_OK;

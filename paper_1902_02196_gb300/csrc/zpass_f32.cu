@@ -161,11 +161,13 @@ __global__ void __launch_bounds__(ZFCfg<LZ, TB_>::NT, ZFCfg<LZ, TB_>::MINB)
     float2* tw = sb + 2 * BUF;
     float2* gsec = tw + LZ;  // [NPAIR pairs][2 sets][NG] Green values of the item that holds kz = LZ/2
     const int tid = threadIdx.x;
+    grid_release();
+    if (z.nact) grid_wait();  // the count first: an empty list ends here
     const int R = z.nact ? min(*z.nact, z.R) : z.R;
     dev_bytes_add(z.bctr, 8.0 * (2.0 * R * 12 * z.nz * z.Ly * z.Lx + (double)NG * z.Ox * z.Oy * z.Oz),
                   R > 0 && blockIdx.y == 0);
     const int r0 = blockIdx.y, rstep = gridDim.y;  // this CTA's right-hand sides
-    if (r0 >= R) return;
+    if (r0 >= R) return;  // (only after the wait: without a count the grid has no such CTA)
     for (int m = tid; m < LZ; m += NT) tw[m] = twg[m];
     const int ntile = z.Lx / TB;
     const int py = blockIdx.x / ntile, ct = blockIdx.x % ntile, sc0 = ct * TB;
@@ -256,6 +258,7 @@ __global__ void __launch_bounds__(ZFCfg<LZ, TB_>::NT, ZFCfg<LZ, TB_>::MINB)
         }
     }
 
+    grid_wait();  // the tables above are older than any launch in flight; the spectrum is not
     issue(r0, sb);
     int odd = 0;
 #pragma unroll 1
@@ -345,8 +348,7 @@ static int launch_zf_LT(const vie_handle* h, const ZFArgs& z, cudaStream_t s, co
     const unsigned parts = (unsigned)std::min<long long>(z.R, std::max<long long>(1, (4 * places + blocks - 1) / blocks));
     // with a device count the kernel adds its bytes to z.bctr
     const double bytes = z.nact ? kDevCounted : 8.0 * (2.0 * z.R * 12 * z.nz * z.Ly * z.Lx + NG * z.Ox * z.Oy * z.Oz);
-    VIE_KLAUNCH_B(name, s, bytes,
-                  zfused_kernel<LZ, TB, KOP><<<dim3((unsigned)blocks, parts), Cfg::NT, smem, s>>>(z, h->tw32 + LZ));
+    VIE_LAUNCH(name, s, bytes, (zfused_kernel<LZ, TB, KOP>), dim3((unsigned)blocks, parts), Cfg::NT, smem, z, h->tw32 + LZ);
     VIE_CHECK_LAUNCH();
     return VIE_OK;
 }

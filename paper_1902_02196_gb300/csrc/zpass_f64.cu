@@ -198,6 +198,8 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     // the digits of the warp's next octant point, copied while the current one is multiplied
     uint4* gbuf = reinterpret_cast<uint4*>(kin + 32 * RB) + wid * (NG * 2);
+    grid_release();
+    if (z.nact) grid_wait();
     const int R = z.nact ? min(*z.nact, z.R) : z.R;
     dev_bytes_add(z.bctr, 16.0 * (2.0 * R * 12 * z.nz * z.Ly * z.Lx + (double)NG * z.Ox * z.Oy * z.Oz), R > 0);
     if (R <= 0) return;
@@ -244,6 +246,7 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
         cp_async_commit();
     };
     if (wid < nq) fetch(wid);
+    grid_wait();
 
 #pragma unroll 1
     for (int r0 = 0; r0 < R; r0 += RB) {
@@ -538,8 +541,8 @@ int launch_zd_L(const vie_handle* h, const ZDArgs& z, cudaStream_t s) {
     VIE_CUDA(cudaFuncSetAttribute(zfused64_kernel<LZ, KOP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const long long blocks = (long long)z.Ly * (z.Lx / 2);
     const double bytes = z.nact ? kDevCounted : 16.0 * (2.0 * z.R * 12 * z.nz * z.Ly * z.Lx + NG * z.Ox * z.Oy * z.Oz);
-    VIE_KLAUNCH_B(KOP ? "zpass_block_k_f64" : "zpass_block_f64", s, bytes,
-                  zfused64_kernel<LZ, KOP><<<(unsigned)blocks, ZDCfg<LZ>::NT, smem, s>>>(z, h->twfx + LZ));
+    VIE_LAUNCH(KOP ? "zpass_block_k_f64" : "zpass_block_f64", s, bytes, (zfused64_kernel<LZ, KOP>), (unsigned)blocks,
+               ZDCfg<LZ>::NT, smem, z, h->twfx + LZ);
     VIE_CHECK_LAUNCH();
     return VIE_OK;
 }

@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
     unsigned* kin = reinterpret_cast<unsigned*>(s + 3 * GS + LZ);  // [3] keys of the inputs, of the product, of pass 1
     unsigned *kout = kin + 3, *kmid = kin + 4;
     const int tid = threadIdx.x, lane = tid & 31;
+    grid_release();
     for (int m = tid; m < LZ; m += NT) {
         if constexpr (F64)
             twi[m] = twfx[m];
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
             twf[m] = tw32[m];
     }
     if (tid < 5) kin[tid] = 0;
+    grid_wait();
     __syncthreads();
     const int ntile = z.Lx / TB;
     const int py = blockIdx.x / ntile, sc0 = (blockIdx.x % ntile) * TB;
@@ -226,9 +228,8 @@ int launch_L(const vie_handle* h, const ZPArgs& z, cudaStream_t s) {
     // set on every call: the attribute is per device and launches may come from several threads
     VIE_CUDA(cudaFuncSetAttribute(zpwc_kernel<T, LZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::smem));
     const double bytes = (sizeof(T) == 8 ? 16.0 : 8.0) * (2.0 * z.R * 3 * z.nz * z.Ly * z.Lx + 6.0 * z.Ox * z.Oy * z.Oz);
-    VIE_KLAUNCH_B(sizeof(T) == 8 ? "zpass_block_pwc_f64" : "zpass_block_pwc_f32", s, bytes,
-                  (zpwc_kernel<T, LZ><<<(unsigned)(z.Ly * (z.Lx / Cfg::TB)), Cfg::NT, Cfg::smem, s>>>(z, h->tw32 + LZ,
-                                                                                                    h->twfx + LZ)));
+    VIE_LAUNCH(sizeof(T) == 8 ? "zpass_block_pwc_f64" : "zpass_block_pwc_f32", s, bytes, (zpwc_kernel<T, LZ>),
+               (unsigned)(z.Ly * (z.Lx / Cfg::TB)), Cfg::NT, Cfg::smem, z, h->tw32 + LZ, h->twfx + LZ);
     VIE_CHECK_LAUNCH();
     return VIE_OK;
 }
