@@ -16,10 +16,18 @@
 // A CTA owns one ky row and one mirror pair of stored columns, and loops over groups of four
 // right-hand sides (two for Lz = 512): 8 column lines per component in shared memory, slot
 // 2 rr + c for right-hand side rr of the group and column c.  Tile row r holds slot r % TB at
-// the item's first kz position (r < TB) or second (r >= TB).  The component stride is 4 mod 16
-// float2, so the fragment loads and stores of a half warp (4 slots x 4 components) hit 32
-// distinct banks.  The Green tensor is read as precomputed bf16 hi/lo pairs ([Oy][Ox][Oz][60]
-// of (hi, lo), each a bf16 (re, im) pair).
+// 2 rr + c for right-hand side rr of the group and column c.  Tile row r holds slot r % TB at
+// the point's kz (r < TB) or at its mirror (r >= TB).  A warp takes one octant point at a time,
+// and its 60 tensors come to a buffer of the warp while the point before is multiplied.  The
+// Green tensor is read as precomputed bf16 hi/lo pairs ([Oy][Ox][Oz][60] of (hi, lo), each a
+// bf16 (re, im) pair).
+//
+// Shared memory bounds the kernel: its wavefronts keep the load/store unit busy for two thirds
+// of the time, so the component stride is chosen for the transforms, which make eight of the
+// ten accesses to an element: TB float2 of padding put the two (TB = 8) or four (TB = 4)
+// components of a half warp on distinct banks.  With 4 for either, which is free of conflicts
+// in the fragments' accesses only, the kernel took 5.99 ms instead of 5.34 ms for 32 right-hand
+// sides on 64^3 voxels; before the buffered tensors and the signs taken out of the loop 6.09.
 #include <cuda_bf16.h>
 
 #include "block.cuh"
@@ -34,8 +42,8 @@ struct ZBCfg {
     static constexpr int TB = TB_;  // column lines per component: 2 columns x TB/2 right-hand sides (8 or 4)
     static constexpr int RG = TB / 2;             // right-hand sides per group
     static constexpr int NT = 256;
-    static constexpr int GS = LZ * TB + 4;  // component stride in float2, 4 mod 16
-    static constexpr size_t smem = sizeof(float2) * (size_t)(12 * GS + LZ);
+    static constexpr int GS = LZ * TB + TB;       // component stride in float2
+    static constexpr size_t smem = sizeof(float2) * (size_t)(12 * GS + LZ + (NT / 32) * 60);
     static constexpr int MINB = smem <= 110 * 1024 ? 2 : 1;
 };
 
@@ -67,7 +75,7 @@ template <int LZ, int TB_>
 __global__ void __launch_bounds__(256, ZBCfg<LZ, TB_>::MINB)
     zbf16_kernel(ZFArgs z, const uint2* __restrict__ gbf, const float2* __restrict__ twg) {
     using Cfg = ZBCfg<LZ, TB_>;
-    constexpr int A = fft2::Split<LZ>::A, B = fft2::Split<LZ>::B, NT = Cfg::NT, TB = Cfg::TB, RG = Cfg::RG;
+    constexpr int NT = Cfg::NT, TB = Cfg::TB, RG = Cfg::RG;
     constexpr int GS = Cfg::GS;
     constexpr int NWARP = NT / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -97,82 +105,89 @@ __global__ void __launch_bounds__(256, ZBCfg<LZ, TB_>::MINB)
     // after the optional (re, im) swap: the table sign on both halves, -Bi for a real output
     int tix[9];
     unsigned flp[9];
-    const bool swp = (g & 1) != 0;
+    const unsigned swp = (g & 1) ? 0x1032u : 0x3210u;
 #pragma unroll
     for (int nt = 0; nt < 3; ++nt)
 #pragma unroll
         for (int e = 0; e < 3; ++e) {
             const int a = 4 * nt + (g >> 1), b = e == 0 ? q : (e == 1 ? q + 4 : 8 + q);
             tix[3 * nt + e] = tensor_of(a, b);
-            flp[3 * nt + e] = (swp ? 0u : 0x80000000u) ^ (sign_of(a, b) < 0 ? 0x80008000u : 0u);
+            flp[3 * nt + e] = ((g & 1) ? 0u : 0x80000000u) ^ (sign_of(a, b) < 0 ? 0x80008000u : 0u);
         }
-    // tile rows of the lane: r0 = g and r1 = g + 8 (valid when r1 < 2 TB)
+    // tile rows of the lane: r0 = g and r1 = g + 8 (valid when r1 < 2 TB); rows from TB on are the mirrors in kz
     const bool r1ok = g + 8 < 2 * TB;
     const int slot0 = g % TB, slot1 = (g + 8) % TB;
-    const bool second0 = g >= TB, second1 = true;  // r1 = g + 8 >= TB for TB <= 8
+    const bool second0 = g >= TB;
     const int c0 = slot0 & 1, c1 = slot1 & 1;
+    // the reflections' signs of the rows' components q, q + 4 and 8 + q, inputs and outputs alike
+    unsigned sg0[3], sg1[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+        sg0[e] = sbit(fy ^ (c0 ? fx1 : fx0) ^ (second0 ? z.mz : 0u), q + 4 * e);
+        sg1[e] = sbit(fy ^ (c1 ? fx1 : fx0) ^ z.mz, q + 4 * e);
+    }
+    // octant points of this CTA, a warp each in turn: kz = 0..LZ/2, for each column where they are self-mirrored.
+    constexpr int NO = LZ / 2 + 1;
+    const int nq = xsplit ? 2 * NO : NO;
+    uint2* gbuf = reinterpret_cast<uint2*>(tw + LZ) + warp * 60;
+    auto fetch = [&](int p) {
+        const bool col = p >= NO;
+        const uint4* src = reinterpret_cast<const uint4*>(
+            gbf + (((long long)kyo * z.Ox + (col ? kxo1 : kxo0)) * z.Oz + (p - (col ? NO : 0))) * 60);
+        if (lane < 30) cp_async16(reinterpret_cast<uint4*>(gbuf) + lane, src + lane);
+        cp_async_commit();
+    };
+    if (warp < nq) fetch(warp);
+    // row e = a nz + l of a right-hand side's spectrum: component a = e / nz (e < 2^13, nz <= 512)
+    const unsigned nzq = 0xffffffffu / (unsigned)nz + 1u;
+    auto place = [&](int e) {
+        const int a = nz > 1 ? (int)__umulhi((unsigned)e, nzq) : e;
+        return a * (GS - nz * TB) + e * TB;
+    };
 
     auto line = [](int n) { return (n / TB) * GS + n % TB; };
 #pragma unroll 1
     for (int rb = 0; rb < R; rb += RG) {
         // loads: slot pair (2 rr, 2 rr + 1) of component a, plane l = 16 contiguous bytes
         for (int idx = tid; idx < 12 * nz * RG; idx += NT) {
-            const int rr = idx % RG, l = (idx / RG) % nz, a = idx / (RG * nz);
+            const int rr = idx % RG, e = idx / RG;
             const bool in = rb + rr < R;
-            const float2* src = in ? z.w + ((long long)(rb + rr) * 12 * nz + (long long)a * nz + l) * plane +
-                                         (long long)py * z.Lx + sc0
-                                   : z.w;
-            cp_async16z(s + a * GS + l * TB + 2 * rr, src, in ? 16 : 0);
+            const float2* src = in ? z.w + ((long long)(rb + rr) * 12 * nz + e) * plane + (long long)py * z.Lx + sc0 : z.w;
+            cp_async16z(s + place(e) + 2 * rr, src, in ? 16 : 0);
         }
         cp_async_commit();
         cp_async_wait<0>();
         __syncthreads();
         fft2::forward<LZ, NT>(s, 12 * TB, line, TB, tw, nz);
 #pragma unroll 1
-        for (int j = warp; j < LZ / 2; j += NWARP) {
-            // kz positions of item j (as in the FP32 kernel): pa with its mirror pb, or, for
-            // the item of kz = 0, the self-mirrored kz = LZ/2 at pc with its own octant point
-            constexpr int NREG = (A / 2 - 1) * B;
-            int pa, p1;
-            bool zsplit = false;
-            if (j < NREG) {
-                const int k1 = 1 + j / B, k2 = j % B;
-                pa = k2 + B * k1;
-                p1 = (B - 1 - k2) + B * (A - k1);
-            } else if (j < NREG + B / 2) {
-                const int k2 = j - NREG;
-                pa = k2 + B * (A / 2);
-                p1 = (B - 1 - k2) + B * (A / 2);
-            } else {
-                const int k2 = j - NREG - B / 2;
-                pa = k2;
-                p1 = k2 == 0 ? B / 2 : B - k2;
-                zsplit = k2 == 0;
+        for (int p = warp; p < nq; p += NWARP) {
+            const int col = p >= NO, ko = p - (col ? NO : 0);
+            const bool self = ko == 0 || ko == LZ / 2;  // no mirror
+            const int posa = fft2::tpos(LZ, ko), posb = fft2::tpos(LZ, ko ? LZ - ko : 0);
+            const int off0 = (second0 ? posb : posa) * TB + slot0, off1 = posb * TB + slot1;
+            const bool ok0 = !(second0 && self) && !(xsplit && c0 != col);
+            const bool ok1 = r1ok && !self && !(xsplit && c1 != col);
+            cp_async_wait<0>();
+            __syncwarp();
+            unsigned bh[9], bl[9];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                const uint2 v = gbuf[tix[e]];
+                bh[e] = __byte_perm(v.x, 0, swp) ^ flp[e];
+                bl[e] = __byte_perm(v.y, 0, swp) ^ flp[e];
             }
-            const int kza = fft2::freq_at(LZ, pa), kzb = fft2::freq_at(LZ, p1);
-            const int kzoa = kza <= LZ / 2 ? kza : LZ - kza, kzob = kzb <= LZ / 2 ? kzb : LZ - kzb;
-            const unsigned fza = kza > LZ / 2 ? z.mz : 0u, fzb = kzb > LZ / 2 ? z.mz : 0u;
-            // the lane's rows: position, reflection mask, Green group (octant point)
-            const int pos0 = second0 ? p1 : pa, pos1 = p1;
-            const unsigned m0 = fy ^ (c0 ? fx1 : fx0) ^ (second0 ? fzb : fza);
-            const unsigned m1 = fy ^ (c1 ? fx1 : fx0) ^ fzb;
-            const int grp0 = (zsplit && second0 ? 1 : 0) + (xsplit && c0 ? 2 : 0);
-            const int grp1 = (zsplit && second1 ? 1 : 0) + (xsplit && c1 ? 2 : 0);
+            __syncwarp();
+            fetch(p + NWARP < nq ? p + NWARP : warp);  // after the last one, the next group's first
             // A fragments: x^T rows r0, r1, inputs (re, im) of components q, q + 4 (k-tile 0) and 8 + q (k-tile 1)
             unsigned ah[2][4], al[2][4];
             {
-                const float2* x0 = s + pos0 * TB + slot0;
-                const float2* x1 = s + pos1 * TB + slot1;
-                const int comp[3] = {q, q + 4, 8 + q};
                 unsigned h[2][3], l[2][3];
 #pragma unroll
                 for (int e = 0; e < 3; ++e) {
-                    const int b = comp[e];
-                    split2(flip2(x0[b * GS], sbit(m0, b)), h[0][e], l[0][e]);
-                    if (r1ok)
-                        split2(flip2(x1[b * GS], sbit(m1, b)), h[1][e], l[1][e]);
-                    else
-                        h[1][e] = l[1][e] = 0u;
+                    const int b = (q + 4 * e) * GS;
+                    h[0][e] = l[0][e] = h[1][e] = l[1][e] = 0u;
+                    if (ok0) split2(flip2(s[b + off0], sg0[e]), h[0][e], l[0][e]);
+                    if (ok1) split2(flip2(s[b + off1], sg1[e]), h[1][e], l[1][e]);
                 }
                 // k-tile 0: a0 (r0, q), a1 (r1, q), a2 (r0, q + 4), a3 (r1, q + 4); k-tile 1: (., 8 + q), zero
                 ah[0][0] = h[0][0], ah[0][1] = h[1][0], ah[0][2] = h[0][1], ah[0][3] = h[1][1];
@@ -180,61 +195,39 @@ __global__ void __launch_bounds__(256, ZBCfg<LZ, TB_>::MINB)
                 ah[1][0] = h[0][2], ah[1][1] = h[1][2], ah[1][2] = 0u, ah[1][3] = 0u;
                 al[1][0] = l[0][2], al[1][1] = l[1][2], al[1][2] = 0u, al[1][3] = 0u;
             }
-            const int ngrp = (zsplit ? 2 : 1) * (xsplit ? 2 : 1);
-#pragma unroll 1
-            for (int gi = 0; gi < 4; ++gi) {
-                if (!((gi & 1) ? zsplit : true) || !((gi & 2) ? xsplit : true)) continue;
-                const int kxo = (gi & 2) ? kxo1 : kxo0, kzo = (gi & 1) ? kzob : kzoa;
-                const uint2* gp = gbf + (((long long)kyo * z.Ox + kxo) * z.Oz + kzo) * 60;
-                unsigned bh[9], bl[9];
+            float d[3][4];
 #pragma unroll
-                for (int e = 0; e < 9; ++e) {
-                    const uint2 v = __ldg(gp + tix[e]);
-                    const unsigned vh = swp ? __byte_perm(v.x, 0, 0x1032) : v.x;
-                    const unsigned vl = swp ? __byte_perm(v.y, 0, 0x1032) : v.y;
-                    bh[e] = vh ^ flp[e];
-                    bl[e] = vl ^ flp[e];
-                }
-                float d[3][4];
+            for (int nt = 0; nt < 3; ++nt) {
 #pragma unroll
-                for (int nt = 0; nt < 3; ++nt) {
+                for (int i = 0; i < 4; ++i) d[nt][i] = 0.f;
+                // small partial products first
+                mma_bf16(d[nt], al[0], bh[3 * nt], bh[3 * nt + 1]);
+                mma_bf16(d[nt], al[1], bh[3 * nt + 2], 0u);
+                mma_bf16(d[nt], ah[0], bl[3 * nt], bl[3 * nt + 1]);
+                mma_bf16(d[nt], ah[1], bl[3 * nt + 2], 0u);
+                mma_bf16(d[nt], ah[0], bh[3 * nt], bh[3 * nt + 1]);
+                mma_bf16(d[nt], ah[1], bh[3 * nt + 2], 0u);
+            }
+            // D rows r0 (d[.][0..1]) and r1 (d[.][2..3]): output component 4 nt + q, (re, im)
+            __syncwarp();
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) d[nt][i] = 0.f;
-                    // small partial products first
-                    mma_bf16(d[nt], al[0], bh[3 * nt], bh[3 * nt + 1]);
-                    mma_bf16(d[nt], al[1], bh[3 * nt + 2], 0u);
-                    mma_bf16(d[nt], ah[0], bl[3 * nt], bl[3 * nt + 1]);
-                    mma_bf16(d[nt], ah[1], bl[3 * nt + 2], 0u);
-                    mma_bf16(d[nt], ah[0], bh[3 * nt], bh[3 * nt + 1]);
-                    mma_bf16(d[nt], ah[1], bh[3 * nt + 2], 0u);
-                }
-                // D rows r0 (d[.][0..1]) and r1 (d[.][2..3]): output component 4 nt + q, (re, im)
-                if (ngrp == 1 || grp0 == gi) {
-#pragma unroll
-                    for (int nt = 0; nt < 3; ++nt) {
-                        const int a = 4 * nt + q;
-                        s[a * GS + pos0 * TB + slot0] = flip2(make_float2(d[nt][0], d[nt][1]), sbit(m0, a));
-                    }
-                }
-                if (r1ok && (ngrp == 1 || grp1 == gi)) {
-#pragma unroll
-                    for (int nt = 0; nt < 3; ++nt) {
-                        const int a = 4 * nt + q;
-                        s[a * GS + pos1 * TB + slot1] = flip2(make_float2(d[nt][2], d[nt][3]), sbit(m1, a));
-                    }
-                }
+            for (int nt = 0; nt < 3; ++nt) {
+                const int a = (4 * nt + q) * GS;
+                if (ok0) s[a + off0] = flip2(make_float2(d[nt][0], d[nt][1]), sg0[nt]);
+                if (ok1) s[a + off1] = flip2(make_float2(d[nt][2], d[nt][3]), sg1[nt]);
             }
         }
         __syncthreads();
         fft2::inverse<LZ, NT>(s, 12 * TB, line, TB, tw, nz);
         for (int idx = tid; idx < 12 * nz * RG; idx += NT) {
-            const int rr = idx % RG, l = (idx / RG) % nz, a = idx / (RG * nz);
+            const int rr = idx % RG, e = idx / RG;
             if (rb + rr >= R) continue;
-            float2* dst = z.w + ((long long)(rb + rr) * 12 * nz + (long long)a * nz + l) * plane + (long long)py * z.Lx + sc0;
-            *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(s + a * GS + l * TB + 2 * rr);
+            float2* dst = z.w + ((long long)(rb + rr) * 12 * nz + e) * plane + (long long)py * z.Lx + sc0;
+            *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(s + place(e) + 2 * rr);
         }
         __syncthreads();
     }
+    cp_async_wait<0>();
 }
 
 template <int LZ, int TB>
