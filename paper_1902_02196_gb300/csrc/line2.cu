@@ -1,4 +1,4 @@
-// Line transforms of the matvec's line path (Section IV-A on grids whose xy circulant is not
+// FP32 line transforms of the matvec's line path (Section IV-A on grids whose xy circulant is not
 // square or is longer than 128): the forward FFTs along x and along y and the inverse FFT along
 // y, TB lines to a CTA, each line in shared memory with the two-pass register FFT of fft2.cuh
 // (two passes through shared memory per transform instead of one per radix-4 stage).
@@ -28,20 +28,17 @@ struct Line2Cfg {
     static constexpr int NT0 = TB * B;
     static constexpr int NT = NT0 < 64 ? 64 : NT0;
     // shared memory: TB lines and the twiddles
-    template <typename C>
-    static constexpr size_t smem() {
-        return sizeof(C) * (size_t)(TB * LS + L);
-    }
+    static constexpr size_t smem = sizeof(float2) * (size_t)(TB * LS + L);
 };
 
 // KIND 0: forward (natural in, spectrum out in the stored order); 1: inverse (stored order in,
 // natural out, cropped).
 // colkx: stored position q holds frequency colkx[q] (the x transforms), or NULL: position q
 // holds transposed position q (the y transforms).
-template <typename T, int L, int KIND>
+template <int L, int KIND>
 __global__ void __launch_bounds__(Line2Cfg<L>::NT)
-    line2_kernel(LineArgs a, const int* __restrict__ colkx, const typename CT<T>::C* __restrict__ twg) {
-    using C = typename CT<T>::C;
+    line2_kernel(LineArgs a, const int* __restrict__ colkx, const float2* __restrict__ twg) {
+    using C = float2;
     using Cfg = Line2Cfg<L>;
     constexpr int TB = Cfg::TB, LS = Cfg::LS, NT = Cfg::NT;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -62,7 +59,7 @@ __global__ void __launch_bounds__(Line2Cfg<L>::NT)
         for (int idx = tid; idx < TB * a.n_in; idx += NT) {
             const int n = cin ? idx / a.n_in : idx % TB, l = cin ? idx % a.n_in : idx / TB;
             const int b = b0 + n;
-            s[off(n) + l] = b < a.nb ? in[ai * a.ia + (long long)l * a.il + (long long)b * a.ib] : mk(T(0), T(0));
+            s[off(n) + l] = b < a.nb ? in[ai * a.ia + (long long)l * a.il + (long long)b * a.ib] : make_float2(0.f, 0.f);
         }
         __syncthreads();
         fft2::forward<L, NT>(s, TB, off, 1, tw, a.n_in);
@@ -97,29 +94,17 @@ __global__ void __launch_bounds__(Line2Cfg<L>::NT)
     }
 }
 
-template <typename T>
-const typename CT<T>::C* twiddles(const vie_handle* h, int L);
-template <>
-const float2* twiddles<float>(const vie_handle* h, int L) {
-    return h->tw32 + L;
-}
-template <>
-const double2* twiddles<double>(const vie_handle* h, int L) {
-    return h->tw64 + L;
-}
-
-template <typename T, int L, int KIND>
+template <int L, int KIND>
 int launch_L(const char* name, const vie_handle* h, const LineArgs& a, const int* colkx, cudaStream_t s) {
-    using C = typename CT<T>::C;
     using Cfg = Line2Cfg<L>;
     // the two-pass transforms take at most L/2 non-zero inputs (forward) or outputs (inverse)
     if ((KIND == 0 ? a.n_in : a.n_out) > L / 2 || (KIND == 0 ? a.n_out : a.n_in) != L) {
         set_error("line transform: a line needs at most L/2 inputs and L outputs (forward), or the reverse");
         return VIE_EINVAL;
     }
-    constexpr size_t smem = Cfg::template smem<C>();
+    constexpr size_t smem = Cfg::smem;
     // set on every call: the attribute is per device and launches may come from several threads
-    VIE_CUDA(cudaFuncSetAttribute(line2_kernel<T, L, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    VIE_CUDA(cudaFuncSetAttribute(line2_kernel<L, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const long long blocks = (long long)a.na * ((a.nb + Cfg::TB - 1) / Cfg::TB);
     if (blocks <= 0) return VIE_OK;
     if (blocks > 0x7fffffffLL) {
@@ -127,23 +112,23 @@ int launch_L(const char* name, const vie_handle* h, const LineArgs& a, const int
         return VIE_EINVAL;
     }
     // algorithmic bytes: inputs read once, outputs written once
-    const double bytes = (double)sizeof(C) * (double)a.na * a.nb * (a.n_in + a.n_out);
+    const double bytes = (double)sizeof(float2) * (double)a.na * a.nb * (a.n_in + a.n_out);
     VIE_KLAUNCH_B(name, s, bytes,
-                  line2_kernel<T, L, KIND><<<(unsigned)blocks, Cfg::NT, smem, s>>>(a, colkx, twiddles<T>(h, L)));
+                  line2_kernel<L, KIND><<<(unsigned)blocks, Cfg::NT, smem, s>>>(a, colkx, h->tw32 + L));
     VIE_CHECK_LAUNCH();
     return VIE_OK;
 }
 
-template <typename T, int KIND>
+template <int KIND>
 int launch(const char* name, const vie_handle* h, int L, const LineArgs& a, const int* colkx, cudaStream_t s) {
     switch (L) {
-        case 8: return launch_L<T, 8, KIND>(name, h, a, colkx, s);
-        case 16: return launch_L<T, 16, KIND>(name, h, a, colkx, s);
-        case 32: return launch_L<T, 32, KIND>(name, h, a, colkx, s);
-        case 64: return launch_L<T, 64, KIND>(name, h, a, colkx, s);
-        case 128: return launch_L<T, 128, KIND>(name, h, a, colkx, s);
-        case 256: return launch_L<T, 256, KIND>(name, h, a, colkx, s);
-        case 512: return launch_L<T, 512, KIND>(name, h, a, colkx, s);
+        case 8: return launch_L<8, KIND>(name, h, a, colkx, s);
+        case 16: return launch_L<16, KIND>(name, h, a, colkx, s);
+        case 32: return launch_L<32, KIND>(name, h, a, colkx, s);
+        case 64: return launch_L<64, KIND>(name, h, a, colkx, s);
+        case 128: return launch_L<128, KIND>(name, h, a, colkx, s);
+        case 256: return launch_L<256, KIND>(name, h, a, colkx, s);
+        case 512: return launch_L<512, KIND>(name, h, a, colkx, s);
     }
     set_error("line transform: unsupported length " + std::to_string(L));
     return VIE_EINVAL;
@@ -153,12 +138,10 @@ int launch(const char* name, const vie_handle* h, int L, const LineArgs& a, cons
 
 bool line2_ok(int L) { return L >= 8 && L <= 512 && (L & (L - 1)) == 0; }
 
-int line2_forward(const char* name, const vie_handle* h, int L, bool fp64, const LineArgs& a, const int* colkx,
-                  cudaStream_t s) {
-    return fp64 ? launch<double, 0>(name, h, L, a, colkx, s) : launch<float, 0>(name, h, L, a, colkx, s);
+int line2_forward(const char* name, const vie_handle* h, int L, const LineArgs& a, const int* colkx, cudaStream_t s) {
+    return launch<0>(name, h, L, a, colkx, s);
 }
 
-int line2_inverse(const char* name, const vie_handle* h, int L, bool fp64, const LineArgs& a, const int* colkx,
-                  cudaStream_t s) {
-    return fp64 ? launch<double, 1>(name, h, L, a, colkx, s) : launch<float, 1>(name, h, L, a, colkx, s);
+int line2_inverse(const char* name, const vie_handle* h, int L, const LineArgs& a, const int* colkx, cudaStream_t s) {
+    return launch<1>(name, h, L, a, colkx, s);
 }

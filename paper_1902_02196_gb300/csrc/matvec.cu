@@ -543,14 +543,18 @@ static int launch_line(const char* name, const vie_handle* h, int L, const LineA
     switch (L) {
         case 2: return launch_line_L<T, 2, EPI>(name, h, a, e, s);
         case 4: return launch_line_L<T, 4, EPI>(name, h, a, e, s);
-        case 8: return launch_line_L<T, 8, EPI>(name, h, a, e, s);
-        case 16: return launch_line_L<T, 16, EPI>(name, h, a, e, s);
-        case 32: return launch_line_L<T, 32, EPI>(name, h, a, e, s);
-        case 64: return launch_line_L<T, 64, EPI>(name, h, a, e, s);
-        case 128: return launch_line_L<T, 128, EPI>(name, h, a, e, s);
-        case 256: return launch_line_L<T, 256, EPI>(name, h, a, e, s);
-        case 512: return launch_line_L<T, 512, EPI>(name, h, a, e, s);
         case 1024: return launch_line_L<T, 1024, EPI>(name, h, a, e, s);
+    }
+    if constexpr (sizeof(T) == 4 || !EPI) {  // the others with an epilogue in FP64: line_f64.cu
+        switch (L) {
+            case 8: return launch_line_L<T, 8, EPI>(name, h, a, e, s);
+            case 16: return launch_line_L<T, 16, EPI>(name, h, a, e, s);
+            case 32: return launch_line_L<T, 32, EPI>(name, h, a, e, s);
+            case 64: return launch_line_L<T, 64, EPI>(name, h, a, e, s);
+            case 128: return launch_line_L<T, 128, EPI>(name, h, a, e, s);
+            case 256: return launch_line_L<T, 256, EPI>(name, h, a, e, s);
+            case 512: return launch_line_L<T, 512, EPI>(name, h, a, e, s);
+        }
     }
     set_error("unsupported FFT length " + std::to_string(L));
     return VIE_EINVAL;
@@ -849,8 +853,8 @@ static int matvec_impl(vie_handle* h, int R, const void* x, void* y, int op, cud
         set_error("internal: the line-transform matvec takes full-grid vectors only");
         return VIE_EINVAL;
     }
-    // The line transforms: the two-pass kernels (line2.cu) for lengths 8..512, else the radix-4
-    // line kernels; the inverse x transform with the voxel-wise terms always on the radix-4 one.
+    // The line transforms: the two-pass kernels (line2.cu, FP64 line_f64.cu) for lengths 8..512, else the
+    // radix-4 line kernels; the FP32 inverse x transform with the voxel-wise terms always on the radix-4 one.
     // Both store the x spectrum in the column order of colkx32; the y spectrum's rows are in
     // fft2's transposed order after the two-pass kernel (row py holds ky = py / B + A (py % B),
     // A B = Ly) and in natural order after the radix-4 one.
@@ -867,7 +871,7 @@ static int matvec_impl(vie_handle* h, int R, const void* x, void* y, int op, cud
     a.n_in = nx, a.n_out = Lx, a.dir = -1;
     a.pout = h->colpos32;
     if (x2)
-        VIE_TRY(line2_forward(fp64 ? "fft_x_f64" : "fft_x_f32", h, Lx, fp64, a, h->colkx32, s));
+        VIE_TRY(fp64 ? line64_forward("fft_x_f64", h, Lx, a, h->colkx32, s) : line2_forward("fft_x_f32", h, Lx, a, h->colkx32, s));
     else
         VIE_TRY((launch_line<T, false>(fp64 ? "fft_x_f64" : "fft_x_f32", h, Lx, a, noepi, s)));
     // y-pass
@@ -880,7 +884,7 @@ static int matvec_impl(vie_handle* h, int R, const void* x, void* y, int op, cud
     a.oa = (long long)Ly * Lx, a.ol = Lx, a.ob = 1;
     a.n_in = ny, a.n_out = Ly, a.dir = -1;
     if (y2)
-        VIE_TRY(line2_forward(fp64 ? "fft_y_f64" : "fft_y_f32", h, Ly, fp64, a, nullptr, s));
+        VIE_TRY(fp64 ? line64_forward("fft_y_f64", h, Ly, a, nullptr, s) : line2_forward("fft_y_f32", h, Ly, a, nullptr, s));
     else
         VIE_TRY((launch_line<T, false>(fp64 ? "fft_y_f64" : "fft_y_f32", h, Ly, a, noepi, s)));
     // z-pass with block product: row order (ay, by) of the y spectrum, the natural order as
@@ -899,7 +903,8 @@ static int matvec_impl(vie_handle* h, int R, const void* x, void* y, int op, cud
     a.oa = (long long)ny * Lx, a.ol = Lx, a.ob = 1;
     a.n_in = Ly, a.n_out = ny, a.dir = +1;
     if (y2)
-        VIE_TRY(line2_inverse(fp64 ? "ifft_y_f64" : "ifft_y_f32", h, Ly, fp64, a, nullptr, s));
+        VIE_TRY(fp64 ? line64_inverse("ifft_y_f64", h, Ly, a, nullptr, nullptr, s)
+                     : line2_inverse("ifft_y_f32", h, Ly, a, nullptr, s));
     else
         VIE_TRY((launch_line<T, false>(fp64 ? "ifft_y_f64" : "ifft_y_f32", h, Ly, a, noepi, s)));
     // x-inverse (frequencies read from their stored columns) + crop + material/Gram terms
@@ -911,6 +916,7 @@ static int matvec_impl(vie_handle* h, int R, const void* x, void* y, int op, cud
     a.ia = 0, a.il = 1, a.ib = Lx;
     a.oa = 0, a.ol = 1, a.ob = nx;
     a.n_in = Lx, a.n_out = nx, a.dir = +1;
+    if (fp64 && x2) return line64_inverse("ifft_x_epilogue_f64", h, Lx, a, h->colkx32, &e, s);
     a.pin = h->colpos32;
     VIE_TRY((launch_line<T, true>(fp64 ? "ifft_x_epilogue_f64" : "ifft_x_epilogue_f32", h, Lx, a, e, s)));
     return VIE_OK;

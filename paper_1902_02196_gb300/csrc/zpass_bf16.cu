@@ -16,7 +16,6 @@
 // A CTA owns one ky row and one mirror pair of stored columns, and loops over groups of four
 // right-hand sides (two for Lz = 512): 8 column lines per component in shared memory, slot
 // 2 rr + c for right-hand side rr of the group and column c.  Tile row r holds slot r % TB at
-// 2 rr + c for right-hand side rr of the group and column c.  Tile row r holds slot r % TB at
 // the point's kz (r < TB) or at its mirror (r >= TB).  A warp takes one octant point at a time,
 // and its 60 tensors come to a buffer of the warp while the point before is multiplied.  The
 // Green tensor is read as precomputed bf16 hi/lo pairs ([Oy][Ox][Oz][60] of (hi, lo), each a
@@ -72,7 +71,7 @@ __device__ __forceinline__ void mma_bf16(float* d, const unsigned* a, unsigned b
 }
 
 template <int LZ, int TB_>
-__global__ void __launch_bounds__(256, ZBCfg<LZ, TB_>::MINB)
+__global__ void __launch_bounds__(ZBCfg<LZ, TB_>::NT, ZBCfg<LZ, TB_>::MINB)
     zbf16_kernel(ZFArgs z, const uint2* __restrict__ gbf, const float2* __restrict__ twg) {
     using Cfg = ZBCfg<LZ, TB_>;
     constexpr int NT = Cfg::NT, TB = Cfg::TB, RG = Cfg::RG;

@@ -112,6 +112,12 @@ def test_sizes_and_scales(vie, shape):
     h.close()
 
 
+# line transforms of every length (x, y): 32 x 64, 64 x 32, 128 x 256, 512 x 16, 16 x 512; a last CTA with lines to spare
+@pytest.mark.parametrize("shape", [(9, 20, 3), (32, 11, 2), (50, 128, 1), (200, 5, 3), (6, 256, 2)])
+def test_line_lengths(vie, shape):
+    test_sizes_and_scales(vie, shape)
+
+
 @pytest.mark.parametrize("shape", [(5, 6, 7), (3, 7, 20)])
 @pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
 def test_not_finite(vie, shape, value):
