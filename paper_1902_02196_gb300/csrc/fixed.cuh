@@ -141,5 +141,8 @@ __device__ __forceinline__ double fx_double(long long v, int ex) {
 }
 __device__ __forceinline__ double2 fx_double(fx2 v, int ex) { return make_double2(fx_double(v.x, ex), fx_double(v.y, ex)); }
 
-// v 2^-k, rounded down (the callers keep v at 56 bits or more)
-__device__ __forceinline__ fx2 fx_shift(fx2 v, int k) { return fx2{v.x >> k, v.y >> k}; }
+// v 2^-k, rounded to nearest
+__device__ __forceinline__ fx2 fx_shift(fx2 v, int k) {
+    const long long h = (1LL << k) >> 1;
+    return fx2{(v.x + h) >> k, (v.y + h) >> k};
+}

@@ -9,8 +9,8 @@
 // them, so that a rounding is 2^-56 of the plane's largest value or less, where FP64 rounds every
 // operation to 2^-53 of its own result.
 //
-// Measured, 16 right-hand sides on 64^3 voxels (12288 planes, 128 x 128 spectra): forward 3.1 ms and inverse
-// 4.6 ms, the FP64 kernels 11.2 and 13.1 ms.
+// Measured, 16 right-hand sides on 64^3 voxels (12288 planes, 128 x 128 spectra): forward 3.2 ms and inverse
+// 4.7 ms, the FP64 kernels 11.2 and 13.1 ms.
 //
 // A CTA owns one plane.  The x spectra of its rows stay in shared memory; the y transforms run on
 // chunks of CW stored columns, whose spectra go to or come from global memory in registers, 512
@@ -33,12 +33,6 @@ struct XYCfg64 {
     static constexpr size_t smem = sizeof(fx2) * (size_t)(L * CW + H * RS + L) + sizeof(int4) * H + 2 * L + 128;
 };
 
-// after a pass whose inputs had room for it, |v| <= 2^60.5: bits that the next pass, of n points, has
-// to drop if any value needs it (0 or log2 n + 1); the decision is the CTA's, and a barrier
-template <int N>
-__device__ __forceinline__ int rescale(unsigned key) {
-    return __syncthreads_or(fx_bits(key) > fx_room(N)) ? fx_log2(N) + 1 : 0;
-}
 __device__ __forceinline__ fx2 down(fx2 v, int k) {  // v 2^-k to nearest, k uniform
     if (k) {
         const long long h = 1LL << (k - 1);
@@ -58,6 +52,15 @@ __device__ __forceinline__ void collect_or(unsigned key, unsigned* dst) {
     if ((threadIdx.x & 31) == 0) atomicOr(dst, key);
 }
 
+// after a pass whose inputs had room for it, |v| <= 2^60.5: bits that the next pass, of N points, has to drop.
+// The CTA's decision, by *slot (zeroed before, used once); ends with a barrier.
+template <int N>
+__device__ __forceinline__ int rescale(unsigned key, unsigned* slot) {
+    collect_or(key, slot);
+    __syncthreads();
+    return max(fx_bits(*slot) - fx_room(N), 0);
+}
+
 // Forward: plane (r, alpha, z) of x -> W2 plane [Ly][Lx] (transposed ky, stored kx).  x is
 // [R][nc][Nz][Ny][Nx], or [R][nc][ns] on a support (rows != NULL; zeros outside it).
 template <int L>
@@ -73,7 +76,8 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
     int4* tw = reinterpret_cast<int4*>(xr + H * RS);
     int4* rw = tw + L;  // [H] support rows of this plane
     unsigned char* pos = reinterpret_cast<unsigned char*>(rw + H);
-    unsigned* keys = reinterpret_cast<unsigned*>(pos + 2 * L);  // of the input, of the x spectra
+    // of the input, of the x spectra, after the first x pass, after the first y pass of each chunk
+    unsigned* keys = reinterpret_cast<unsigned*>(pos + 2 * L);
     const int tid = threadIdx.x;
     const long long p = blockIdx.x;  // spectrum plane; the input plane is pin (rmap: active right-hand sides)
     const long long rplanes = (long long)dc.nc * nz;  // planes per right-hand side
@@ -88,7 +92,7 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
         tw[m] = twg[m];
         pos[m] = cpos[m];
     }
-    if (tid < 2) keys[tid] = 0;
+    if (tid < 3 + Cfg::NCH) keys[tid] = 0;
     const long long pin = rmap ? (long long)rmap[p / rplanes] * rplanes + p % rplanes : p;
     const double2* src = x + pin * (long long)ny * nx;
     if (rows) {
@@ -149,7 +153,7 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
             key |= fx_key(v[k1]);
         }
     }
-    int k = rescale<B>(key);
+    int k = rescale<B>(key, keys + 2);
     ex += k;
     key = 0;
     for (int t = tid; t < H * A; t += NT) {
@@ -198,7 +202,7 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
                 key |= fx_key(v[q]);
             }
         }
-        k = rescale<B>(key);
+        k = rescale<B>(key, keys + 3 + c0 / CW);
         for (int t = tid; t < CW * A; t += NT) {
             const int c = t % CW, k1 = t / CW;
             const fx2* ln = ck + B * k1 * CW + c;
@@ -233,10 +237,12 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
     int4* rw = tw + L;
     unsigned char* pos = reinterpret_cast<unsigned char*>(rw + H);
     unsigned char* chunk_of = pos + L;  // chunk of an x-transform position
-    // per chunk: the key of its spectrum, the key of its y-transformed rows, their exponent
+    // per chunk: the key of its spectrum, the key of its y-transformed rows, their exponent, the key after its first
+    // pass; the key after the first x pass
     unsigned* kin = reinterpret_cast<unsigned*>(pos + 2 * L);
     unsigned* kout = kin + NCH;
     int* cex = reinterpret_cast<int*>(kout + NCH);
+    unsigned* kmid = kout + 2 * NCH;
     const int tid = threadIdx.x;
     const int nx = epi.nx, ny = epi.ny, nz = epi.nz;
     const long long p = blockIdx.x;  // spectrum plane (r * nc + alpha) * nz + z; output plane po
@@ -254,7 +260,7 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
         pos[m] = cpos[m];
         chunk_of[cpos[m]] = (unsigned char)(m / CW);
     }
-    if (tid < 2 * NCH) kin[tid] = 0;
+    if (tid < 4 * NCH + 1) kin[tid] = 0;
     const long long po = epi.rmap ? (long long)epi.rmap[p / rplanes] * rplanes + p % rplanes : p;
     if (epi.rows)
         for (int yy = tid; yy < ny; yy += NT) rw[yy] = epi.rows[(p % nz) * ny + yy];
@@ -298,7 +304,7 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
                 key |= fx_key(v[b]);
             }
         }
-        const int k = rescale<A>(key);
+        const int k = rescale<A>(key, kmid + h);
         // pass 2: rows y < Ny scattered to the x-transform buffer at the column's x position
         key = 0;
         for (int t = tid; t < CW * B; t += NT) {
@@ -365,7 +371,7 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
             key |= fx_key(v[b]);
         }
     }
-    const int k = rescale<A>(key);
+    const int k = rescale<A>(key, kmid + NCH);
     ex += k;
     for (int t = tid; t < H * B; t += NT) {
         const int n = t % H, b = t / H;
