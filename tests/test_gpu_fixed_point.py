@@ -171,3 +171,52 @@ def test_pwc_sizes_and_scales(vie, shape):
     assert not np.any(np.isfinite(bad[0])) and np.array_equal(bad[1:], got[1:])
     h12.close()
     h3.close()
+
+
+# FFT lengths along z 8, 16, 32, 64 and 64: the FP32 z pass deals the right-hand sides of small spectra to several
+# CTAs and an item's points to idle threads
+@pytest.mark.parametrize("shape", [(4, 4, 4), (5, 4, 8), (10, 9, 12), (16, 13, 20), (6, 30, 32)])
+@pytest.mark.parametrize("op", ["NSCAT", "K"])
+def test_fp32_small_spectra(vie, shape, op):
+    """Each of 9 right-hand sides bitwise as alone, and within 2e-6 (some tens of FP32 roundings) of FP64."""
+    nx, ny, nz = shape
+    h = vie.vie_setup((nx, ny, nz, 0.01, 0.01, 0.01), 3e8, np.full((nz, ny, nx), 4.0), np.zeros((nz, ny, nx)))
+    rng = np.random.default_rng(8)
+    x = torch.from_numpy(rng.standard_normal((9, 12, nz, ny, nx)) + 1j * rng.standard_normal((9, 12, nz, ny, nx))).cuda()
+    x = x.to(torch.complex64).to(torch.complex128)
+    torch.cuda.synchronize()
+    opc = getattr(vie, "VIE_OP_" + op)
+    y64 = torch.empty_like(x)
+    vie.vie_matvec(h, x, y64, vie.VIE_FP64, opc)
+    x32 = x.to(torch.complex64)
+    torch.cuda.synchronize()
+    y32 = torch.empty_like(x32)
+    vie.vie_matvec(h, x32, y32, vie.VIE_FP32, opc)
+    for r in range(9):
+        alone = torch.empty_like(x32[:1])
+        vie.vie_matvec(h, x32[r:r + 1], alone, vie.VIE_FP32, opc)
+        torch.cuda.synchronize()  # the calls return before the device is done
+        assert torch.equal(alone[0], y32[r])
+        assert torch.linalg.vector_norm(y32[r] - y64[r]) <= 2e-6 * torch.linalg.vector_norm(y64[r])
+    h.close()
+
+
+@pytest.mark.parametrize("restart", [1, 2, 31, 33, 128])
+def test_restart_lengths(vie, restart):
+    """The triangular solve and the rotations at their smallest and largest sizes, and around a warp's: the residual
+    of the returned x, formed here with the FP64 operator, is the one asked for (1e-10, with 1 % for its own rounding)."""
+    n = 6
+    rng = np.random.default_rng(9)
+    h = vie.vie_setup((n, n, n, 0.01, 0.01, 0.01), 3e8, 1.0 + rng.random((n, n, n)), np.zeros((n, n, n)))
+    b = torch.from_numpy(rng.standard_normal((3, 12, n, n, n)) + 1j * rng.standard_normal((3, 12, n, n, n))).cuda()
+    x = torch.zeros_like(b)
+    rc, info = vie.vie_solve(h, b, x, tol=1e-10, restart=restart, maxit=400, mode=vie.VIE_SOLVE_FP64, true_resid=True)
+    assert rc == vie.VIE_OK, info
+    ax = torch.empty_like(b)
+    vie.vie_matvec(h, x, ax, vie.VIE_FP64, vie.VIE_OP_A)
+    torch.cuda.synchronize()
+    for r in range(3):
+        true = (torch.linalg.vector_norm(b[r] - ax[r]) / torch.linalg.vector_norm(b[r])).item()
+        assert info[r]["resid"] <= 1e-10
+        assert abs(true - info[r]["true_resid"]) <= 0.01 * true
+    h.close()
