@@ -93,7 +93,7 @@ typedef struct {
  * vie_setup -- build a handle for one grid, frequency and dielectric map.
  * Computes on the GPU, in FP64: the Galerkin entries of N for every offset
  * (Section III-C, Eq. 25, Eq. 34, Eq. 42-43), their circulant embedding and 3-D
- * FFT (Section IV-A), stored once in FP64 and once in FP32; and the per-voxel
+ * FFT (Section IV-A), stored in FP64, FP32 and split digits; and the per-voxel
  * material coefficients eps, chi = eps - 1, tau = chi/eps (Eq. 7, Eq. 17, Eq. 29).
  *   grid          : voxel counts and sizes (see above)
  *   freq_hz       : frequency f > 0; omega = 2 pi f, k0 = omega / c0
@@ -146,8 +146,8 @@ void vie_destroy(vie_handle* h);
  *   precision : VIE_FP64, VIE_FP32 or VIE_BF16X3 (VIE_OP_K: VIE_FP64 or VIE_FP32)
  *   op        : VIE_OP_A, VIE_OP_PA, VIE_OP_NSCAT or VIE_OP_K.  VIE_OP_K transforms the 30
  *               tensors of vie_green_toeplitz_k once per handle into octant spectra (30 Ox Oy Oz
- *               values in FP64 and FP32, each in two layouts: 48 bytes per value in all, kept
- *               until vie_destroy and counted by vie_info) and runs
+ *               values in FP64, in FP32 in two layouts and as digits of 32 bytes: 64 bytes per value
+ *               in all, kept until vie_destroy and counted by vie_info) and runs
  *               the same transforms as the N operator with the K block (96 signed entries) at
  *               every frequency point, the other octants from the K parities.
  */
@@ -236,7 +236,7 @@ int vie_rhs_dipoles(vie_handle* h, int nrhs, const double* pos, const double* mo
  * Each restart cycle runs on the device without host round trips: the Arnoldi steps work on a
  * device list of the right-hand sides still above their target, and the host reads the list
  * once per cycle.  On a stream other than the legacy or per-thread default stream, the cycle is
- * captured once per solve as a CUDA graph (m Arnoldi steps of about 15 kernels each) and replayed.
+ * captured once per solve as a CUDA graph (m Arnoldi steps of about 11 kernels each) and replayed.
  * Where chi, b and the guess all vanish (air), the rows of P^-1 A are the identity and
  * the solution is zero; the solver's vectors cover only each grid row's span of the
  * other voxels (the whole grid when that span covers it), so air costs no iterations'
