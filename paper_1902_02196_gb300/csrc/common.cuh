@@ -118,7 +118,7 @@ struct vie_handle {
     // FP32 copy in the layout of the z pass of the FP32 three-kernel path: [Oy][Ox][Oz][60]
     float2* green32t;
     // the FP64 values' digits for the FP64 fused z pass (zpass_f64.cu): per octant point and tensor seven
-    // 9-bit digits as fp16 (re, im) pairs, [Oy][Ox][Oz][60][2], then the exponent of each column [Oy][Ox]
+    // 9-bit digits as fp16 (re, im) pairs and a word with the point's exponent, [Oy][Ox][Oz][60][2]
     // (PWL handles with an FFT length along z of 8..512, else null)
     uint4* green_d;
     // the 30 K tensors' transformed circulants, octant storage [30][Oz][Oy][Ox], scaled by

@@ -604,7 +604,7 @@ static bool zfused_ok(const vie_handle* h) { return h->L[2] >= 8 && h->L[2] <= 5
 
 size_t green_digit_bytes(const vie_handle* h, int ng) {
     if (h->nc != 12 || !zfused_ok(h)) return 0;
-    return 2 * sizeof(uint4) * ng * (size_t)h->O[0] * h->O[1] * h->O[2] + sizeof(int) * (size_t)h->O[0] * h->O[1];
+    return 2 * sizeof(uint4) * ng * (size_t)h->O[0] * h->O[1] * h->O[2];
 }
 
 // FP32 kernels (the FP64 ones are in xy_f64.cu)
@@ -754,7 +754,6 @@ static int matvec_impl(vie_handle* h, int R, const void* x, void* y, int op, cud
                 ZDArgs z{};
                 z.w = reinterpret_cast<double2*>(W2);
                 z.green_d = h->kgreen_d;
-                z.gexp = digit_exponents(h, 30, h->kgreen_d);
                 z.colkx = h->colkx32;
                 z.R = Rs, z.nz = nz, z.Lx = Lx, z.Ly = Ly;
                 z.Ox = h->O[0], z.Oy = h->O[1], z.Oz = h->O[2];
@@ -822,7 +821,6 @@ static int matvec_impl(vie_handle* h, int R, const void* x, void* y, int op, cud
             ZDArgs z{};
             z.w = reinterpret_cast<double2*>(W2);
             z.green_d = h->green_d;
-            z.gexp = digit_exponents(h, 60, h->green_d);
             z.colkx = h->colkx32;
             z.R = Rs, z.nz = nz, z.Lx = Lx, z.Ly = Ly;
             z.Ox = h->O[0], z.Oy = h->O[1], z.Oz = h->O[2];

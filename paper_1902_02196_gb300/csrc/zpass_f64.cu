@@ -8,22 +8,28 @@
 // scaled integers (fixed.cuh) and on the tensor cores:
 //  - a CTA owns one ky row and one mirror pair of columns and loops over groups of RB right-hand
 //    sides, 24 RB lines in shared memory.  The two lines of a component share one power-of-two
-//    scale, taken from their largest element, and the transforms are those of fft2.cuh on 64-bit
-//    integers;
+//    scale, taken from their largest element and again before the second pass, and the transforms are
+//    those of fft2.cuh on 64-bit integers;
 //  - the block product is exact up to its last digits: with X the spectrum and B the block in 62
 //    bits below their largest values (the digit tables of green_digits), both are cut into seven
 //    signed 9-bit digits, X = sum_i x_i 2^(9(6-i)), and the products of digits with i + j <= 6 are
 //    summed by fp16 mma.sync into FP32, where every sum is an integer below 2^22 and so exact (the
 //    splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012).  The dropped digits
 //    are 2^-59 of the product, where FP64 rounds its operands and every sum to 2^-53;
+//  - B has an exponent per octant point, and X the one that goes with it, so that a unit of the product is 2^-58 of the
+//    largest product of the two at any one point (not of X's largest value times B's, which a smooth
+//    field has at different kz); a component of the product is then scaled by its own largest value.  With one exponent per
+//    column and one for all twelve components the linear components of smooth fields came out up to twelve
+//    times further off than from the FP64 kernel (8 x 7 x 200 voxels);
 //  - the accumulators start at 1.5 2^23, so that their bit patterns are the integers and no
 //    conversion instruction (16 per clock) is needed.
 //
-// Measured, 16 right-hand sides on 64^3 voxels (Lx = Ly = Lz = 128): 15.3 ms, the FP64 kernel of the same
-// structure 70.8 ms; the K block of 8 right-hand sides 6.5 ms against 29.1 ms.  The bound is instruction
-// issue: 260 warp instructions per frequency point, half of them the product (digits, sums, recombination).
-// The matvec's 2-norm error against long double sums is 0.5 to 0.8 times that with the FP64 kernels; the linear
-// components alone reach 1.3 times it where the inputs are dominated by their mean.
+// Measured, 16 right-hand sides on 64^3 voxels (Lx = Ly = Lz = 128): 15.8 ms, the FP64 kernel of the same
+// structure 70.8 ms; the K block of 8 right-hand sides 6.9 ms against 29.1 ms.
+//
+// What the integers do not keep: FP64 holds 53 bits of every value, here a value has 58 bits below the largest of its
+// line and of the twelve components at its point.  A component a million times weaker than the strongest
+// of its right-hand side, in an output that the strong one does not reach, loses 20 of them.
 //
 // Roles in the mma: the 24 x 24 real form of B (rows re, im of the outputs; columns re, im of the
 // inputs) is the 16-row operand, the points that share an octant point, +-kx, +-kz and RB = 2
@@ -44,8 +50,9 @@ constexpr unsigned kMagicBits = 0x4B400000u;  // 1.5 2^23
 // 256 in each digit: makes them 0..511 in a plain bit field
 constexpr unsigned long long kBias =
     256ull * ((1ull << 54) + (1ull << 45) + (1ull << 36) + (1ull << 27) + (1ull << 18) + (1ull << 9) + 1);
+constexpr int kLow = -100000;  // below every exponent
 constexpr int kBits = 62;   // |X|, |B| < 2^62
-constexpr int kShift = 68;  // Y = X B 2^-68: |Y| < 24 2^(62 + 62 - 68) < 2^61
+constexpr int kShift = 66;  // Y = X B 2^-66: |Y| < 24 2^(62 + 62 - 66) < 2^63
 
 template <int LZ>
 struct ZDCfg {
@@ -54,7 +61,10 @@ struct ZDCfg {
     static constexpr int NT = LZ <= 8 ? 96 : (LZ <= 128 ? 192 : 384);
     static constexpr int MINB = LZ <= 128 ? 2 : 1;
     static constexpr int GS = 2 * LZ + 2;  // component stride: four components and two columns on distinct banks
-    static constexpr size_t smem = sizeof(fx2) * (size_t)(RB * 12 * GS + LZ) + 4 * 32 * RB + (size_t)(NT / 32) * 60 * 32;
+    static constexpr int KEYS = 64 * RB;  // words for the keys
+    static constexpr int NTW = (fft2::Split<LZ>::A - 1) * (fft2::Split<LZ>::B - 1) + 1;  // twiddles in use
+    static constexpr size_t smem = sizeof(fx2) * (size_t)(RB * 12 * GS + NTW) + sizeof(int) * KEYS +
+                                   (size_t)(NT / 32) * 60 * 32 + sizeof(short) * 2 * (LZ / 2 + 2);
 };
 
 __device__ __forceinline__ void mma16(float* c, unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
@@ -133,26 +143,26 @@ __device__ __forceinline__ void block_digits(const unsigned (&a)[3][3][kD], cons
     int s[6], low[6];
     digit_sums<0>(a, b, s, h, g);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) y[q] = (long long)s[q] << 40;
+    for (int q = 0; q < 6; ++q) y[q] = (long long)s[q] << 42;
     digit_sums<1>(a, b, s, g, h);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) y[q] += (long long)s[q] << 31;
+    for (int q = 0; q < 6; ++q) y[q] += (long long)s[q] << 33;
     digit_sums<2>(a, b, s, h, g);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) y[q] = fx_mad(s[q], 1 << 22, y[q]);
+    for (int q = 0; q < 6; ++q) y[q] = fx_mad(s[q], 1 << 24, y[q]);
     digit_sums<3>(a, b, s, g, h);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) y[q] = fx_mad(s[q], 1 << 13, y[q]);
+    for (int q = 0; q < 6; ++q) y[q] = fx_mad(s[q], 1 << 15, y[q]);
     digit_sums<4>(a, b, s, h, g);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) low[q] = s[q] * 16;
+    for (int q = 0; q < 6; ++q) low[q] = s[q] * 64;
     digit_sums<5>(a, b, s, g, h);
     int t5[6];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) t5[q] = s[q] + 16;
+    for (int q = 0; q < 6; ++q) t5[q] = s[q] + 4;
     digit_sums<6>(a, b, s, h, g);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) y[q] += low[q] + ((t5[q] + ((s[q] + 256) >> 9)) >> 5);
+    for (int q = 0; q < 6; ++q) y[q] += low[q] + ((t5[q] + ((s[q] + 256) >> 9)) >> 3);
 }
 
 // Digits of one complex value as fp16 pairs (re, im), most significant first: w = v 2^sh + bias,
@@ -178,6 +188,9 @@ __device__ __forceinline__ void split_digits(fx2 v, int sh, __half2 sg, unsigned
     }
 }
 
+// bits that values with these keys have to drop before a pass of n points
+__device__ __forceinline__ int excess(unsigned key, int n) { return max(fx_bits(key) - fx_room(n), 0); }
+
 __device__ __forceinline__ int pos_of(int L, int k) { return fft2::tpos(L, k); }
 
 template <int LZ, bool KOP>
@@ -186,26 +199,33 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
     using Cfg = ZDCfg<LZ>;
     constexpr int NG = KOP ? 30 : 60;  // tensors per octant point
     constexpr int A = fft2::Split<LZ>::A, B = fft2::Split<LZ>::B, NT = Cfg::NT, RB = Cfg::RB, GS = Cfg::GS, NL = Cfg::NL;
-    // bits of the inputs of the forward transform, and of the two passes of the inverse one
-    constexpr int TF = fx_room(LZ / 2), TI1 = fx_room(B), TI2 = fx_room(A);
+    // bits of the inputs of the two passes of the forward transform, and of the inverse one
+    constexpr int TF1 = fx_room(A / 2), TF2 = fx_room(B), TI1 = fx_room(B);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fx2* s = reinterpret_cast<fx2*>(smem_raw);
     int4* tw = reinterpret_cast<int4*>(s + RB * 12 * GS);
-    // largest elements (fx_key): [RB][12] of the inputs and of the spectrum of each component, [RB] of the
-    // product and after the inverse's first pass; [RB] the exponent of X, [RB] Inf or NaN among the inputs
-    unsigned* kin = reinterpret_cast<unsigned*>(tw + LZ);
-    unsigned *kspec = kin + 12 * RB, *kout = kspec + 12 * RB, *kmid = kout + RB;
-    int *xexp = reinterpret_cast<int*>(kmid + RB), *bad = xexp + RB;
+    // per right-hand side and component: keys of the inputs, after the first forward pass, of the product and after the
+    // first inverse pass; the spectrum's exponent; per right-hand side the product's exponent in both
+    // columns, and Inf or NaN among the inputs
+    unsigned* kin = reinterpret_cast<unsigned*>(tw + Cfg::NTW);
+    unsigned *kfwd = kin + 12 * RB, *kout = kfwd + 12 * RB, *kmid = kout + 12 * RB;
+    int *sex = reinterpret_cast<int*>(kmid + 12 * RB), *pex = sex + 12 * RB, *bad = pex + 2 * RB;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     // the digits of the warp's next octant point, copied while the current one is multiplied
-    uint4* gbuf = reinterpret_cast<uint4*>(kin + 32 * RB) + wid * (NG * 2);
+    uint4* gbuf = reinterpret_cast<uint4*>(kin + Cfg::KEYS) + wid * (NG * 2);
+    // exponents of B at the octant points of the two columns
+    short* bex = reinterpret_cast<short*>(reinterpret_cast<uint4*>(kin + Cfg::KEYS) + NT / 32 * 60 * 2);
     grid_release();
     if (z.nact) grid_wait();
     const int R = z.nact ? min(*z.nact, z.R) : z.R;
     dev_bytes_add(z.bctr, 16.0 * (2.0 * R * 12 * z.nz * z.Ly * z.Lx + (double)NG * z.Ox * z.Oy * z.Oz), R > 0);
     if (R <= 0) return;
-    for (int m = tid; m < LZ; m += NT) tw[m] = twg[m];
-    if (tid < 26 * RB) kin[tid] = 0;
+    for (int m = tid; m < Cfg::NTW; m += NT) tw[m] = twg[m];
+    auto reset = [&] {
+        for (int i = tid; i < 48 * RB; i += NT) kin[i] = 0;
+        if (tid < 2 * RB) pex[tid] = kLow;
+    };
+    reset();
     __syncthreads();
     const int ntile = z.Lx / 2;
     const int py = blockIdx.x / ntile, ct = blockIdx.x % ntile, sc0 = 2 * ct;
@@ -221,7 +241,6 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
     const int kxo0 = kx0 <= z.Lx / 2 ? kx0 : z.Lx - kx0, kxo1 = kx1 <= z.Lx / 2 ? kx1 : z.Lx - kx1;
     const unsigned fx0 = kx0 > z.Lx / 2 ? z.mx : 0u, fx1 = kx1 > z.Lx / 2 ? z.mx : 0u;
     const int gc0 = kyo * z.Ox + kxo0, gc1 = kyo * z.Ox + kxo1;
-    const int gex0 = z.gexp[gc0], gex1 = z.gexp[gc1];
 
     // block-product roles of this lane.  Points (mma columns) 0..7: bit 0 the column, bit 1 the sign of
     // kz, bit 2 the right-hand side; n is the point whose X this lane splits, components t, t + 4, t + 8.
@@ -237,8 +256,15 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
     const unsigned bsel = part ? 0x1032u : 0x3210u;
     const unsigned bneg = (part ? 0u : 0x80000000u) ^ (swapneg ? 0x80008000u : 0u);
 
+    // exponents of the points, and the raises of the two columns' linear functions (the last word of tensor 0)
+    constexpr int NO = LZ / 2 + 1;
+    auto point_word = [&](int c, int ko) {
+        return reinterpret_cast<const int*>(z.green_d)[(((long long)(c ? gc1 : gc0) * z.Oz + ko) * NG + 1) * 8 - 1];
+    };
+    for (int i = tid; i < 2 * NO; i += NT) bex[i] = (short)(point_word(i / NO, i % NO) >> 8);
+    const int up0 = point_word(0, 0) & 255, up1 = point_word(1, 0) & 255;
     // octant points q of this CTA: 0..LZ/2, for each column when the columns are self-mirrored
-    constexpr int NO = LZ / 2 + 1, NW = NT / 32;
+    constexpr int NW = NT / 32;
     const int nq = single ? 2 * NO : NO;
     auto fetch = [&](int q) {
         const bool col = q >= NO;
@@ -284,7 +310,7 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
         for (int w = tid; w < NL * B; w += NT) {
             const int ln = w % NL, b = w / NL, rr = ln / 24;
             if (RB > 1 && rr >= nr) continue;
-            const FxScale sc(kin[ln >> 1], TF);
+            const FxScale sc(kin[ln >> 1], TF1);
             fx2* p = s + (ln >> 1) * GS + (ln & 1);
             fx2 v[A];
 #pragma unroll
@@ -296,25 +322,51 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
 #pragma unroll
             for (int k1 = 1; k1 < A; ++k1)
                 if (b) v[k1] = cmul(v[k1], tw[b * k1]);
+            unsigned m = 0;
 #pragma unroll
-            for (int k1 = 0; k1 < A; ++k1) p[2 * (b + B * k1)] = v[k1];
+            for (int k1 = 0; k1 < A; ++k1) {
+                p[2 * (b + B * k1)] = v[k1];
+                m |= fx_key(v[k1]);
+            }
+            atomicOr(kfwd + (ln >> 1), m);
         }
         __syncthreads();
         for (int w = tid; w < NL * A; w += NT) {
             const int ln = w % NL, k1 = w / NL;
             if (RB > 1 && ln / 24 >= nr) continue;
+            const int k = excess(kfwd[ln >> 1], B);
             fx2* p = s + (ln >> 1) * GS + (ln & 1) + 2 * B * k1;
             fx2 v[B];
 #pragma unroll
-            for (int b = 0; b < B; ++b) v[b] = p[2 * b];
+            for (int b = 0; b < B; ++b) v[b] = fx_shift(p[2 * b], k);
             fft2::DFT<B, fx2>::run(v, -1);
-            unsigned m = 0;
 #pragma unroll
-            for (int k2 = 0; k2 < B; ++k2) {
-                p[2 * k2] = v[k2];
-                m |= fx_key(v[k2]);
+            for (int k2 = 0; k2 < B; ++k2) p[2 * k2] = v[k2];
+        }
+        if (tid < 12 * RB) sex[tid] = FxScale(kin[tid], TF1).ex + excess(kfwd[tid], B);
+        __syncthreads();
+        // The product's exponent: the largest, over the points, of the spectrum's exponent less that of B.  (In a pass of its
+        // own: an exponent per point would be a reduction between the product's loads and its digits.)
+        for (int w = tid; w < 2 * LZ * RB; w += NT) {  // whole warps
+            const int c = w & 1, pos = (w >> 1) % LZ, rr = w / (2 * LZ), kz = fft2::freq_at(LZ, pos);
+            const fx2* p = s + rr * 12 * GS + 2 * pos + c;
+            int ec = kLow, el = kLow;
+#pragma unroll
+            for (int a = 0; a < 12; ++a) {
+                const int e = fx_bits(fx_key(p[a * GS])) + sex[rr * 12 + a];
+                if (a % 4)
+                    el = max(el, e);
+                else
+                    ec = max(ec, e);
             }
-            atomicOr(kspec + (ln >> 1), m);
+            int g = max(ec, el - (c ? up1 : up0)) - bex[c * NO + (kz <= LZ / 2 ? kz : LZ - kz)];
+            if (single || LZ < 16) {
+                atomicMax(pex + 2 * rr + c, g);
+                if (!single) atomicMax(pex + 2 * rr + (c ^ 1), g);
+            } else {
+                g = __reduce_max_sync(0xffffffffu, g);
+                if (lane < 2) atomicMax(pex + 2 * rr + lane, g);
+            }
         }
         __syncthreads();
         // block product, a warp per octant point
@@ -323,34 +375,25 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
             const bool nval = RB == 1 ? nr_ == 0 : nr_ < nr;
             const int rout = t >> 1;
             const bool oval = RB == 1 ? rout == 0 : rout < nr;
-            // X = spectrum 2^(kBits - E), the linear components' a quarter of that (their rows and
-            // columns of B are raised by 4): E the exponent of the largest
-            int E = 0, sh[3];
+            // exponents of this lane's components t, t + 4, t + 8
+            int xe[3];
 #pragma unroll
-            for (int rr = 0; rr < RB; ++rr) {
-                int e = -100000;
-                bool b = false;
-                if (lane < 12) {
-                    const unsigned k = kin[rr * 12 + lane];
-                    e = fx_bits(kspec[rr * 12 + lane]) + FxScale(k, TF).ex - (lane % 4 ? 2 : 0);
-                    b = k >= 0x7ff00000u;
-                }
-                e = __reduce_max_sync(0xffffffffu, e);
-                b = __any_sync(0xffffffffu, b);
-                if (rr == nrx) E = e;
-                if (tid == 0) xexp[rr] = e, bad[rr] = b;
+            for (int e = 0; e < 3; ++e) xe[e] = sex[nrx * 12 + t + 4 * e];
+            if (tid < RB) {
+                int b = 0;
+                for (int c = 0; c < 12; ++c) b |= kin[tid * 12 + c] >= 0x7ff00000u;
+                bad[tid] = b;
             }
-#pragma unroll
-            for (int e = 0; e < 3; ++e)
-                sh[e] = max(kBits - E + FxScale(kin[nrx * 12 + t + 4 * e], TF).ex - (t ? 2 : 0), -63);
-            unsigned key = 0;
+            const int xlift = kBits - pex[2 * nrx + ncol] - (t ? (ncol ? up1 : up0) : 0);
+            unsigned key[3] = {0, 0, 0};  // of the lane's outputs, components ra, ra + 4, ra + 8
             for (int q = wid; q < nq; q += NW) {
                 const int col = q >= NO, ko = q - (col ? NO : 0);
                 const bool self = ko == 0 || ko == LZ / 2;
-                // digits of B: rows ra + 4 p, inputs t + 4 q
+                // the point's exponent and digits of B: rows ra + 4 p, inputs t + 4 q
                 unsigned a[3][3][kD];
                 cp_async_wait<0>();
                 __syncwarp();
+                const int lift = xlift - bex[q];  // of X (its columns share an octant point unless they are self-mirrored)
 #pragma unroll
                 for (int p = 0; p < 3; ++p)
 #pragma unroll
@@ -358,7 +401,7 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
                         const bool zero = KOP && p == e;
                         const int tens = (KOP ? 10 * (3 - p - e) : 10 * pq_index(p, e)) + ll;
                         const unsigned neg = bneg ^ (KOP && kblock::levi_civita(p, 3 - p - e, e) > 0 ? 0x80008000u : 0u);
-const uint4 g = zero ? make_uint4(0, 0, 0, 0) : gbuf[tens * 2];
+                        const uint4 g = zero ? make_uint4(0, 0, 0, 0) : gbuf[tens * 2];
                         const uint4 f = zero ? make_uint4(0, 0, 0, 0) : gbuf[tens * 2 + 1];
                         const unsigned v[kD] = {g.x, g.y, g.z, g.w, f.x, f.y, f.z};
 #pragma unroll
@@ -366,7 +409,8 @@ const uint4 g = zero ? make_uint4(0, 0, 0, 0) : gbuf[tens * 2];
                     }
                 __syncwarp();
                 fetch(q + NW < nq ? q + NW : wid);  // after the last one, the next group's first
-                // digits of X: components t + 4 e of point n
+                // digits of X: components t + 4 e of point n, X = spectrum 2^lift: with that, every point's product has the exponent
+                // pex, and X stays below 2^62; the linear components are lower by the raise of B's linear rows and columns
                 unsigned b[3][kD];
                 {
                     const bool v = nval && !(nneg && self) && !(single && ncol != col);
@@ -377,7 +421,7 @@ const uint4 g = zero ? make_uint4(0, 0, 0, 0) : gbuf[tens * 2];
                     for (int e = 0; e < 3; ++e) {
                         const fx2 x = v ? p[4 * e * GS] : fx2{0, 0};
                         const __half2 sg = __float2half2_rn(((m >> (t + 4 * e)) & 1u) ? -1.f : 1.f);
-                        split_digits(x, sh[e], sg, b[e]);
+                        split_digits(x, max(lift + xe[e], -62), sg, b[e]);
                     }
                 }
                 long long y[6];
@@ -398,7 +442,7 @@ const uint4 g = zero ? make_uint4(0, 0, 0, 0) : gbuf[tens * 2];
                             for (int e = 0; e < 3; ++e) {
                                 long long v = y[2 * e + c];
                                 if ((m >> (ra + 4 * e)) & 1u) v = -v;
-                                key |= fx_key(v);
+                                key[e] |= fx_key(v);
                                 p[8 * e * GS + 2 * c] = v;
                             }
                         }
@@ -406,58 +450,46 @@ const uint4 g = zero ? make_uint4(0, 0, 0, 0) : gbuf[tens * 2];
                 }
                 __syncwarp();
             }
-            // a lane's outputs belong to one right-hand side
+            if (oval) {  // a lane's outputs belong to one right-hand side
 #pragma unroll
-            for (int rr = 0; rr < RB; ++rr) {
-                const unsigned m = __reduce_or_sync(0xffffffffu, RB == 1 || rout == rr ? key : 0u);
-                if (lane == 0) atomicOr(kout + rr, m);
+                for (int e = 0; e < 3; ++e) atomicOr(kout + (RB == 1 ? 0 : rout) * 12 + ra + 4 * e, key[e]);
             }
         }
         __syncthreads();
-        // inverse z transform, rescaled before each pass
-        {
-            unsigned key[RB] = {};
-            for (int w = tid; w < NL * A; w += NT) {
-                const int ln = w % NL, k1 = w / NL, rr = ln / 24;
-                if (RB > 1 && rr >= nr) continue;
-                const int k = max(fx_bits(kout[rr]) - TI1, 0);
-                fx2* p = s + (ln >> 1) * GS + (ln & 1) + 2 * B * k1;
-                fx2 v[B];
+        // inverse z transform, a component rescaled before each pass
+        for (int w = tid; w < NL * A; w += NT) {
+            const int ln = w % NL, k1 = w / NL;
+            if (RB > 1 && ln / 24 >= nr) continue;
+            const int k = excess(kout[ln >> 1], B);
+            fx2* p = s + (ln >> 1) * GS + (ln & 1) + 2 * B * k1;
+            fx2 v[B];
 #pragma unroll
-                for (int k2 = 0; k2 < B; ++k2) v[k2] = fx_shift(p[2 * k2], k);
-                fft2::DFT<B, fx2>::run(v, +1);
+            for (int k2 = 0; k2 < B; ++k2) v[k2] = fx_shift(p[2 * k2], k);
+            fft2::DFT<B, fx2>::run(v, +1);
 #pragma unroll
-                for (int b = 1; b < B; ++b)
-                    if (k1) v[b] = cmul(v[b], fx_conj(tw[b * k1]));
-                unsigned m = 0;
+            for (int b = 1; b < B; ++b)
+                if (k1) v[b] = cmul(v[b], fx_conj(tw[b * k1]));
+            unsigned m = 0;
 #pragma unroll
-                for (int b = 0; b < B; ++b) {
-                    p[2 * b] = v[b];
-                    m |= fx_key(v[b]);
-                }
-#pragma unroll
-                for (int u = 0; u < RB; ++u) key[u] |= rr == u ? m : 0u;
+            for (int b = 0; b < B; ++b) {
+                p[2 * b] = v[b];
+                m |= fx_key(v[b]);
             }
-#pragma unroll
-            for (int rr = 0; rr < RB; ++rr) {
-                const unsigned m = __reduce_or_sync(0xffffffffu, key[rr]);
-                if (lane == 0) atomicOr(kmid + rr, m);
-            }
+            atomicOr(kmid + (ln >> 1), m);
         }
         __syncthreads();
         for (int w = tid; w < NL * B; w += NT) {
             const int ln = w % NL, b = w / NL, rr = ln / 24;
             if (RB > 1 && rr >= nr) continue;
             const fx2* p = s + (ln >> 1) * GS + (ln & 1);
-            const int k = max(fx_bits(kmid[rr]) - TI2, 0);
+            const int k = excess(kmid[ln >> 1], A);
             fx2 v[A];
 #pragma unroll
             for (int k1 = 0; k1 < A; ++k1) v[k1] = fx_shift(p[2 * (b + B * k1)], k);
             fft2::dft_half_out<A>(v, +1);
-            // exponent of the result: that of X, of Y, of B and of the two shifts
             const int comp = (ln % 24) >> 1, c = ln & 1;
-            const int ex = xexp[rr] - kBits + kShift - (c ? gex1 : gex0) + max(fx_bits(kout[rr]) - TI1, 0) + k -
-                           (comp % 4 ? 2 : 0);
+            // exponent of the result: that of the product and the bits dropped since
+            const int ex = pex[2 * rr + c] - (comp % 4 ? (c ? up1 : up0) : 0) - kBits + kShift + excess(kout[ln >> 1], B) + k;
             double2* out = z.w + (long long)(r0 + rr) * 12 * nz * plane + (long long)py * z.Lx + sc0 + c;
 #pragma unroll
             for (int a = 0; a < A / 2; ++a) {
@@ -470,51 +502,65 @@ const uint4 g = zero ? make_uint4(0, 0, 0, 0) : gbuf[tens * 2];
             }
         }
         __syncthreads();
-        if (tid < 26 * RB) kin[tid] = 0;
+        reset();
         __syncthreads();
     }
     cp_async_wait<0>();
 }
 
-// Digit tables from the octant spectra g [NG][Oz][Oy][Ox]: per column (ky, kx) the exponent of its
-// values (|B 2^gexp| < 2^62 with the linear functions' rows and columns raised by 4, which brings them to
-// the size of the constant ones: their Gram entries are 1/12) and seven signed 9-bit digits per value.
+// Digit tables from the octant spectra g [NG][Oz][Oy][Ox].  Every octant point has an exponent be and every column a raise
+// up: an entry B is stored as seven signed 9-bit digits of B 2^(be + c up), c the number of linear functions in its pair,
+// below 2^62; be << 8 | up is in the unused last word of tensor 0.  The raise brings the linear rows and columns
+// up to the constant ones (their Gram entries are 1/12, and where the spectrum is large they couple through
+// differences); it is the largest that leaves the pairs of constant functions the largest values, give or
+// take a bit or two.
 // A block takes kDigitCols neighbouring columns, whose values of one (tensor, kz) are 128 contiguous bytes, and reads
 // them twice; the digits of a value are 32 contiguous bytes.
-constexpr int kDigitCols = 8;
+constexpr int kDigitCols = 8, kMaxOz = 257;
 __global__ void __launch_bounds__(256) digits_kernel(const double2* __restrict__ g, int Ox, int Oy, int Oz, int NG,
-                                                     uint4* __restrict__ d, int* __restrict__ gexp) {
-    __shared__ unsigned key[kDigitCols];
+                                                     uint4* __restrict__ d) {
+    __shared__ int top[3][kMaxOz][kDigitCols];  // per class of pairs: |B| < 2^(top - 1022); then [0]: be
+    __shared__ int ctop[3][kDigitCols];         // the same over a column
     const int c = threadIdx.x % kDigitCols, kx = blockIdx.x * kDigitCols + c, ky = blockIdx.y;
-    if (threadIdx.x < kDigitCols) key[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < 3 * kMaxOz * kDigitCols; i += 256) (&top[0][0][0])[i] = kLow;
+    if (threadIdx.x < 3 * kDigitCols) (&ctop[0][0])[threadIdx.x] = kLow;
     __syncthreads();
     const int n = NG * Oz;
-    auto raise = [&](int t) {  // pairs (1,1), (1,l') and (l,l'): by 2^0, 2^2 and 2^4
+    auto linear = [](int t) {  // linear functions in the pair
         const int ll = t % 10;
-        return ll == 0 ? 0 : (ll < 4 ? 2 : 4);
+        return ll == 0 ? 0 : (ll < 4 ? 1 : 2);
     };
-    if (kx < Ox) {
-        unsigned m = 0;
+    if (kx < Ox)
         for (int i = threadIdx.x / kDigitCols; i < n; i += 256 / kDigitCols) {
-            const double2 v = g[((long long)i * Oy + ky) * Ox + kx];
-            const unsigned k = fx_key(v);
-            m = max(m, k >= 0x00100000u ? k + (raise(i / Oz) << 20) : 0u);
+            const int t = i / Oz, kz = i - t * Oz;
+            double2 v = g[((long long)i * Oy + ky) * Ox + kx];
+            int e = (int)(fx_key(v) >> 20);
+            if (e == 0) {  // subnormal numbers
+                v = make_double2(0x1p64 * v.x, 0x1p64 * v.y);
+                e = v.x == 0.0 && v.y == 0.0 ? kLow : (int)(fx_key(v) >> 20) - 64;
+            }
+            atomicMax(&top[linear(t)][kz][c], e);
         }
-        atomicMax(key + c, m);
+    __syncthreads();
+    for (int q = 0; q < 3; ++q)
+        for (int kz = threadIdx.x / kDigitCols; kz < Oz; kz += 256 / kDigitCols) atomicMax(&ctop[q][c], top[q][kz][c]);
+    __syncthreads();
+    const int up = min(max(min((ctop[0][c] - ctop[2][c] + 1) >> 1, ctop[0][c] - ctop[1][c] + 2), 0), 60);
+    for (int kz = threadIdx.x / kDigitCols; kz < Oz; kz += 256 / kDigitCols) {
+        const int e = max(top[0][kz][c], max(top[1][kz][c] + up, top[2][kz][c] + 2 * up));
+        top[0][kz][c] = e > kLow / 2 ? kBits + 1022 - e : 0;
     }
     __syncthreads();
     if (kx >= Ox) return;
-    const int sb = key[c] ? kBits + 1022 - (int)(key[c] >> 20) : 0;
     const long long col = (long long)ky * Ox + kx;
-    if (threadIdx.x < kDigitCols) gexp[col] = sb;
     for (int i = threadIdx.x / kDigitCols; i < n; i += 256 / kDigitCols) {
         const int t = i / Oz, kz = i - t * Oz;
-        const int up = sb + raise(t);
+        const int be = top[0][kz][c], sc = be + linear(t) * up;
         double2 v = g[((long long)i * Oy + ky) * Ox + kx];
-        if (up > 1000 || up < -1000) {
-            v = make_double2(scalbn(v.x, up), scalbn(v.y, up));
+        if (sc > 1000 || sc < -1000) {
+            v = make_double2(scalbn(v.x, sc), scalbn(v.y, sc));
         } else {
-            const double f = __hiloint2double((1023 + up) << 20, 0);
+            const double f = __hiloint2double((1023 + sc) << 20, 0);
             v = make_double2(f * v.x, f * v.y);
         }
         unsigned long long re = (unsigned long long)__double2ll_rn(v.x) + kBias;
@@ -530,7 +576,7 @@ __global__ void __launch_bounds__(256) digits_kernel(const double2* __restrict__
         }
         uint4* out = d + 2 * ((col * Oz + kz) * NG + t);
         out[0] = make_uint4(u[0], u[1], u[2], u[3]);
-        out[1] = make_uint4(u[4], u[5], u[6], 0);
+        out[1] = make_uint4(u[4], u[5], u[6], t == 0 ? (unsigned)(be << 8 | up) : 0u);
     }
 }
 
@@ -568,7 +614,7 @@ int launch_zd(const vie_handle* h, const ZDArgs& z, cudaStream_t s) {
 int green_digits(const vie_handle* h, const double2* g, int ng, uint4* d, cudaStream_t s) {
     const dim3 grid((unsigned)((h->O[0] + kDigitCols - 1) / kDigitCols), (unsigned)h->O[1]);
     VIE_KLAUNCH("green_digits", s,
-                digits_kernel<<<grid, 256, 0, s>>>(g, h->O[0], h->O[1], h->O[2], ng, d, digit_exponents(h, ng, d)));
+                digits_kernel<<<grid, 256, 0, s>>>(g, h->O[0], h->O[1], h->O[2], ng, d));
     VIE_CHECK_LAUNCH();
     return VIE_OK;
 }

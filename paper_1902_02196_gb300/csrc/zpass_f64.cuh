@@ -6,7 +6,6 @@
 struct ZDArgs {
     double2* w;                // spectrum [R*12][Nz][Ly][Lx], in place
     const uint4* green_d;      // digits of the block's tensors (green_digits): [Oy][Ox][Oz][60 (N) or 30 (K)][2]
-    const int* gexp;           // [Oy][Ox] their exponents
     const int* colkx;          // [Lx] kx of each stored column (mirror pairs)
     int R, nz, Lx, Ly, Ox, Oy, Oz;
     int ay, by;                // row py holds ky = py / by + ay * (py % by)
@@ -15,12 +14,8 @@ struct ZDArgs {
     unsigned long long* bctr;
 };
 
-// Digit tables of the octant spectra g [ng][Oz][Oy][Ox] (device) into d, green_digit_bytes(h, ng) bytes: the
-// digits [Oy][Ox][Oz][ng][2], then the exponents [Oy][Ox].
+// Digit tables [Oy][Ox][Oz][ng][2] of the octant spectra g [ng][Oz][Oy][Ox] (device) into d, green_digit_bytes(h, ng) bytes.
 int green_digits(const vie_handle* h, const double2* g, int ng, uint4* d, cudaStream_t s);
-inline int* digit_exponents(const vie_handle* h, int ng, uint4* d) {
-    return reinterpret_cast<int*>(d + 2 * (size_t)ng * h->O[0] * h->O[1] * h->O[2]);
-}
 // Launches the FP64 z pass (Lz in 8..512, Lx >= 4).
 int zpass_f64_fused(const vie_handle* h, const ZDArgs& z, cudaStream_t s);
 // The same z pass with the K block (VIE_OP_K) on the K octant [Oy][Ox][Oz][30].
