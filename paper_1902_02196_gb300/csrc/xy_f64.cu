@@ -4,17 +4,21 @@
 // (fixed.cuh): sm_103a's two FP64 operations per clock and SM made these transforms take 11 to 13 ms each way
 // for 16 right-hand sides on a 64^3 grid.
 //
-// Precision.  A plane's scale is taken from its largest element.  Before each of the four passes the
-// values are brought to the bits which that pass's worst case leaves room for (fx_room): 56 to 58 of
-// them, so that a rounding is 2^-56 of the plane's largest value or less, where FP64 rounds every
-// operation to 2^-53 of its own result.
+// Precision.  Every line has its own scale, a row along x and a column along y, from its largest element; with one scale for
+// a plane, planes whose values or spectra have a peak came out up to five times further off.  Before each of
+// the four passes a line is brought to the bits which that pass's worst case leaves room for (fx_room): 56 to
+// 58 of them, so that a rounding is 2^-56 of the line's largest value or less, where FP64 rounds every
+// operation to 2^-53 of its own result.  The lanes of a warp are on different lines, so a line's key is an atomic
+// without conflicts.
 //
-// Measured, 16 right-hand sides on 64^3 voxels (12288 planes, 128 x 128 spectra): forward 3.2 ms and inverse
-// 4.7 ms, the FP64 kernels 11.2 and 13.1 ms.
+// Measured, 16 right-hand sides on 64^3 voxels (12288 planes, 128 x 128 spectra): forward 3.24 ms and inverse
+// 4.73 ms, the FP64 kernels 11.2 and 13.1 ms (and 3.18 and 4.67 ms with a scale for a plane).
 //
 // A CTA owns one plane.  The x spectra of its rows stay in shared memory; the y transforms run on
 // chunks of CW stored columns, whose spectra go to or come from global memory in registers, 512
 // contiguous bytes to a warp.
+#include <climits>
+
 #include "block.cuh"
 #include "fft2.cuh"
 #include "fixed.cuh"
@@ -27,39 +31,13 @@ struct XYCfg64 {
     static constexpr int H = L / 2;                // rows that are non-zero before / needed after the y transform
     static constexpr int RS = L + 1;               // odd row stride
     static constexpr int CW = L < 32 ? L : 32;     // stored columns per y-transform chunk
-    static constexpr int NCH = L / CW;
     static constexpr int NT = L >= 128 ? 512 : (L >= 32 ? 256 : 64);
     static constexpr int MINB = L >= 128 ? 1 : (L >= 64 ? 2 : 4);
-    static constexpr size_t smem = sizeof(fx2) * (size_t)(L * CW + H * RS + L) + sizeof(int4) * H + 2 * L + 128;
+    static constexpr size_t smem = sizeof(fx2) * (size_t)(L * CW + H * RS + L) + sizeof(int4) * H + L + sizeof(int) * (4 * L);
 };
 
-__device__ __forceinline__ fx2 down(fx2 v, int k) {  // v 2^-k to nearest, k uniform
-    if (k) {
-        const long long h = 1LL << (k - 1);
-        v.x = (v.x + h) >> k;
-        v.y = (v.y + h) >> k;
-    }
-    return v;
-}
-
-// largest key of the CTA into *dst (zeroed before): followed by a barrier of the caller
-__device__ __forceinline__ void collect_max(unsigned key, unsigned* dst) {
-    key = __reduce_max_sync(0xffffffffu, key);
-    if ((threadIdx.x & 31) == 0) atomicMax(dst, key);
-}
-__device__ __forceinline__ void collect_or(unsigned key, unsigned* dst) {
-    key = __reduce_or_sync(0xffffffffu, key);
-    if ((threadIdx.x & 31) == 0) atomicOr(dst, key);
-}
-
-// after a pass whose inputs had room for it, |v| <= 2^60.5: bits that the next pass, of N points, has to drop.
-// The CTA's decision, by *slot (zeroed before, used once); ends with a barrier.
-template <int N>
-__device__ __forceinline__ int rescale(unsigned key, unsigned* slot) {
-    collect_or(key, slot);
-    __syncthreads();
-    return max(fx_bits(*slot) - fx_room(N), 0);
-}
+// bits that a line whose values have these keys has to drop before a pass of n points
+__device__ __forceinline__ int excess(unsigned key, int n) { return max(fx_bits(key) - fx_room(n), 0); }
 
 // Forward: plane (r, alpha, z) of x -> W2 plane [Ly][Lx] (transposed ky, stored kx).  x is
 // [R][nc][Nz][Ny][Nx], or [R][nc][ns] on a support (rows != NULL; zeros outside it).
@@ -76,8 +54,11 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
     int4* tw = reinterpret_cast<int4*>(xr + H * RS);
     int4* rw = tw + L;  // [H] support rows of this plane
     unsigned char* pos = reinterpret_cast<unsigned char*>(rw + H);
-    // of the input, of the x spectra, after the first x pass, after the first y pass of each chunk
-    unsigned* keys = reinterpret_cast<unsigned*>(pos + 2 * L);
+    unsigned* krow = reinterpret_cast<unsigned*>(pos + L);  // [H] keys of the rows
+    unsigned* kmid = krow + H;                              // [H] after the first x pass
+    unsigned* kspec = kmid + H;                             // [H] of their x spectra
+    int* rsh = reinterpret_cast<int*>(kspec + H);           // [H] shift of a row to the plane's scale
+    unsigned* kcol = reinterpret_cast<unsigned*>(rsh + H);  // [L] of the stored columns after the first y pass
     const int tid = threadIdx.x;
     const long long p = blockIdx.x;  // spectrum plane; the input plane is pin (rmap: active right-hand sides)
     const long long rplanes = (long long)dc.nc * nz;  // planes per right-hand side
@@ -92,7 +73,7 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
         tw[m] = twg[m];
         pos[m] = cpos[m];
     }
-    if (tid < 3 + Cfg::NCH) keys[tid] = 0;
+    for (int m = tid; m < 4 * H + L; m += NT) krow[m] = 0;
     const long long pin = rmap ? (long long)rmap[p / rplanes] * rplanes + p % rplanes : p;
     const double2* src = x + pin * (long long)ny * nx;
     if (rows) {
@@ -101,43 +82,46 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
         src = x + (pin / nz) * ns;
     }
     __syncthreads();
-    {
-        unsigned key = 0;
-        for (int i0 = tid; i0 < ny * nx; i0 += 4 * NT) {  // four loads in flight
-            double2 v[4];
-            int dst[4];
+    for (int i0 = tid; i0 < ny * nx; i0 += 4 * NT) {  // four loads in flight
+        double2 v[4];
+        int dst[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int idx = i0 + q * NT, yy = idx / nx, xx = idx - yy * nx;
-                v[q] = make_double2(0.0, 0.0);
-                dst[q] = idx < ny * nx ? yy * RS + xx : -1;
-                if (idx < ny * nx) {
-                    if (rows) {
-                        const int4 s = rw[yy];
-                        if (xx >= s.x && xx < s.y) v[q] = src[s.z + (xx - s.x)];
-                    } else {
-                        v[q] = src[idx];
-                    }
+        for (int q = 0; q < 4; ++q) {
+            const int idx = i0 + q * NT, yy = idx / nx, xx = idx - yy * nx;
+            v[q] = make_double2(0.0, 0.0);
+            dst[q] = idx < ny * nx ? yy * RS + xx : -1;
+            if (idx < ny * nx) {
+                if (rows) {
+                    const int4 s = rw[yy];
+                    if (xx >= s.x && xx < s.y) v[q] = src[s.z + (xx - s.x)];
+                } else {
+                    v[q] = src[idx];
                 }
             }
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (dst[q] >= 0) {
-                    *reinterpret_cast<double2*>(xr + dst[q]) = v[q];
-                    key = max(key, fx_key(v[q]));
-                }
         }
-        collect_max(key, keys);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (dst[q] >= 0) *reinterpret_cast<double2*>(xr + dst[q]) = v[q];
     }
     __syncthreads();
-    const bool bad = keys[0] >= 0x7ff00000u;  // an Inf or NaN reaches the whole spectrum
-    const FxScale sc(keys[0], fx_room(A / 2));
-    int ex = sc.ex;
-    // x transform
-    unsigned key = 0;
+    // x transform; lanes are on different rows
     for (int t = tid; t < H * B; t += NT) {
         const int n = t % H, b = t / H;
         if (n >= ny) continue;
+        const double2* ln = reinterpret_cast<const double2*>(xr + n * RS);
+        unsigned key = 0;
+#pragma unroll
+        for (int a = 0; a < A / 2; ++a) {
+            const int l = b + B * a;
+            if (l < nx) key = max(key, fx_key(ln[l]));
+        }
+        atomicMax(krow + n, key);
+    }
+    __syncthreads();
+    for (int t = tid; t < H * B; t += NT) {
+        const int n = t % H, b = t / H;
+        if (n >= ny) continue;
+        const FxScale sc(krow[n], fx_room(A / 2));
         fx2* ln = xr + n * RS;
         fx2 v[A];
 #pragma unroll
@@ -146,40 +130,53 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
             v[a] = l < nx ? sc(*reinterpret_cast<const double2*>(ln + l)) : fx2{0, 0};
         }
         fft2::dft_half_in<A>(v, -1);
+        unsigned key = 0;
 #pragma unroll
         for (int k1 = 0; k1 < A; ++k1) {
             if (k1 && b) v[k1] = cmul(v[k1], tw[b * k1]);
             ln[b + B * k1] = v[k1];
             key |= fx_key(v[k1]);
         }
+        atomicOr(kmid + n, key);
     }
-    int k = rescale<B>(key, keys + 2);
-    ex += k;
-    key = 0;
+    __syncthreads();
     for (int t = tid; t < H * A; t += NT) {
         const int n = t % H, k1 = t / H;
         if (n >= ny) continue;
+        const int k = excess(kmid[n], B);
         fx2* ln = xr + n * RS + B * k1;
         fx2 v[B];
 #pragma unroll
-        for (int b = 0; b < B; ++b) v[b] = down(ln[b], k);
+        for (int b = 0; b < B; ++b) v[b] = fx_shift(ln[b], k);
         fft2::DFT<B, fx2>::run(v, -1);
+        unsigned key = 0;
 #pragma unroll
         for (int k2 = 0; k2 < B; ++k2) {
             ln[k2] = v[k2];
             key |= fx_key(v[k2]);
         }
+        atomicOr(kspec + n, key);
     }
-    collect_or(key, keys + 1);
     __syncthreads();
-    const int ks = max(fx_bits(keys[1]) - fx_room(A / 2), 0);  // to the room of the y transform
-    ex += ks;
+    // The rows' spectra go to one scale, with room for the y transform.  (No row is shifted up: a spectrum is as
+    // large as its row, so its exponent is below the common one as it is.)
+    auto row_ex = [&](int n) { return FxScale(krow[n], fx_room(A / 2)).ex + excess(kmid[n], B); };
+    int ex = INT_MIN;
+    unsigned kall = 0;
+    for (int n = tid & 31; n < ny; n += 32) {
+        const int e = row_ex(n);
+        ex = max(ex, max(fx_bits(kspec[n]) - fx_room(A / 2), 0) + e);
+        kall = max(kall, krow[n]);
+    }
+    ex = __reduce_max_sync(0xffffffffu, ex);
+    for (int n = tid; n < ny; n += NT) rsh[n] = min(ex - row_ex(n), 62);
+    const bool bad = __reduce_max_sync(0xffffffffu, kall) >= 0x7ff00000u;  // an Inf or NaN reaches the whole spectrum
+    __syncthreads();
     double2* dst = w + p * (long long)L * L;
 #pragma unroll 1
     for (int c0 = 0; c0 < L; c0 += CW) {
         // y transform, pass 1: stored column c0 + c from the x spectra.  An A-point DFT of A/2 values
         // is two A/2-point ones, of the even and (twisted) of the odd frequencies: a task each
-        key = 0;
         for (int t = tid; t < 2 * CW * B; t += NT) {
             const int c = t % CW, b = (t / CW) % B, odd = t / (CW * B);
             const fx2* col = xr + pos[c0 + c];
@@ -187,13 +184,14 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
 #pragma unroll
             for (int a = 0; a < A / 2; ++a) {  // ny <= L/2: the upper half is zero
                 const int yy = b + B * a;
-                v[a] = yy < ny ? down(col[yy * RS], ks) : fx2{0, 0};
+                v[a] = yy < ny ? fx_shift(col[yy * RS], rsh[yy]) : fx2{0, 0};
             }
             if (odd) {
 #pragma unroll
                 for (int a = 0; a < A / 2; ++a) v[a] = fft2::twist<A>(v[a], a, -1);
             }
             fft2::DFT<A / 2, fx2>::run(v, -1);
+            unsigned key = 0;
 #pragma unroll
             for (int q = 0; q < A / 2; ++q) {
                 const int k1 = 2 * q + odd;
@@ -201,14 +199,16 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
                 ck[(b + B * k1) * CW + c] = v[q];
                 key |= fx_key(v[q]);
             }
+            atomicOr(kcol + c0 + c, key);
         }
-        k = rescale<B>(key, keys + 3 + c0 / CW);
+        __syncthreads();
         for (int t = tid; t < CW * A; t += NT) {
             const int c = t % CW, k1 = t / CW;
+            const int k = excess(kcol[c0 + c], B);
             const fx2* ln = ck + B * k1 * CW + c;
             fx2 v[B];
 #pragma unroll
-            for (int b = 0; b < B; ++b) v[b] = down(ln[b * CW], k);
+            for (int b = 0; b < B; ++b) v[b] = fx_shift(ln[b * CW], k);
             fft2::DFT<B, fx2>::run(v, -1);
 #pragma unroll
             for (int k2 = 0; k2 < B; ++k2) {
@@ -229,20 +229,17 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
                     const unsigned char* __restrict__ cpos, const int4* __restrict__ twg) {
     using Cfg = XYCfg64<L>;
     constexpr int A = fft2::Split<L>::A, B = fft2::Split<L>::B, NT = Cfg::NT, RS = Cfg::RS, CW = Cfg::CW, H = Cfg::H;
-    constexpr int NCH = Cfg::NCH;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     fx2* ck = reinterpret_cast<fx2*>(smem_raw);
     fx2* xr = ck + L * CW;
     int4* tw = reinterpret_cast<int4*>(xr + H * RS);
     int4* rw = tw + L;
     unsigned char* pos = reinterpret_cast<unsigned char*>(rw + H);
-    unsigned char* chunk_of = pos + L;  // chunk of an x-transform position
-    // per chunk: the key of its spectrum, the key of its y-transformed rows, their exponent, the key after its first
-    // pass; the key after the first x pass
-    unsigned* kin = reinterpret_cast<unsigned*>(pos + 2 * L);
-    unsigned* kout = kin + NCH;
-    int* cex = reinterpret_cast<int*>(kout + NCH);
-    unsigned* kmid = kout + 2 * NCH;
+    unsigned* kcol = reinterpret_cast<unsigned*>(pos + L);   // [L] keys of the stored columns
+    unsigned* kmid = kcol + L;                               // [L] after the first y pass
+    int* cex = reinterpret_cast<int*>(kmid + L);             // [L] by x position: the exponent after the y transform
+    int* rtop = cex + L;                                     // [H] bits and exponent of the largest value of a row
+    unsigned* krow = reinterpret_cast<unsigned*>(rtop + H);  // [H] keys of the rows after the first x pass
     const int tid = threadIdx.x;
     const int nx = epi.nx, ny = epi.ny, nz = epi.nz;
     const long long p = blockIdx.x;  // spectrum plane (r * nc + alpha) * nz + z; output plane po
@@ -258,41 +255,42 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
     for (int m = tid; m < L; m += NT) {
         tw[m] = twg[m];
         pos[m] = cpos[m];
-        chunk_of[cpos[m]] = (unsigned char)(m / CW);
+        kcol[m] = kmid[m] = 0;
     }
-    if (tid < 4 * NCH + 1) kin[tid] = 0;
+    for (int n = tid; n < H; n += NT) {
+        rtop[n] = INT_MIN;
+        krow[n] = 0;
+    }
     const long long po = epi.rmap ? (long long)epi.rmap[p / rplanes] * rplanes + p % rplanes : p;
     if (epi.rows)
         for (int yy = tid; yy < ny; yy += NT) rw[yy] = epi.rows[(p % nz) * ny + yy];
     __syncthreads();
     const double2* src = w + p * (long long)L * L;
-    bool bad = false;
 #pragma unroll 1
-    for (int h = 0; h < NCH; ++h) {
+    for (int c0 = 0; c0 < L; c0 += CW) {
         // inverse y transform, pass 1.  One task per thread (CW A <= NT), so its inputs wait in registers
-        // for the chunk's scale
+        // for the column's scale
         static_assert(CW * A <= NT || L < 32, "one pass-1 task per thread");
         constexpr int NTASK = (CW * A + NT - 1) / NT;
         double2 d[NTASK][B];
-        unsigned key = 0;
 #pragma unroll
         for (int q = 0; q < NTASK; ++q) {
             const int t = tid + q * NT, c = t % CW, k1 = t / CW;
+            unsigned key = 0;
 #pragma unroll
             for (int k2 = 0; k2 < B; ++k2) {
-                d[q][k2] = t < CW * A ? src[(long long)(B * k1 + k2) * L + h * CW + c] : make_double2(0.0, 0.0);
+                d[q][k2] = t < CW * A ? src[(long long)(B * k1 + k2) * L + c0 + c] : make_double2(0.0, 0.0);
                 key = max(key, fx_key(d[q][k2]));
             }
+            if (t < CW * A) atomicMax(kcol + c0 + c, key);
         }
-        collect_max(key, kin + h);
         __syncthreads();
-        bad = bad || kin[h] >= 0x7ff00000u;
-        const FxScale sc(kin[h], fx_room(B));
-        key = 0;
 #pragma unroll
         for (int q = 0; q < NTASK; ++q) {
             const int t = tid + q * NT, c = t % CW, k1 = t / CW;
             if (t >= CW * A) continue;
+            const FxScale sc(kcol[c0 + c], fx_room(B));
+            unsigned key = 0;
             fx2 v[B];
 #pragma unroll
             for (int k2 = 0; k2 < B; ++k2) v[k2] = sc(d[q][k2]);
@@ -303,30 +301,38 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
                 ck[(b + B * k1) * CW + c] = v[b];
                 key |= fx_key(v[b]);
             }
+            atomicOr(kmid + c0 + c, key);
         }
-        const int k = rescale<A>(key, kmid + h);
+        __syncthreads();
         // pass 2: rows y < Ny scattered to the x-transform buffer at the column's x position
-        key = 0;
         for (int t = tid; t < CW * B; t += NT) {
-            const int c = t % CW, b = t / CW;
+            const int c = t % CW, b = t / CW, px = pos[c0 + c];
+            const int k = excess(kmid[c0 + c], A);
             fx2 v[A];
 #pragma unroll
-            for (int k1 = 0; k1 < A; ++k1) v[k1] = down(ck[(b + B * k1) * CW + c], k);
+            for (int k1 = 0; k1 < A; ++k1) v[k1] = fx_shift(ck[(b + B * k1) * CW + c], k);
             fft2::dft_half_out<A>(v, +1);
-            fx2* col = xr + pos[h * CW + c];
+            const int ex = FxScale(kcol[c0 + c], fx_room(B)).ex + k;
+            fx2* col = xr + px;
 #pragma unroll
             for (int a = 0; a < A / 2; ++a) {  // ny <= L/2
-                const int yy = b + B * a;
-                if (yy < ny) {
-                    col[yy * RS] = v[a];
-                    key |= fx_key(v[a]);
+                const int yy = b + B * a, top = fx_bits(fx_key(v[a])) + ex;
+                if (yy >= ny) continue;
+                col[yy * RS] = v[a];
+                if constexpr (CW == 32) {  // a warp is on one row
+                    const int m = __reduce_max_sync(0xffffffffu, top);
+                    if (c == 0) atomicMax(rtop + yy, m);
+                } else {
+                    atomicMax(rtop + yy, top);
                 }
             }
+            if (b == 0) cex[px] = ex;
         }
-        collect_or(key, kout + h);
-        if (tid == 0) cex[h] = sc.ex + k;
         __syncthreads();
     }
+    unsigned kall = 0;
+    for (int m = tid & 31; m < L; m += 32) kall = max(kall, kcol[m]);
+    const bool bad = __reduce_max_sync(0xffffffffu, kall) >= 0x7ff00000u;  // an Inf or NaN reaches the whole plane
     const long long base = po * (long long)ny * nx;
     const long long cbase = (po / nz) * epi.ns;  // component block on the support
     const double2* xin = reinterpret_cast<const double2*>(epi.x);
@@ -346,46 +352,45 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
         }
         cp_async_commit();
     }
-    // inverse x transform: the chunks' columns on the scale of the largest
-    int E = -100000;
-#pragma unroll
-    for (int h = 0; h < NCH; ++h) E = max(E, fx_bits(kout[h]) + cex[h]);
-    int ex = E - fx_room(B);
-    unsigned key = 0;
+    // inverse x transform: a row's values, one of each column, on the scale of its largest
     for (int t = tid; t < H * A; t += NT) {
         const int n = t % H, k1 = t / H;
         if (n >= ny) continue;
+        const int ex = rtop[n] - fx_room(B);
         fx2* ln = xr + n * RS + B * k1;
         fx2 v[B];
 #pragma unroll
         for (int k2 = 0; k2 < B; ++k2) {
-            const int s = max(cex[chunk_of[B * k1 + k2]] - ex, -63);  // <= 25: the key counts 32 bits at least
-            const fx2 u = ln[k2];
-            v[k2] = s >= 0 ? fx2{u.x << s, u.y << s} : fx2{u.x >> -s, u.y >> -s};
+            const int s = ex - cex[B * k1 + k2], up = max(-s, 0);  // up <= 25: the bits count 32 at least
+            const fx2 u = fx_shift(ln[k2], min(max(s, 0), 62));
+            v[k2] = fx2{u.x << up, u.y << up};
         }
         fft2::DFT<B, fx2>::run(v, +1);
+        unsigned key = 0;
 #pragma unroll
         for (int b = 0; b < B; ++b) {
             if (b && k1) v[b] = cmul(v[b], fx_conj(tw[b * k1]));
             ln[b] = v[b];
             key |= fx_key(v[b]);
         }
+        atomicOr(krow + n, key);
     }
-    const int k = rescale<A>(key, kmid + NCH);
-    ex += k;
+    __syncthreads();
     for (int t = tid; t < H * B; t += NT) {
         const int n = t % H, b = t / H;
         if (n >= ny) continue;
+        const int k = excess(krow[n], A);
         fx2* ln = xr + n * RS;
         fx2 v[A];
 #pragma unroll
-        for (int k1 = 0; k1 < A; ++k1) v[k1] = down(ln[b + B * k1], k);
+        for (int k1 = 0; k1 < A; ++k1) v[k1] = fx_shift(ln[b + B * k1], k);
         fft2::dft_half_out<A>(v, +1);
 #pragma unroll
         for (int a = 0; a < A / 2; ++a) {
             const int l = b + B * a;
             if (l < nx) ln[l] = v[a];
         }
+        if (b == 0) rtop[n] += k - fx_room(B);  // now the exponent of the row's results
     }
     if (pre) cp_async_wait<0>();
     __syncthreads();
@@ -408,7 +413,7 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
             o = cbase + q.z + (xx - q.x);
         }
         if (!CONV && !in) continue;
-        double2 v = fx_double(xr[yy * RS + xx], ex);
+        double2 v = fx_double(xr[yy * RS + xx], rtop[yy]);
         if (bad) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
         if (CONV) conv[base + idx] = v;  // every voxel of the plane, full-grid layout
         if (!in) continue;
