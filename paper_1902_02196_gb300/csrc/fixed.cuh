@@ -101,6 +101,8 @@ __device__ __forceinline__ unsigned fx_key(long long v) {
 __device__ __forceinline__ unsigned fx_key(fx2 v) { return fx_key(v.x) | fx_key(v.y); }
 // bits b with |v| <= 2^b for every v of a block with these keys
 __device__ __forceinline__ int fx_bits(unsigned key) { return 64 - __clz((int)key); }
+// bits that a line whose values have these keys has to drop before a pass of n points
+__device__ __forceinline__ int excess(unsigned key, int n) { return max(fx_bits(key) - fx_room(n), 0); }
 
 // A block's scale: v -> v 2^(T + 1022 - E).  Blocks below 2^-958 are raised by 2^512 first, so
 // that no value of theirs is subnormal.

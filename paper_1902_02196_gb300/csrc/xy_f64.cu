@@ -36,9 +36,6 @@ struct XYCfg64 {
     static constexpr size_t smem = sizeof(fx2) * (size_t)(L * CW + H * RS + L) + sizeof(int4) * H + L + sizeof(int) * (4 * L);
 };
 
-// bits that a line whose values have these keys has to drop before a pass of n points
-__device__ __forceinline__ int excess(unsigned key, int n) { return max(fx_bits(key) - fx_room(n), 0); }
-
 // Forward: plane (r, alpha, z) of x -> W2 plane [Ly][Lx] (transposed ky, stored kx).  x is
 // [R][nc][Nz][Ny][Nx], or [R][nc][ns] on a support (rows != NULL; zeros outside it).
 template <int L>

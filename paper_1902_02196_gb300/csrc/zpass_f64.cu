@@ -188,9 +188,6 @@ __device__ __forceinline__ void split_digits(fx2 v, int sh, __half2 sg, unsigned
     }
 }
 
-// bits that values with these keys have to drop before a pass of n points
-__device__ __forceinline__ int excess(unsigned key, int n) { return max(fx_bits(key) - fx_room(n), 0); }
-
 __device__ __forceinline__ int pos_of(int L, int k) { return fft2::tpos(L, k); }
 
 template <int LZ, bool KOP>

@@ -4,7 +4,7 @@
 // (fixed.cuh).  It replaces the generic z pass (matvec.cu: radix-4 transforms, log4 L trips through
 // shared memory) for FFT lengths along z of 8..512 and Lx >= 8: one right-hand side on 61^3 voxels (128^3 points)
 // took 0.95 ms there in FP64, which the FP64 unit's two operations per clock bound.  The product itself,
-// nine complex multiply-adds a point, stays on that unit.
+// nine complex multiply-adds a point, stays on that unit.  Every line has its own scale, renewed before each pass.
 //
 // The six Green values of a point come from the octant spectra [60][Oz][Oy][Ox] (every tenth tensor), served by
 // L2: a reordered copy would save less than it costs to set up for a system that is solved once or twice.
@@ -22,7 +22,7 @@ struct ZPCfg {
     static constexpr int NT = LZ <= 16 ? 96 : (LZ == 256 ? 384 : 192);
     static constexpr int MINB = LZ <= 128 ? 3 : (LZ == 256 ? 1 : 2);
     static constexpr int GS = LZ * TB + 8;  // component stride: 8 elements of padding keep half-warps apart
-    static constexpr size_t smem = (sizeof(T) == 8 ? 16 : 8) * (size_t)(3 * GS + LZ) + 64;
+    static constexpr size_t smem = (sizeof(T) == 8 ? 16 : 8) * (size_t)(3 * GS + LZ) + (sizeof(T) == 8 ? 4 * sizeof(int) * NL : 0);
 };
 
 // y = B x at one point: entry (p, q) is tensor 10 pq(p, q); m: components whose sign flips at this reflected point
@@ -61,8 +61,9 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
     fx2* f = reinterpret_cast<fx2*>(smem_raw);  // FP64: the same places, between the conversions
     float2* twf = reinterpret_cast<float2*>(s + 3 * GS);
     int4* twi = reinterpret_cast<int4*>(s + 3 * GS);
-    unsigned* kin = reinterpret_cast<unsigned*>(s + 3 * GS + LZ);  // [3] keys of the inputs, of the product, of pass 1
-    unsigned *kout = kin + 3, *kmid = kin + 4;
+    // FP64: per line the keys of the inputs, after the first forward pass, of the product, after the first inverse pass
+    unsigned* kin = reinterpret_cast<unsigned*>(s + 3 * GS + LZ);
+    unsigned *kfwd = kin + NL, *kout = kfwd + NL, *kmid = kout + NL;
     const int tid = threadIdx.x, lane = tid & 31;
     grid_release();
     for (int m = tid; m < LZ; m += NT) {
@@ -71,7 +72,8 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
         else
             twf[m] = tw32[m];
     }
-    if (tid < 5) kin[tid] = 0;
+    if (F64)
+        for (int i = tid; i < 4 * NL; i += NT) kin[i] = 0;
     grid_wait();
     __syncthreads();
     const int ntile = z.Lx / TB;
@@ -86,6 +88,12 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
     const C* green = reinterpret_cast<const C*>(z.green);
     const long long tstride = (long long)z.Ox * z.Oy * z.Oz;
     auto line = [](int n) { return (n / TB) * GS + n % TB; };
+    // the largest key of the lanes on one column, TB apart, to the column's line of component a
+    auto collect = [&](unsigned key, unsigned* dst, int a) {
+#pragma unroll
+        for (int d = TB; d < 32; d *= 2) key = max(key, __shfl_xor_sync(0xffffffffu, key, d));
+        if (lane < TB) atomicMax(dst + a * TB + lane, key);
+    };
 
 #pragma unroll 1
     for (int r = 0; r < z.R; ++r) {
@@ -103,12 +111,10 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
                 if (idx < 3 * nz * TB) s[a * GS + (e - a * nz) * TB + idx % TB] = v[q];
                 if constexpr (F64) {
                     const unsigned key = fx_key(v[q]);
-                    if (__all_sync(0xffffffffu, a == __shfl_sync(0xffffffffu, a, 0))) {
-                        const unsigned m = __reduce_max_sync(0xffffffffu, key);
-                        if (lane == 0) atomicMax(kin + a, m);
-                    } else {
-                        atomicMax(kin + a, key);
-                    }
+                    if (__all_sync(0xffffffffu, a == __shfl_sync(0xffffffffu, a, 0)))
+                        collect(key, kin, a);
+                    else
+                        atomicMax(kin + a * TB + lane % TB, key);
                 }
             }
         }
@@ -116,7 +122,7 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
         if constexpr (F64) {
             for (int w = tid; w < NL * B; w += NT) {
                 const int ln = w % NL, b = w / NL;
-                const FxScale sc(kin[ln / TB], fx_room(LZ / 2));
+                const FxScale sc(kin[ln], fx_room(A / 2));
                 fx2* p = f + line(ln);
                 fx2 v[A];
 #pragma unroll
@@ -125,20 +131,23 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
                     v[a] = l < nz ? sc(*reinterpret_cast<const double2*>(p + l * TB)) : fx2{0, 0};
                 }
                 fft2::dft_half_in<A>(v, -1);
+                unsigned key = 0;
 #pragma unroll
                 for (int k1 = 0; k1 < A; ++k1) {
                     if (k1 && b) v[k1] = cmul(v[k1], twi[b * k1]);
                     p[(b + B * k1) * TB] = v[k1];
+                    key |= fx_key(v[k1]);
                 }
+                atomicOr(kfwd + ln, key);
             }
             __syncthreads();
             for (int w = tid; w < NL * A; w += NT) {
                 const int ln = w % NL, k1 = w / NL;
-                const int ex = FxScale(kin[ln / TB], fx_room(LZ / 2)).ex;
+                const int k = excess(kfwd[ln], B), ex = FxScale(kin[ln], fx_room(A / 2)).ex + k;
                 fx2* p = f + line(ln) + B * k1 * TB;
                 fx2 v[B];
 #pragma unroll
-                for (int b = 0; b < B; ++b) v[b] = p[b * TB];
+                for (int b = 0; b < B; ++b) v[b] = fx_shift(p[b * TB], k);
                 fft2::DFT<B, fx2>::run(v, -1);
 #pragma unroll
                 for (int k2 = 0; k2 < B; ++k2) *reinterpret_cast<double2*>(p + k2 * TB) = fx_double(v[k2], ex);
@@ -148,7 +157,8 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
             fft2::forward<LZ, NT>(s, NL, line, TB, twf, nz);
         }
         // block product
-        unsigned key = 0;
+        static_assert(NT % TB == 0, "a thread stays on one column");
+        unsigned key[3] = {0, 0, 0};
         for (int i = tid; i < LZ * TB; i += NT) {
             const int c = i % TB, p = i / TB;
             const int kz = fft2::freq_at(LZ, p), kx = z.colkx ? z.colkx[sc0 + c] : sc0 + c;
@@ -161,22 +171,23 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 s[a * GS + i] = x[a];
-                if constexpr (F64) key = max(key, fx_key(x[a]));
+                if constexpr (F64) key[a] = max(key[a], fx_key(x[a]));
             }
         }
         if constexpr (F64) {
-            key = __reduce_max_sync(0xffffffffu, key);
-            if (lane == 0) atomicMax(kout, key);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) collect(key[a], kout, a);
         }
         __syncthreads();
         if constexpr (F64) {
-            const bool bad = max(max(kin[0], kin[1]), max(kin[2], *kout)) >= 0x7ff00000u;
-            const FxScale sc(*kout, fx_room(B));
-            key = 0;
+            // an Inf or NaN reaches every component
+            const bool bad = __any_sync(0xffffffffu, max(kin[lane % NL], kout[lane % NL]) >= 0x7ff00000u);
             for (int w = tid; w < NL * A; w += NT) {
                 const int ln = w % NL, k1 = w / NL;
+                const FxScale sc(kout[ln], fx_room(B));
                 fx2* p = f + line(ln) + B * k1 * TB;
                 fx2 v[B];
+                unsigned key = 0;
 #pragma unroll
                 for (int k2 = 0; k2 < B; ++k2) v[k2] = sc(*reinterpret_cast<const double2*>(p + k2 * TB));
                 fft2::DFT<B, fx2>::run(v, +1);
@@ -186,13 +197,12 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
                     p[b * TB] = v[b];
                     key |= fx_key(v[b]);
                 }
+                atomicOr(kmid + ln, key);
             }
-            key = __reduce_or_sync(0xffffffffu, key);
-            if (lane == 0) atomicOr(kmid, key);
             __syncthreads();
-            const int k = max(fx_bits(*kmid) - fx_room(A), 0), ex = sc.ex + k;
             for (int w = tid; w < NL * B; w += NT) {
                 const int ln = w % NL, b = w / NL;
+                const int k = excess(kmid[ln], A), ex = FxScale(kout[ln], fx_room(B)).ex + k;
                 const fx2* p = f + line(ln);
                 fx2 v[A];
 #pragma unroll
@@ -210,7 +220,7 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
                 }
             }
             __syncthreads();
-            if (tid < 5) kin[tid] = 0;
+            for (int i = tid; i < 4 * NL; i += NT) kin[i] = 0;
         } else {
             fft2::inverse<LZ, NT>(s, NL, line, TB, twf, nz);
             for (int idx = tid; idx < 3 * nz * TB; idx += NT) {
