@@ -129,19 +129,25 @@ struct FxScale {
     __device__ __forceinline__ fx2 operator()(double2 v) const { return fx2{(*this)(v.x), (*this)(v.y)}; }
 };
 
-// v 2^ex, rounded to nearest; out of range to infinity, below the normal range to zero
+// v 2^ex, rounded to nearest (to a subnormal number where it is one); out of range to infinity.  INRANGE: fx_in_range(ex),
+// where no v gives either
+__device__ __forceinline__ bool fx_in_range(int ex) { return ex >= -1022 && ex <= 960; }
+template <bool INRANGE = false>
 __device__ __forceinline__ double fx_double(long long v, int ex) {
     const long long sg = v >> 63;
     const unsigned long long a = (unsigned long long)((v ^ sg) - sg);
     const int lz = __clzll((long long)a);
-    const unsigned long long m = (((a << (lz & 63)) >> 10) + 1) >> 1;
     const int e = 1085 - lz + ex;  // biased exponent, the leading bit of m counts as one
-    unsigned long long bits = ((unsigned long long)(unsigned)e << 52) + m;
-    if (a == 0 || e < 0) bits = 0;
-    if (e >= 2046 && a != 0) bits = 0x7ff0000000000000ull;
+    const unsigned long long m = (((a << (lz & 63)) >> (INRANGE ? 10 : min(max(10 - e, 10), 63))) + 1) >> 1;
+    unsigned long long bits = ((unsigned long long)(unsigned)(INRANGE ? e : max(e, 0)) << 52) + m;
+    if (!INRANGE && e >= 2046) bits = 0x7ff0000000000000ull;
+    if (a == 0) bits = 0;
     return __longlong_as_double((long long)(bits | ((unsigned long long)sg & 0x8000000000000000ull)));
 }
-__device__ __forceinline__ double2 fx_double(fx2 v, int ex) { return make_double2(fx_double(v.x, ex), fx_double(v.y, ex)); }
+template <bool INRANGE = false>
+__device__ __forceinline__ double2 fx_double(fx2 v, int ex) {
+    return make_double2(fx_double<INRANGE>(v.x, ex), fx_double<INRANGE>(v.y, ex));
+}
 
 // v 2^-k, rounded to nearest
 __device__ __forceinline__ fx2 fx_shift(fx2 v, int k) {

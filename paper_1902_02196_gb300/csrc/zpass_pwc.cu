@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
             }
         }
         __syncthreads();
+        int top = 0;
         if constexpr (F64) {
             for (int w = tid; w < NL * B; w += NT) {
                 const int ln = w % NL, b = w / NL;
@@ -141,9 +142,13 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
                 atomicOr(kfwd + ln, key);
             }
             __syncthreads();
+            // the spectrum becomes FP64 numbers relative to its largest exponent: none of them, nor of the product, is subnormal
+            // or out of range for the size of the inputs
+            const int n = lane % NL;
+            top = __reduce_max_sync(0xffffffffu, FxScale(kin[n], fx_room(A / 2)).ex + excess(kfwd[n], B));
             for (int w = tid; w < NL * A; w += NT) {
                 const int ln = w % NL, k1 = w / NL;
-                const int k = excess(kfwd[ln], B), ex = FxScale(kin[ln], fx_room(A / 2)).ex + k;
+                const int k = excess(kfwd[ln], B), ex = FxScale(kin[ln], fx_room(A / 2)).ex + k - top;
                 fx2* p = f + line(ln) + B * k1 * TB;
                 fx2 v[B];
 #pragma unroll
@@ -202,7 +207,7 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
             __syncthreads();
             for (int w = tid; w < NL * B; w += NT) {
                 const int ln = w % NL, b = w / NL;
-                const int k = excess(kmid[ln], A), ex = FxScale(kout[ln], fx_room(B)).ex + k;
+                const int k = excess(kmid[ln], A), ex = FxScale(kout[ln], fx_room(B)).ex + k + top;
                 const fx2* p = f + line(ln);
                 fx2 v[A];
 #pragma unroll

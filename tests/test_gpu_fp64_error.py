@@ -230,3 +230,25 @@ def test_pwc(vie, shape, kind):
     h12.close()
     e = (torch.linalg.vector_norm(y - want) / torch.linalg.vector_norm(want)).item()
     assert e <= 4e-16, e
+
+
+# the square xy kernels, the line ones, and an FFT length along z of 512
+@pytest.mark.parametrize("shape", [(4, 4, 4), (9, 20, 5), (4, 3, 140)])
+@pytest.mark.parametrize("kind", ["N", "PWC"])
+def test_subnormal_results(vie, shape, kind):
+    """Inputs so small that the results are subnormal numbers give those of ordinary ones times the power of two, within
+    the spacing of the subnormal numbers, 2^-1074, for each of the values of a plane that are summed (a quarter of
+    its points, half a spacing each)."""
+    nx, ny, nz = shape
+    eps = np.full((nz, ny, nx), 3.0)
+    h = vie.vie_setup((nx, ny, nz, 0.5, 0.4, 0.45), 3e6, eps, 0 * eps, vie.VIE_SETUP_PWC if kind == "PWC" else 0)
+    x = torch.from_numpy(field("random", 3 if kind == "PWC" else 12, shape)).cuda()
+    want = matvec(vie, h, x)
+    top = want.abs().max().item()
+    scale = 2.0 ** -(1030 + int(np.ceil(np.log2(top))))  # the largest result 2^-1030
+    got = matvec(vie, h, x * scale)
+    h.close()
+    planes = 4 * nx * ny * 4  # points of a plane at most
+    err = torch.linalg.vector_norm((torch.view_as_real(got) - torch.view_as_real(want) * scale).reshape(-1) * 2.0 ** 1000,
+                                   ord=float("inf")).item() * 2.0 ** -1000
+    assert err <= planes / 8 * 2.0 ** -1074, err / 2.0 ** -1074
