@@ -61,7 +61,7 @@ struct ZDCfg {
     static constexpr int NT = LZ <= 8 ? 96 : (LZ <= 128 ? 192 : 384);
     static constexpr int MINB = LZ <= 128 ? 2 : 1;
     static constexpr int GS = 2 * LZ + 2;  // component stride: four components and two columns on distinct banks
-    static constexpr int KEYS = 64 * RB;  // words for the keys
+    static constexpr int KEYS = 68 * RB;  // words for the keys, a multiple of four
     static constexpr int NTW = (fft2::Split<LZ>::A - 1) * (fft2::Split<LZ>::B - 1) + 1;  // twiddles in use
     static constexpr size_t smem = sizeof(fx2) * (size_t)(RB * 12 * GS + NTW) + sizeof(int) * KEYS +
                                    (size_t)(NT / 32) * 60 * 32 + sizeof(short) * 2 * (LZ / 2 + 2);
@@ -203,10 +203,11 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
     int4* tw = reinterpret_cast<int4*>(s + RB * 12 * GS);
     // per right-hand side and component: keys of the inputs, after the first forward pass, of the product and after the
     // first inverse pass; the spectrum's exponent; per right-hand side the product's exponent in both
-    // columns, and Inf or NaN among the inputs
+    // columns, and the components that an Inf or NaN of the inputs reaches; those that one of the tensors reaches
     unsigned* kin = reinterpret_cast<unsigned*>(tw + Cfg::NTW);
     unsigned *kfwd = kin + 12 * RB, *kout = kfwd + 12 * RB, *kmid = kout + 12 * RB;
-    int *sex = reinterpret_cast<int*>(kmid + 12 * RB), *pex = sex + 12 * RB, *bad = pex + 2 * RB;
+    int *sex = reinterpret_cast<int*>(kmid + 12 * RB), *pex = sex + 12 * RB, *bad = pex + 2 * RB,
+        *gbad = bad + RB;  // [2 columns]
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     // the digits of the warp's next octant point, copied while the current one is multiplied
     uint4* gbuf = reinterpret_cast<uint4*>(kin + Cfg::KEYS) + wid * (NG * 2);
@@ -223,6 +224,7 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
         if (tid < 2 * RB) pex[tid] = kLow;
     };
     reset();
+    if (tid < 2) gbad[tid] = 0;
     __syncthreads();
     const int ntile = z.Lx / 2;
     const int py = blockIdx.x / ntile, ct = blockIdx.x % ntile, sc0 = 2 * ct;
@@ -253,13 +255,18 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
     const unsigned bsel = part ? 0x1032u : 0x3210u;
     const unsigned bneg = (part ? 0u : 0x80000000u) ^ (swapneg ? 0x80008000u : 0u);
 
-    // exponents of the points, and the raises of the two columns' linear functions (the last word of tensor 0)
+    // exponents of the points and the raises of the two columns' linear functions (the last word of tensor 0), and the
+    // outputs that a tensor with an Inf or NaN reaches (that of tensor 1)
     constexpr int NO = LZ / 2 + 1;
-    auto point_word = [&](int c, int ko) {
-        return reinterpret_cast<const int*>(z.green_d)[(((long long)(c ? gc1 : gc0) * z.Oz + ko) * NG + 1) * 8 - 1];
+    auto point_word = [&](int c, int ko, int t) {
+        return reinterpret_cast<const int*>(z.green_d)[(((long long)(c ? gc1 : gc0) * z.Oz + ko) * NG + t) * 8 + 7];
     };
-    for (int i = tid; i < 2 * NO; i += NT) bex[i] = (short)(point_word(i / NO, i % NO) >> 8);
-    const int up0 = point_word(0, 0) & 255, up1 = point_word(1, 0) & 255;
+    for (int i = tid; i < 2 * NO; i += NT) {
+        const int c = i / NO, ko = i % NO, w = point_word(c, ko, 1);
+        bex[i] = (short)(point_word(c, ko, 0) >> 8);
+        if (w) atomicOr(gbad + c, w);
+    }
+    const int up0 = point_word(0, 0, 0) & 255, up1 = point_word(1, 0, 0) & 255;
     // octant points q of this CTA: 0..LZ/2, for each column when the columns are self-mirrored
     constexpr int NW = NT / 32;
     const int nq = single ? 2 * NO : NO;
@@ -377,9 +384,9 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
 #pragma unroll
             for (int e = 0; e < 3; ++e) xe[e] = sex[nrx * 12 + t + 4 * e];
             if (tid < RB) {
-                int b = 0;
-                for (int c = 0; c < 12; ++c) b |= kin[tid * 12 + c] >= 0x7ff00000u;
-                bad[tid] = b;
+                bool b = false;
+                for (int c = 0; c < 12; ++c) b = b || kin[tid * 12 + c] >= 0x7ff00000u;
+                bad[tid] = b ? 0xFFF : 0;  // it reaches every output
             }
             const int xlift = kBits - pex[2 * nrx + ncol] - (t ? (ncol ? up1 : up0) : 0);
             unsigned key[3] = {0, 0, 0};  // of the lane's outputs, components ra, ra + 4, ra + 8
@@ -485,6 +492,7 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
             for (int k1 = 0; k1 < A; ++k1) v[k1] = fx_shift(p[2 * (b + B * k1)], k);
             fft2::dft_half_out<A>(v, +1);
             const int comp = (ln % 24) >> 1, c = ln & 1;
+            const bool nan = ((bad[rr] | gbad[c]) >> comp) & 1;
             // exponent of the result: that of the product and the bits dropped since
             const int ex = pex[2 * rr + c] - (comp % 4 ? (c ? up1 : up0) : 0) - kBits + kShift + excess(kout[ln >> 1], B) + k;
             double2* out = z.w + (long long)(r0 + rr) * 12 * nz * plane + (long long)py * z.Lx + sc0 + c;
@@ -493,7 +501,7 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
                 const int l = b + B * a;
                 if (l < nz) {
                     double2 o = fx_double(v[a], ex);
-                    if (bad[rr]) o.x = o.y = __longlong_as_double(0x7ff8000000000000ll);  // it reaches every output
+                    if (nan) o.x = o.y = __longlong_as_double(0x7ff8000000000000ll);
                     out[((long long)comp * nz + l) * plane] = o;
                 }
             }
@@ -507,7 +515,8 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
 
 // Digit tables from the octant spectra g [NG][Oz][Oy][Ox].  Every octant point has an exponent be and every column a raise
 // up: an entry B is stored as seven signed 9-bit digits of B 2^(be + c up), c the number of linear functions in its pair,
-// below 2^62; be << 8 | up is in the unused last word of tensor 0.  The raise brings the linear rows and columns
+// below 2^62; be << 8 | up is in the unused last word of tensor 0, and
+// in that of tensor 1 a mask of the outputs whose rows have an Inf or a NaN at that point (stored as zero).  The raise brings the linear rows and columns
 // up to the constant ones (their Gram entries are 1/12, and where the spectrum is large they couple through
 // differences); it is the largest that leaves the pairs of constant functions the largest values, give or
 // take a bit or two.
@@ -518,8 +527,10 @@ __global__ void __launch_bounds__(256) digits_kernel(const double2* __restrict__
                                                      uint4* __restrict__ d) {
     __shared__ int top[3][kMaxOz][kDigitCols];  // per class of pairs: |B| < 2^(top - 1022); then [0]: be
     __shared__ int ctop[3][kDigitCols];         // the same over a column
+    __shared__ unsigned reach[kMaxOz][kDigitCols];
     const int c = threadIdx.x % kDigitCols, kx = blockIdx.x * kDigitCols + c, ky = blockIdx.y;
     for (int i = threadIdx.x; i < 3 * kMaxOz * kDigitCols; i += 256) (&top[0][0][0])[i] = kLow;
+    for (int i = threadIdx.x; i < kMaxOz * kDigitCols; i += 256) (&reach[0][0])[i] = 0;
     if (threadIdx.x < 3 * kDigitCols) (&ctop[0][0])[threadIdx.x] = kLow;
     __syncthreads();
     const int n = NG * Oz;
@@ -527,11 +538,23 @@ __global__ void __launch_bounds__(256) digits_kernel(const double2* __restrict__
         const int ll = t % 10;
         return ll == 0 ? 0 : (ll < 4 ? 1 : 2);
     };
+    auto outputs_of = [&](int t) {
+        unsigned m = 0;
+        if (NG == 60)
+            for (int i = kBlock.start[t]; i < kBlock.start[t + 1]; ++i) m |= 1u << kBlock.e[i].a;
+        else
+            for (int i = kKBlock.start[t]; i < kKBlock.start[t + 1]; ++i) m |= 1u << kKBlock.e[i].a;
+        return m;
+    };
     if (kx < Ox)
         for (int i = threadIdx.x / kDigitCols; i < n; i += 256 / kDigitCols) {
             const int t = i / Oz, kz = i - t * Oz;
             double2 v = g[((long long)i * Oy + ky) * Ox + kx];
             int e = (int)(fx_key(v) >> 20);
+            if (e >= 2047) {
+                atomicOr(&reach[kz][c], outputs_of(t));
+                continue;
+            }
             if (e == 0) {  // subnormal numbers
                 v = make_double2(0x1p64 * v.x, 0x1p64 * v.y);
                 e = v.x == 0.0 && v.y == 0.0 ? kLow : (int)(fx_key(v) >> 20) - 64;
@@ -554,6 +577,7 @@ __global__ void __launch_bounds__(256) digits_kernel(const double2* __restrict__
         const int t = i / Oz, kz = i - t * Oz;
         const int be = top[0][kz][c], sc = be + linear(t) * up;
         double2 v = g[((long long)i * Oy + ky) * Ox + kx];
+        if (fx_key(v) >= 0x7ff00000u) v = make_double2(0.0, 0.0);
         if (sc > 1000 || sc < -1000) {
             v = make_double2(scalbn(v.x, sc), scalbn(v.y, sc));
         } else {
@@ -573,7 +597,7 @@ __global__ void __launch_bounds__(256) digits_kernel(const double2* __restrict__
         }
         uint4* out = d + 2 * ((col * Oz + kz) * NG + t);
         out[0] = make_uint4(u[0], u[1], u[2], u[3]);
-        out[1] = make_uint4(u[4], u[5], u[6], t == 0 ? (unsigned)(be << 8 | up) : 0u);
+        out[1] = make_uint4(u[4], u[5], u[6], t == 0 ? (unsigned)(be << 8 | up) : (t == 1 ? reach[kz][c] : 0u));
     }
 }
 

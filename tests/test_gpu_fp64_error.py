@@ -252,3 +252,33 @@ def test_subnormal_results(vie, shape, kind):
     err = torch.linalg.vector_norm((torch.view_as_real(got) - torch.view_as_real(want) * scale).reshape(-1) * 2.0 ** 1000,
                                    ord=float("inf")).item() * 2.0 ** -1000
     assert err <= planes / 8 * 2.0 ** -1074, err / 2.0 ** -1074
+
+
+# the square xy kernels and the line ones, FFT lengths along z of 16, 64 and 512
+@pytest.mark.parametrize("shape", [(5, 6, 7), (3, 7, 20), (4, 3, 130)])
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_not_finite_table(vie, shape, value):
+    """A NaN or an Inf in one tensor makes the outputs that it couples to any input not finite, for every input, zero
+    among them, and leaves the others as the table without it gives them (to 1e-14)."""
+    nx, ny, nz = shape
+    clean = far_table(shape)
+    for (p, q), (l, m) in [((0, 0), (0, 0)), ((0, 2), (0, 1)), ((1, 1), (2, 3))]:
+        bad = {k: t.copy() for k, t in clean.items()}
+        bad[(p, q), (l, m)][1, 2, 1] = value
+        reached = {4 * u + v for u in (p, q) for v in (l, m)}
+        x = torch.from_numpy(field("random", 12, shape)).cuda()
+        h = handle_of(vie, shape, clean)
+        want = matvec(vie, h, x)
+        h.close()
+        h = handle_of(vie, shape, bad)
+        for v in (x, 0 * x, 1e-300 * x):
+            y = matvec(vie, h, v)
+            for a in range(12):
+                if a in reached:
+                    assert not torch.isfinite(torch.view_as_real(y[a])).all(-1).any(), (a, v[0, 0, 0, 0])
+                else:
+                    assert torch.isfinite(torch.view_as_real(y[a])).all()
+            if v is x:
+                for a in set(range(12)) - reached:
+                    assert torch.linalg.vector_norm(y[a] - want[a]) <= 1e-14 * torch.linalg.vector_norm(want[a])
+        h.close()
