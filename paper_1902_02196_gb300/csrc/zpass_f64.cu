@@ -51,6 +51,7 @@ constexpr unsigned kMagicBits = 0x4B400000u;  // 1.5 2^23
 constexpr unsigned long long kBias =
     256ull * ((1ull << 54) + (1ull << 45) + (1ull << 36) + (1ull << 27) + (1ull << 18) + (1ull << 9) + 1);
 constexpr int kLow = -100000;  // below every exponent
+constexpr int kLowest = -2000;  // below the exponents of the spectra
 constexpr int kBits = 62;   // |X|, |B| < 2^62
 constexpr int kShift = 66;  // Y = X B 2^-66: |Y| < 24 2^(62 + 62 - 66) < 2^63
 
@@ -347,7 +348,14 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
 #pragma unroll
             for (int k2 = 0; k2 < B; ++k2) p[2 * k2] = v[k2];
         }
-        if (tid < 12 * RB) sex[tid] = FxScale(kin[tid], TF1).ex + excess(kfwd[tid], B);
+        if (wid == 0) {  // a component with an Inf or NaN: so far down that the product has a unit of it at most
+            const bool in = lane < 12 * RB, nan = in && kin[lane] >= 0x7ff00000u;
+            if (in) sex[lane] = nan ? kLowest : FxScale(kin[lane], TF1).ex + excess(kfwd[lane], B);
+            const unsigned m = __ballot_sync(0xffffffffu, nan) >> (12 * (lane % RB)) & 0xFFFu;
+            // it reaches every output, through K those of the other two directions
+            if (lane < RB)
+                bad[lane] = KOP ? (m & 0xFF0 ? 0xF : 0) | (m & 0xF0F ? 0xF0 : 0) | (m & 0xFF ? 0xF00 : 0) : (m ? 0xFFF : 0);
+        }
         __syncthreads();
         // The product's exponent: the largest, over the points, of the spectrum's exponent less that of B.  (In a pass of its
         // own: an exponent per point would be a reduction between the product's loads and its digits.)
@@ -383,11 +391,6 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
             int xe[3];
 #pragma unroll
             for (int e = 0; e < 3; ++e) xe[e] = sex[nrx * 12 + t + 4 * e];
-            if (tid < RB) {
-                bool b = false;
-                for (int c = 0; c < 12; ++c) b = b || kin[tid * 12 + c] >= 0x7ff00000u;
-                bad[tid] = b ? 0xFFF : 0;  // it reaches every output
-            }
             const int xlift = kBits - pex[2 * nrx + ncol] - (t ? (ncol ? up1 : up0) : 0);
             unsigned key[3] = {0, 0, 0};  // of the lane's outputs, components ra, ra + 4, ra + 8
             for (int q = wid; q < nq; q += NW) {

@@ -282,3 +282,35 @@ def test_not_finite_table(vie, shape, value):
                 for a in set(range(12)) - reached:
                     assert torch.linalg.vector_norm(y[a] - want[a]) <= 1e-14 * torch.linalg.vector_norm(want[a])
         h.close()
+
+
+# the square xy kernels and the line ones, FFT lengths along z of 16, 64 and 512
+@pytest.mark.parametrize("shape", [(5, 6, 7), (3, 7, 20), (4, 3, 130)])
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+def test_k_not_finite(vie, shape, value):
+    """K does not couple a direction's components to themselves: a NaN or an Inf leaves them as they were (to 1e-13, a
+    hundred times the error of the product) and no finite value in the other two directions'; the other right-hand
+    side stays as it is."""
+    nx, ny, nz = shape
+    eps = np.full((nz, ny, nx), 3.0)
+    h = vie.vie_setup((nx, ny, nz, 0.01, 0.012, 0.011), 298e6, eps, 0 * eps)
+    x = torch.from_numpy(np.stack([field("random", 12, shape, seed) for seed in (4, 5)])).cuda()
+
+    def apply(v):
+        y = torch.empty_like(v)
+        torch.cuda.synchronize()
+        vie.vie_matvec(h, v, y, vie.VIE_FP64, vie.VIE_OP_K)
+        torch.cuda.synchronize()
+        return y
+
+    want = apply(x)
+    for comp in (1, 4, 11):
+        v = x.clone()
+        v[0, comp, nz // 2, 1, 1] = value
+        y = apply(v)
+        own = list(range(4 * (comp // 4), 4 * (comp // 4) + 4))
+        other = [a for a in range(12) if a not in own]
+        assert torch.linalg.vector_norm(y[0, own] - want[0, own]) <= 1e-13 * torch.linalg.vector_norm(want[0, own])
+        assert not torch.isfinite(torch.view_as_real(y[0, other])).all(-1).any()
+        assert torch.equal(y[1], want[1])
+    h.close()
