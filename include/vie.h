@@ -93,7 +93,8 @@ typedef struct {
  * vie_setup -- build a handle for one grid, frequency and dielectric map.
  * Computes on the GPU, in FP64: the Galerkin entries of N for every offset
  * (Section III-C, Eq. 25, Eq. 34, Eq. 42-43), their circulant embedding and 3-D
- * FFT (Section IV-A), stored in FP64, FP32 and split digits; and the per-voxel
+ * FFT (Section IV-A), stored in FP32, in BF16 halves and as digits of FP64, 48 bytes per
+ * octant value (for FFT lengths that the fused z passes do not take in FP64 and FP32); and the per-voxel
  * material coefficients eps, chi = eps - 1, tau = chi/eps (Eq. 7, Eq. 17, Eq. 29).
  *   grid          : voxel counts and sizes (see above)
  *   freq_hz       : frequency f > 0; omega = 2 pi f, k0 = omega / c0
@@ -146,8 +147,8 @@ void vie_destroy(vie_handle* h);
  *   precision : VIE_FP64, VIE_FP32 or VIE_BF16X3 (VIE_OP_K: VIE_FP64 or VIE_FP32)
  *   op        : VIE_OP_A, VIE_OP_PA, VIE_OP_NSCAT or VIE_OP_K.  VIE_OP_K transforms the 30
  *               tensors of vie_green_toeplitz_k once per handle into octant spectra (30 Ox Oy Oz
- *               values in FP64, in FP32 in two layouts and as digits of 32 bytes: 64 bytes per value
- *               in all, kept until vie_destroy and counted by vie_info) and runs
+ *               values in FP32 and as FP64 digits, 40 bytes per value in all, or 24 for FFT lengths
+ *               outside 8..512 along z; kept until vie_destroy and counted by vie_info) and runs
  *               the same transforms as the N operator with the K block (96 signed entries) at
  *               every frequency point, the other octants from the K parities.
  */

@@ -225,12 +225,6 @@ int vie_setup_green_external(const vie_grid* grid, double freq_hz, const double*
 
 }  // extern "C"
 
-size_t handle_green_bytes(const vie_handle* h) {
-    const size_t ov = (size_t)h->O[0] * h->O[1] * h->O[2];
-    return 60 * ov * (sizeof(double2) + 2 * sizeof(float2) + sizeof(uint2)) + green_digit_bytes(h, 60) +
-           60 * h->nv * sizeof(double2) + 2048 * (sizeof(double2) + sizeof(float2) + sizeof(int4)) + 2 * (size_t)h->L[0];
-}
-
 int handle_create(const vie_grid* grid, double freq_hz, const double* eps_real, const double* sigma,
                   const vie_handle* share, vie_handle** out, const void* ext, int nc) {
     *out = nullptr;

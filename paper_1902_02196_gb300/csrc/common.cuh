@@ -112,7 +112,7 @@ struct vie_handle {
     double2 *eps64, *chi64, *tau64, *ieps64;
     float2 *chi32, *tau32, *ieps32;
     // FFT'd circulant Green tensors (of N - G), octant k_i in [0, L_i/2], pre-scaled by 1/(Lx Ly Lz):
-    // layout [60][Oz][Oy][Ox]
+    // layout [60][Oz][Oy][Ox], for the generic z pass and the PWC one (null where the fused z passes apply)
     double2* green64;
     float2* green32;
     // FP32 copy in the layout of the z pass of the FP32 three-kernel path: [Oy][Ox][Oz][60]
@@ -122,7 +122,7 @@ struct vie_handle {
     // (PWL handles with an FFT length along z of 8..512, else null)
     uint4* green_d;
     // the 30 K tensors' transformed circulants, octant storage [30][Oz][Oy][Ox], scaled by
-    // 1/(Lx Ly Lz), FP64 and FP32 (kmatvec.cu, built on the first K product)
+    // 1/(Lx Ly Lz), FP64 and FP32 (kmatvec.cu, built on the first K product; null where the fused z passes apply)
     double2* kgreen64;
     float2* kgreen32;
     // copy [Oy][Ox][Oz][30] for the FP32 fused z pass with the K block (zpass_f32.cu)
@@ -188,8 +188,6 @@ struct vie_handle {
 // nc: unknowns per voxel, 12 (PWL) or 3 (PWC, vie_setup flag VIE_SETUP_PWC).
 int handle_create(const vie_grid* grid, double freq_hz, const double* eps_real, const double* sigma,
                   const vie_handle* share, vie_handle** out, const void* ext = nullptr, int nc = 12);
-// device bytes held by a handle's Green tensors, twiddles and column map (shared part)
-size_t handle_green_bytes(const vie_handle* h);
 
 // ---------------------------------------------------------------------------
 // Error reporting

@@ -605,7 +605,8 @@ __global__ void embed_kernel(const double2* __restrict__ T, int nx, int ny, int 
     C[gid] = v;
 }
 
-// Octant k_i in [0, L_i/2] of the transformed circulants, scaled, into FP64 and FP32 tables [60][Oz][Oy][Ox].
+// Octant k_i in [0, L_i/2] of the transformed circulants, scaled, into FP64 and FP32 tables [60][Oz][Oy][Ox] (FP32: if
+// given) and [Oy][Ox][Oz][60].
 __global__ void octant_kernel(const double2* __restrict__ C, int Lx, int Ly, int Lz, int t0, int nt, double scale,
                               double2* __restrict__ g64, float2* __restrict__ g32, float2* __restrict__ g32t) {
     const int Ox = Lx / 2 + 1, Oy = Ly / 2 + 1, Oz = Lz / 2 + 1;
@@ -620,7 +621,7 @@ __global__ void octant_kernel(const double2* __restrict__ C, int Lx, int Ly, int
     v.y *= scale;
     const long long dst = (long long)(t0 + tl) * ovol + o;
     g64[dst] = v;
-    g32[dst] = make_float2((float)v.x, (float)v.y);
+    if (g32) g32[dst] = make_float2((float)v.x, (float)v.y);
     const long long tdst = (((long long)ky * Ox + kx) * Oz + kz) * 60 + t0 + tl;
     g32t[tdst] = make_float2((float)v.x, (float)v.y);
 }
@@ -700,30 +701,39 @@ int green_setup(vie_handle* h) {
 // Circulant embedding, 3-D FFT and octant storage of the 60 Toeplitz tensors T [60][nz][ny][nx]
 // (device, N - G at offsets d >= 0) in FP64 and FP32 (Section IV-A).  Takes ownership of T, also
 // on failure: the handle keeps it for vie_green_toeplitz when keep_table is set, else frees it.
-// The spectra are allocated on the first call and overwritten by later ones.
+// The spectra are allocated on the first call and overwritten by later ones.  Where the fused z passes apply, what is
+// kept is what they read: the FP32 values, their BF16 halves and the FP64 values' digits, 48 bytes per octant
+// value, with the FP64 spectra in scratch; else the FP64 and FP32 tables of the generic z pass (and the PWC one).
 int green_embed(vie_handle* h, double2* T, bool keep_table) {
     cudaStream_t s = h->stream;
     const long long nd = (long long)h->nx * h->ny * h->nz;
     double2* C = nullptr;
     const size_t digit_bytes = green_digit_bytes(h, 60);
+    const bool fused = digit_bytes != 0;
+    double2* g64 = nullptr;
     auto fail = [&](int code) {
         cudaFree(T);
         cudaFree(C);
+        if (fused) cudaFree(g64);
         return code;
     };
     int rc = VIE_OK;
     const int Lx = h->L[0], Ly = h->L[1], Lz = h->L[2];
     const long long vol = (long long)Lx * Ly * Lz;
     const long long ovol = (long long)h->O[0] * h->O[1] * h->O[2];
-    if (!h->green64) {
-        if (cudaMalloc(&h->green64, sizeof(double2) * 60 * ovol) != cudaSuccess ||
-            cudaMalloc(&h->green32, sizeof(float2) * 60 * ovol) != cudaSuccess ||
-            cudaMalloc(&h->green32t, sizeof(float2) * 60 * ovol) != cudaSuccess ||
+    if (!h->green32t) {
+        if (cudaMalloc(&h->green32t, sizeof(float2) * 60 * ovol) != cudaSuccess ||
             cudaMalloc(&h->greenbf, sizeof(uint2) * 60 * ovol) != cudaSuccess ||
-            (digit_bytes && cudaMalloc(&h->green_d, digit_bytes) != cudaSuccess))
+            (fused && cudaMalloc(&h->green_d, digit_bytes) != cudaSuccess) ||
+            (!fused && (cudaMalloc(&h->green64, sizeof(double2) * 60 * ovol) != cudaSuccess ||
+                        cudaMalloc(&h->green32, sizeof(float2) * 60 * ovol) != cudaSuccess)))
             return fail((set_error("green alloc"), VIE_ENOMEM));
-        h->bytes_held += (sizeof(double2) + 2 * sizeof(float2) + sizeof(uint2)) * 60 * ovol + digit_bytes;
+        h->bytes_held += (sizeof(float2) + sizeof(uint2)) * 60 * ovol +
+                         (fused ? digit_bytes : (sizeof(double2) + sizeof(float2)) * 60 * ovol);
     }
+    g64 = h->green64;
+    if (fused && cudaMalloc(&g64, sizeof(double2) * 60 * ovol) != cudaSuccess)
+        return fail((set_error("green scratch"), VIE_ENOMEM));
     int chunk = (int)std::max<long long>(1, std::min<long long>(60, (4LL << 30) / (vol * (long long)sizeof(double2))));
     if (cudaMalloc(&C, sizeof(double2) * vol * chunk) != cudaSuccess) return fail((set_error("embed alloc"), VIE_ENOMEM));
     for (int t0 = 0; t0 < 60; t0 += chunk) {
@@ -735,14 +745,15 @@ int green_embed(vie_handle* h, double2* T, bool keep_table) {
         if (rc < 0) return fail(rc);
         long long tho = ovol * nt;
         VIE_KLAUNCH("octant", s, octant_kernel<<<(unsigned)((tho + 255) / 256), 256, 0, s>>>(C, Lx, Ly, Lz, t0, nt, 1.0 / (double)vol,
-                                                                     h->green64, h->green32, h->green32t));
+                                                                     g64, h->green32, h->green32t));
         if (cudaGetLastError() != cudaSuccess) return fail((set_error("octant launch"), VIE_EDEVICE));
     }
     rc = green_split_bf16(h);
-    if (rc == VIE_OK && digit_bytes) rc = green_digits(h, h->green64, 60, h->green_d, s);
+    if (rc == VIE_OK && fused) rc = green_digits(h, g64, 60, h->green_d, s);
     if (rc < 0) return fail(rc);
     if (cudaStreamSynchronize(s) != cudaSuccess) return fail((set_error("green setup sync"), VIE_EDEVICE));
     cudaFree(C);
+    if (fused) cudaFree(g64);
     if (!keep_table) {
         cudaFree(T);
         return VIE_OK;

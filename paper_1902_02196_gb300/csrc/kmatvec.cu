@@ -6,9 +6,9 @@
 //
 // The 30 Toeplitz tensors P_t (green.cu, assemble_k_kernel) are embedded into full 2N
 // circulants, the entries at negative offsets taken from the reflection parities of the block
-// table (kblock.h), transformed, and their octant k_i in [0, L_i/2] kept, scaled by
-// 1/(Lx Ly Lz), as [30][Oz][Oy][Ox] in FP64 and FP32, and once more as [Oy][Ox][Oz][30] (the 30
-// values of a point side by side, for the fused z passes), in FP32 and as FP64 digits.  The other octants follow
+// table (kblock.h), transformed, and their octant k_i in [0, L_i/2] kept, scaled by 1/(Lx Ly Lz): for
+// the fused z passes as [Oy][Ox][Oz][30] (the 30 values of a point side by side), in FP32 and as
+// FP64 digits, else as [30][Oz][Oy][Ox] in FP64 and FP32.  The other octants follow
 // in the z pass from the same parities: K(R_i k) = -S_i K(k) S_i.  Built on the first K product
 // of a handle and released with it.
 #include <algorithm>
@@ -72,24 +72,26 @@ __global__ void k_octant_kernel(const double2* __restrict__ C, int Lx, int Ly, i
     v.y *= scale;
     const long long dst = (long long)(t0 + tl) * ovol + o;
     g64[dst] = v;
-    g32[dst] = make_float2((float)v.x, (float)v.y);
+    if (g32) g32[dst] = make_float2((float)v.x, (float)v.y);
     const long long dt = (((long long)ky * Ox + kx) * Oz + kz) * 30 + t0 + tl;
-    g32t[dt] = make_float2((float)v.x, (float)v.y);
+    if (g32t) g32t[dt] = make_float2((float)v.x, (float)v.y);
 }
 
 // device bytes of a handle's K spectra
 size_t k_bytes(const vie_handle* h) {
-    return (sizeof(double2) + 2 * sizeof(float2)) * 30 * (size_t)h->O[0] * h->O[1] * h->O[2] + green_digit_bytes(h, 30);
+    const size_t nv = 30 * (size_t)h->O[0] * h->O[1] * h->O[2], digits = green_digit_bytes(h, 30);
+    return digits ? sizeof(float2) * nv + digits : (sizeof(double2) + sizeof(float2)) * nv;
 }
 
 unsigned blocks(long long n) { return (unsigned)((n + 255) / 256); }
 
 }  // namespace
 
-// the K octant spectra of the handle (h->kgreen64, h->kgreen32), built on first use
+// The K octant spectra of the handle, built on first use: kgreen32t and kgreen_d for the fused z passes (the FP64 spectra
+// they are made from in scratch), where those do not apply kgreen64 and kgreen32 for the generic one.
 int k_octants(vie_handle* h, cudaStream_t s) {
     std::lock_guard<std::mutex> lk(g_kmu);
-    if (h->kgreen64) return VIE_OK;
+    if (h->kgreen64 || h->kgreen_d) return VIE_OK;
     const int Lx = h->L[0], Ly = h->L[1], Lz = h->L[2];
     const long long vol = (long long)Lx * Ly * Lz, nd = (long long)h->nv;
     const long long ovol = (long long)h->O[0] * h->O[1] * h->O[2];
@@ -112,8 +114,7 @@ int k_octants(vie_handle* h, cudaStream_t s) {
     if (cudaMalloc(&P, sizeof(double2) * 30 * nd) != cudaSuccess ||
         cudaMalloc(&C, sizeof(double2) * vol * chunk) != cudaSuccess ||
         cudaMalloc(&g64, sizeof(double2) * 30 * ovol) != cudaSuccess ||
-        cudaMalloc(&g32, sizeof(float2) * 30 * ovol) != cudaSuccess ||
-        cudaMalloc(&g32t, sizeof(float2) * 30 * ovol) != cudaSuccess ||
+        cudaMalloc(digit_bytes ? &g32t : &g32, sizeof(float2) * 30 * ovol) != cudaSuccess ||
         (digit_bytes && cudaMalloc(&gd, digit_bytes) != cudaSuccess))
         return fail(VIE_ENOMEM, "K spectrum allocation failed");
     int rc = green_k_toeplitz(h, P, s);
@@ -142,6 +143,10 @@ int k_octants(vie_handle* h, cudaStream_t s) {
     }
     cudaFree(P);
     cudaFree(C);
+    if (digit_bytes) {
+        cudaFree(g64);
+        g64 = nullptr;
+    }
     h->kgreen64 = g64;
     h->kgreen32 = g32;
     h->kgreen32t = g32t;
@@ -157,7 +162,7 @@ int kmatvec_device(vie_handle* h, int R, const double2* x, double2* y, cudaStrea
 
 // frees the handle's K spectra, if any (called when the handle is released)
 void kmatvec_release(vie_handle* h) {
-    if (!h->kgreen64) return;
+    if (!h->kgreen64 && !h->kgreen_d) return;
     cudaFree(h->kgreen64);
     cudaFree(h->kgreen32);
     cudaFree(h->kgreen32t);

@@ -735,7 +735,7 @@ static int matvec_impl(vie_handle* h, int R, const void* x, void* y, int op, cud
     // columns follow colkx32: the fused kernels (FP32, FP64) where they apply, else the line z pass
     auto zpass = [&](int ay, int by) -> int {
         if (op == VIE_OP_K) {  // the K block on the 30 K tensors: the fused z passes, else the generic one
-            if (bf16 || nc != 12 || !h->kgreen64) {
+            if (bf16 || nc != 12 || (!h->kgreen64 && !h->kgreen_d)) {
                 set_error("the K operator runs in FP64 or FP32 on the PWL system");
                 return VIE_EINVAL;
             }
