@@ -314,3 +314,46 @@ def test_k_not_finite(vie, shape, value):
         assert not torch.isfinite(torch.view_as_real(y[0, other])).all(-1).any()
         assert torch.equal(y[1], want[1])
     h.close()
+
+
+# FFT lengths along z of 128 and 512 (two right-hand sides to a group, and one), on the line and on the plane transforms
+@pytest.mark.parametrize("shape", [(5, 9, 40), (9, 12, 50), (4, 7, 140)])
+@pytest.mark.parametrize("op", ["NSCAT", "K"])
+def test_groups_of_right_hand_sides(vie, shape, op):
+    """Five right-hand sides of very different sizes: each has the bits that it has alone, and the K product's error
+    against direct sums is below 1e-12 (its linear entries are small differences of large integrals, good to 1e-14)."""
+    nx, ny, nz = shape
+    eps = np.full((nz, ny, nx), 3.0)
+    h = vie.vie_setup((nx, ny, nz, 0.004, 0.005, 0.0045), 298e6, eps, 0 * eps)
+    sizes = [1.0, 1e-200, 1e100, 1e-9, 0.0]
+    x = torch.from_numpy(np.stack([s * field("random", 12, shape, seed) for seed, s in enumerate(sizes)])).cuda()
+
+    def apply(v):
+        y = torch.empty_like(v)
+        torch.cuda.synchronize()
+        vie.vie_matvec(h, v, y, vie.VIE_FP64, getattr(vie, "VIE_OP_" + op))
+        torch.cuda.synchronize()
+        return y
+
+    y = apply(x)
+    for r in range(5):
+        assert torch.equal(apply(x[r:r + 1].contiguous())[0], y[r]), r
+    if op == "K":
+        tensors = torch.zeros((30, nz, ny, nx), dtype=torch.complex128, device="cuda")
+        torch.cuda.synchronize()
+        vie.vie_green_toeplitz_k(h, tensors)
+        torch.cuda.synchronize()
+
+        def tensor_of(a, b):
+            (p, l), (q, m) = divmod(a, 4), divmod(b, 4)
+            if p == q:
+                return None
+            j = 3 - p - q
+            lo, hi = min(l, m), max(l, m)
+            pair = {0: hi, 1: 3 + hi, 2: 5 + hi, 3: 9}[lo]
+            sign = (-1.0 if (j - p) % 3 == 1 else 1.0) * (-1.0 if l > m and (l > 0) != (m > 0) else 1.0)
+            return tensors[10 * j + pair], sign, [-parity(a, i) * parity(b, i) for i in range(3)]
+
+        for e in errors(y[0], x[0], tensor_of, 8):
+            assert e <= 1e-12, e
+    h.close()
