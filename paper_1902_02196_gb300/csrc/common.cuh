@@ -247,6 +247,7 @@ struct LaunchScope {
 // effect once all of them run.  Under event timing launches stay plain, so that a kernel's time is its own.
 // What earlier kernels write is not read through const __restrict__ pointers: the compiler takes such data as
 // fixed for the whole kernel and may move its loads above the wait.
+constexpr int kSMs = 152;  // of a GB300
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... A>
@@ -263,7 +264,7 @@ inline void launch_dependent(bool overlap, void (*kernel)(P...), dim3 grid, dim3
     cfg.attrs = &attr;
     // Up to eight CTAs per SM: the launch counts for short kernels, and a large grid that starts early takes places
     // from the one before it (8 right-hand sides on 32^3 voxels: a solve was 5% slower with all launches so).
-    cfg.numAttrs = overlap && (long long)grid.x * grid.y * grid.z <= 8 * 152 ? 1 : 0;
+    cfg.numAttrs = overlap && (long long)grid.x * grid.y * grid.z <= 8 * kSMs ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // its error is the next VIE_CHECK_LAUNCH's
 }
 // launch on `stream` with the accounting of VIE_KLAUNCH_B

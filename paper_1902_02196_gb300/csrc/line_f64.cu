@@ -104,17 +104,13 @@ __global__ void __launch_bounds__(Line64Cfg<L>::NT, Line64Cfg<L>::MINB)
     constexpr int N2 = L / N1;
     for (int t = tid; t < TB * N1; t += NT) {
         const int n = t % TB, j = t / TB;
-        const int k = max(fx_bits(kmid[n]) - fx_room(N2), 0);
-        const int r = k ? 1 << (k - 1) : 0;
+        const int k = excess(kmid[n], N2);
         const int ex = FxScale(kin[n], fx_room(NLOAD)).ex + k;
         const bool bad = kin[n] >= 0x7ff00000u;  // an Inf or NaN reaches the whole line
         auto elem2 = [&](int i) { return n * LS + (KIND == FORWARD ? B * j + i : j + B * i); };
         fx2 v[N2];
 #pragma unroll
-        for (int i = 0; i < N2; ++i) {
-            const fx2 u = s[elem2(i)];
-            v[i] = fx2{(u.x + r) >> k, (u.y + r) >> k};
-        }
+        for (int i = 0; i < N2; ++i) v[i] = fx_shift(s[elem2(i)], k);
         if constexpr (KIND == FORWARD)
             fft2::DFT<B, fx2>::run(v, -1);
         else

@@ -196,11 +196,11 @@ __global__ void __launch_bounds__(ZCfg<T, L, NC>::NT) zpass_kernel(ZArgs z, cons
 // ---------------------------------------------------------------------------
 constexpr int kXYThreads = 256;
 
-// i / n and i % n for i < 2^15, 1 <= n <= 512, by one multiplication (exact: i n < 2^32)
+// i / n and i % n for i < 2^15, 2 <= n <= 512, by one multiplication (exact: i n < 2^32)
 struct SmallDiv {
-    unsigned n, m;
-    __device__ __forceinline__ explicit SmallDiv(int d) : n((unsigned)d), m(0xffffffffu / (unsigned)d + 1u) {}
-    __device__ __forceinline__ int div(int i) const { return n > 1 ? (int)__umulhi((unsigned)i, m) : i; }
+    unsigned m;
+    __device__ __forceinline__ explicit SmallDiv(int d) : m(0xffffffffu / (unsigned)d + 1u) {}
+    __device__ __forceinline__ int div(int i) const { return (int)__umulhi((unsigned)i, m); }
 };
 
 template <int L>
@@ -419,7 +419,8 @@ __global__ void __launch_bounds__(kXYThreads, XYCfg<L>::MINB)
     const long long cbase = (po / nz) * epi.ns;  // component block on the support
     const C* xin = reinterpret_cast<const C*>(epi.x);
     // the epilogue's x values of this plane arrive in the free chunk buffer during the x transform
-    const bool pre = epi.op != VIE_OP_NSCAT && L * CW >= ny * nx;
+    static_assert(CW >= L / 4, "a plane of L/2 x L/2 values fits the chunk buffer");
+    const bool pre = epi.op != VIE_OP_NSCAT;
     if (pre) {
         for (int idx = tid; idx < ny * nx; idx += NT) {
             const int yy = dnx.div(idx), xx = idx - yy * nx;
@@ -487,10 +488,10 @@ __global__ void __launch_bounds__(kXYThreads, XYCfg<L>::MINB)
             o = cbase + q.z + (xx - q.x);
         }
         if (epi.op == VIE_OP_A) {
-            const C xv = pre ? ck[idx] : xin[o];
+            const C xv = ck[idx];
             v = csub(mk(gl * xv.x, gl * xv.y), cmul(c2[zoff + idx], v));
         } else if (epi.op == VIE_OP_PA) {
-            const C xv = pre ? ck[idx] : xin[o];
+            const C xv = ck[idx];
             const C t = cmul(c2[zoff + idx], v);
             v = csub(cmul(csub(c1[zoff + idx], sh), xv), mk(ig * t.x, ig * t.y));
         }

@@ -341,7 +341,8 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
     const long long cbase = (po / nz) * epi.ns;  // component block on the support
     const double2* xin = reinterpret_cast<const double2*>(epi.x);
     // the epilogue's x values of this plane arrive in the free chunk buffer during the x transform
-    const bool pre = epi.op != VIE_OP_NSCAT && L * CW >= ny * nx;
+    static_assert(CW >= L / 4, "a plane of L/2 x L/2 values fits the chunk buffer");
+    const bool pre = epi.op != VIE_OP_NSCAT;
     if (pre) {
         for (int idx = tid; idx < ny * nx; idx += NT) {
             const int yy = idx / nx, xx = idx % nx;
@@ -422,10 +423,10 @@ __global__ void __launch_bounds__(XYCfg64<L>::NT, XYCfg64<L>::MINB)
         if (CONV) conv[base + idx] = v;  // every voxel of the plane, full-grid layout
         if (!in) continue;
         if (epi.op == VIE_OP_A) {
-            const double2 xv = pre ? reinterpret_cast<const double2*>(ck)[idx] : xin[o];
+            const double2 xv = reinterpret_cast<const double2*>(ck)[idx];
             v = csub(mk(gl * xv.x, gl * xv.y), cmul(c2[zoff + idx], v));
         } else if (epi.op == VIE_OP_PA) {
-            const double2 xv = pre ? reinterpret_cast<const double2*>(ck)[idx] : xin[o];
+            const double2 xv = reinterpret_cast<const double2*>(ck)[idx];
             const double2 t = cmul(c2[zoff + idx], v);
             v = csub(cmul(csub(c1[zoff + idx], sh), xv), mk(ig * t.x, ig * t.y));
         }

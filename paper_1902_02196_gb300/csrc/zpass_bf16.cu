@@ -137,10 +137,10 @@ __global__ void __launch_bounds__(ZBCfg<LZ, TB_>::NT, ZBCfg<LZ, TB_>::MINB)
         cp_async_commit();
     };
     if (warp < nq) fetch(warp);
-    // row e = a nz + l of a right-hand side's spectrum: component a = e / nz (e < 2^13, nz <= 512)
+    // row e = a nz + l of a right-hand side's spectrum: component a = e / nz (e < 2^13, 3 <= nz <= 512)
     const unsigned nzq = 0xffffffffu / (unsigned)nz + 1u;
     auto place = [&](int e) {
-        const int a = nz > 1 ? (int)__umulhi((unsigned)e, nzq) : e;
+        const int a = (int)__umulhi((unsigned)e, nzq);
         return a * (GS - nz * TB) + e * TB;
     };
 

@@ -181,10 +181,10 @@ __global__ void __launch_bounds__(ZFCfg<LZ, TB_>::NT, ZFCfg<LZ, TB_>::MINB)
     const bool ry = ky > z.Ly / 2;
 
     // row e = a nz + l of a right-hand side's spectrum: component a = e / nz by a multiplication (e < 2^13,
-    // nz <= 512; nz = 1: a = e)
+    // 3 <= nz <= 512: LZ >= 8)
     const unsigned nzq = 0xffffffffu / (unsigned)nz + 1u;
     auto place = [&](int e) {  // its first element in the buffer
-        const int a = nz > 1 ? (int)__umulhi((unsigned)e, nzq) : e;
+        const int a = (int)__umulhi((unsigned)e, nzq);
         return a * (GS - nz * TB) + e * TB;
     };
     auto issue = [&](int r, float2* buf) {
@@ -342,9 +342,9 @@ static int launch_zf_LT(const vie_handle* h, const ZFArgs& z, cudaStream_t s, co
                                   (int)smem));
     const long long blocks = (long long)z.Ly * (z.Lx / TB);
     // Small spectra: the right-hand sides are dealt out to several CTAs per tile, until four CTAs wait for every place on
-    // the 152 SMs; a CTA then loads the Green values for fewer of them.  16 right-hand sides on 10^3 voxels
+    // the SMs; a CTA then loads the Green values for fewer of them.  16 right-hand sides on 10^3 voxels
     // (32^3 points): 142 to 61 us with the items' points split as well; 8 on 32^3 voxels: 211 to 172 us.
-    const long long places = 152LL * Cfg::MINB;
+    const long long places = (long long)kSMs * Cfg::MINB;
     const unsigned parts = (unsigned)std::min<long long>(z.R, std::max<long long>(1, (4 * places + blocks - 1) / blocks));
     // with a device count the kernel adds its bytes to z.bctr
     const double bytes = z.nact ? kDevCounted : 8.0 * (2.0 * z.R * 12 * z.nz * z.Ly * z.Lx + NG * z.Ox * z.Oy * z.Oz);

@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
     const unsigned fy = ky > z.Ly / 2 ? z.my : 0u;
     const bool ry = ky > z.Ly / 2;
     const int nz = z.nz;
-    const unsigned nzq = 0xffffffffu / (unsigned)nz + 1u;  // idx / nz = umulhi(idx, nzq) for idx < 2^14, nz <= 512 (nz > 1)
+    const unsigned nzq = 0xffffffffu / (unsigned)nz + 1u;  // idx / nz = umulhi(idx, nzq) for idx < 2^14, 3 <= nz <= 512
     const bool single = ct == ntile - 1;  // columns 0 and Lx/2: own octant columns
     const int kx0 = z.colkx[sc0], kx1 = z.colkx[sc0 + 1];
     const int kxo0 = kx0 <= z.Lx / 2 ? kx0 : z.Lx - kx0, kxo1 = kx1 <= z.Lx / 2 ? kx1 : z.Lx - kx1;
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const int idx = i0 + q * NT + lane, e = min(idx >> 1, 12 * nz - 1);
-                    const int a = nz > 1 ? (int)__umulhi((unsigned)e, nzq) : e;
+                    const int a = (int)__umulhi((unsigned)e, nzq);
                     if (idx < 24 * nz) *reinterpret_cast<double2*>(s + (rr * 12 + a) * GS + 2 * (e - a * nz) + (idx & 1)) = v[q];
                     const unsigned key = fx_key(v[q]);
                     if (__all_sync(0xffffffffu, a == __shfl_sync(0xffffffffu, a, 0))) {

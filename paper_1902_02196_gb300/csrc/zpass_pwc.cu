@@ -79,12 +79,12 @@ __global__ void __launch_bounds__(ZPCfg<T, LZ>::NT, ZPCfg<T, LZ>::MINB)
     const int ntile = z.Lx / TB;
     const int py = blockIdx.x / ntile, sc0 = (blockIdx.x % ntile) * TB;
     const long long plane = (long long)z.Ly * z.Lx;
-    const int ky = z.by ? py / z.by + z.ay * (py % z.by) : py;
+    const int ky = py / z.by + z.ay * (py % z.by);
     const int kyo = ky <= z.Ly / 2 ? ky : z.Ly - ky;
     const unsigned fy = ky > z.Ly / 2 ? 2u : 0u;  // reflection parity of component p under axis i: -1 iff p = i
     const int nz = z.nz;
-    const unsigned nzq = 0xffffffffu / (unsigned)nz + 1u;  // e / nz = umulhi(e, nzq) for e < 2^11 (nz > 1)
-    auto comp_of = [&](int e) { return nz > 1 ? (int)__umulhi((unsigned)e, nzq) : e; };
+    const unsigned nzq = 0xffffffffu / (unsigned)nz + 1u;  // e / nz = umulhi(e, nzq) for e < 2^11, 3 <= nz <= 512
+    auto comp_of = [&](int e) { return (int)__umulhi((unsigned)e, nzq); };
     const C* green = reinterpret_cast<const C*>(z.green);
     const long long tstride = (long long)z.Ox * z.Oy * z.Oz;
     auto line = [](int n) { return (n / TB) * GS + n % TB; };
