@@ -24,8 +24,8 @@
 //  - the accumulators start at 1.5 2^23, so that their bit patterns are the integers and no
 //    conversion instruction (16 per clock) is needed.
 //
-// Measured, 16 right-hand sides on 64^3 voxels (Lx = Ly = Lz = 128): 15.8 ms, the FP64 kernel of the same
-// structure 70.8 ms; the K block of 8 right-hand sides 6.9 ms against 29.1 ms.
+// Measured, 16 right-hand sides on 64^3 voxels (Lx = Ly = Lz = 128): 15.6 ms, the FP64 kernel of the same
+// structure 70.8 ms; the K block of 8 right-hand sides 6.8 ms against 29.1 ms.
 //
 // What bounds it: 12 warps to an SM (168 registers, 115 KB of shared memory to a CTA), which issue in 49% of the cycles 268
 // instructions per point and right-hand side, half of them the product's (digits, sums, recombination).  A warp's
@@ -405,17 +405,8 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
                 unsigned a[3][3][kD];
                 cp_async_wait<0>();
                 __syncwarp();
-                // X: components t + 4 e of point n.  K leaves registers to load it ahead of B's digits (6.84 to 6.72 ms for 8
-                // right-hand sides on 64^3 voxels), N does not (15.8 to 16.0 ms for 16)
-                fx2 x[3];
-                auto load_x = [&] {
-                    const bool v = nval && !(nneg && self) && !(single && ncol != col);
-                    const fx2* p = s + (nrx * 12 + t) * GS + 2 * pos_of(LZ, nneg && ko ? LZ - ko : ko) + ncol;
-#pragma unroll
-                    for (int e = 0; e < 3; ++e) x[e] = v ? p[4 * e * GS] : fx2{0, 0};
-                };
-                if (KOP) load_x();
-                const int lift = xlift - bex[q];  // of X (its columns share an octant point unless they are self-mirrored)
+                // of X, less B's exponent (its columns share an octant point unless they are self-mirrored)
+                const int lift = xlift - ((int)gbuf[1].w >> 8);
 #pragma unroll
                 for (int p = 0; p < 3; ++p)
 #pragma unroll
@@ -431,16 +422,19 @@ __global__ void __launch_bounds__(ZDCfg<LZ>::NT, ZDCfg<LZ>::MINB)
                     }
                 __syncwarp();
                 fetch(q + NW < nq ? q + NW : wid);  // after the last one, the next group's first
-                if (!KOP) load_x();
-                // digits of X = spectrum 2^lift: with that, every point's product has the exponent
+                // digits of X: components t + 4 e of point n, X = spectrum 2^lift: with that, every point's product has the exponent
                 // pex, and X stays below 2^62; the linear components are lower by the raise of B's linear rows and columns
                 unsigned b[3][kD];
                 {
+                    const bool v = nval && !(nneg && self) && !(single && ncol != col);
+                    const int kz = nneg && ko ? LZ - ko : ko;
                     const unsigned m = fy ^ (ncol ? fx1 : fx0) ^ (nneg ? z.mz : 0u);
+                    const fx2* p = s + (nrx * 12 + t) * GS + 2 * pos_of(LZ, kz) + ncol;
 #pragma unroll
                     for (int e = 0; e < 3; ++e) {
+                        const fx2 x = v ? p[4 * e * GS] : fx2{0, 0};
                         const __half2 sg = __float2half2_rn(((m >> (t + 4 * e)) & 1u) ? -1.f : 1.f);
-                        split_digits(x[e], max(lift + xe[e], -62), sg, b[e]);
+                        split_digits(x, max(lift + xe[e], -62), sg, b[e]);
                     }
                 }
                 long long y[6];
